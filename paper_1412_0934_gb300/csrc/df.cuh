@@ -100,6 +100,114 @@ __device__ __forceinline__ df rsqrt_(const df& x) {  // the square root (named l
   return fast_two_sum(s0, 0.5f * r * i0);
 }
 
+// ------------------------------------------------------------------ unnormalised forms
+// Inside a formula a value may stay an unnormalised pair, |l| up to a few ulp(h) (or, after
+// cancellation, up to a few 2^-24 of the operands): the Fast2Sum that closes each operator above
+// then happens once per result instead of once per operation.  prod_ drops only l*l and rounds its
+// low word three times, sum_ rounds its low word twice: the same absolute bounds (a few u^2 of the
+// operands) as the normalising operators.
+__device__ __forceinline__ df prod_(const df& x, const df& y) {  // 4 operations (mul: 8)
+  const float p = x.h * y.h;
+  return df(p, fmaf(x.h, y.l, fmaf(x.l, y.h, fmaf(x.h, y.h, -p))));
+}
+__device__ __forceinline__ df sum_(const df& x, const df& y) {  // 8 operations (add: 11)
+  const df s = two_sum(x.h, y.h);
+  return df(s.h, s.l + (x.l + y.l));
+}
+__device__ __forceinline__ df norm_(const df& x) { return fast_two_sum(x.h, x.l); }
+
+// Reciprocal, quotient and square root of (possibly unnormalised) pairs, unnormalised results.  The
+// reciprocal r0 (1 + e + e^2), e = 1 - y r0, keeps e^2: the approximation's e is up to 2^-23, so e^2 is
+// the largest error of a step whose reciprocals stop at r0 (1 + e).  The
+// quotient's remainder num.h - den.h q is exact in its leading difference (q is the float quotient to
+// a few ulp); the root is one Newton correction, s = s0 + (x - s0^2) / (2 s0).
+__device__ __forceinline__ df rcpu_(const df& y) {
+  float r0;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(y.h));
+  const float p = y.h * r0;
+  const float e = fmaf(-y.l, r0, (1.f - p) - fmaf(y.h, r0, -p));  // 1 - y r0
+  return df(r0, r0 * fmaf(e, e, e));
+}
+__device__ __forceinline__ df quot_(const df& x, const df& y) {
+  float r0;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(y.h));
+  const float q = x.h * r0, p = y.h * q;
+  const float r = ((x.h - p) - fmaf(y.h, q, -p)) + fmaf(-y.l, q, x.l);
+  return df(q, r * r0);
+}
+__device__ __forceinline__ df rootu_(const df& x) {
+  float s0, i0;  // independent approximations: the root's own error is squared, 1/root's only scales it
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(s0) : "f"(x.h));
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(i0) : "f"(x.h));
+  i0 = x.h > 1.2e-38f ? i0 : 0.f;  // zero (and what .ftz reads as zero) has root zero
+  const float p = s0 * s0;
+  const float r = ((x.h - p) - fmaf(s0, s0, -p)) + x.l;
+  return df(s0, 0.5f * r * i0);
+}
+
+// ------------------------------------------------------------------ two values side by side
+// sm_103a's packed FP32 instructions do two lanes' add, multiply or FMA in one issue slot (at the
+// scalar rate of the pipe: 119 results per clock per SM either way).  A df2 holds two double-float
+// values as pairs of high and of low words; its operations are the ones above, lane by lane, bit for
+// bit.  Operand negation is folded into the instruction.  The double-float step was bound by issue slots
+// (64% of them, ~5730 thread instructions per cell): with the packed and the unnormalised forms a cell
+// takes ~4200, and a 512^3 step of 16x16 tiles went from 32.2 to 25.3 ms, its error against 64-bit
+// arithmetic from 1.5e-15 to 1.2e-15 (2-norm, density).
+struct df2 {
+  float2 h, l;
+};
+__device__ __forceinline__ df2 pair_(const df& a, const df& b) { return df2{make_float2(a.h, b.h), make_float2(a.l, b.l)}; }
+__device__ __forceinline__ df2 both_(const df& a) { return pair_(a, a); }
+__device__ __forceinline__ df first_(const df2& x) { return df(x.h.x, x.l.x); }
+__device__ __forceinline__ df second_(const df2& x) { return df(x.h.y, x.l.y); }
+__device__ __forceinline__ float2 neg_(const float2& a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 add2_(const float2& a, const float2& b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2_(const float2& a, const float2& b) { return __fadd2_rn(a, neg_(b)); }
+__device__ __forceinline__ float2 mul2_(const float2& a, const float2& b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2_(const float2& a, const float2& b, const float2& c) { return __ffma2_rn(a, b, c); }
+
+__device__ __forceinline__ df2 neg_(const df2& x) { return df2{neg_(x.h), neg_(x.l)}; }
+__device__ __forceinline__ df2 half_(const df2& x) {
+  const float2 c = make_float2(0.5f, 0.5f);
+  return df2{mul2_(x.h, c), mul2_(x.l, c)};
+}
+__device__ __forceinline__ df2 norm_(const df2& x) {
+  const float2 s = add2_(x.h, x.l);
+  return df2{s, sub2_(x.l, sub2_(s, x.h))};
+}
+__device__ __forceinline__ df2 sum_(const df2& x, const df2& y) {
+  const float2 s = add2_(x.h, y.h);
+  const float2 b = sub2_(s, x.h);
+  const float2 e = add2_(sub2_(x.h, sub2_(s, b)), sub2_(y.h, b));
+  return df2{s, add2_(e, add2_(x.l, y.l))};
+}
+__device__ __forceinline__ df2 operator+(const df2& x, const df2& y) { return norm_(sum_(x, y)); }
+__device__ __forceinline__ df2 operator-(const df2& x, const df2& y) { return norm_(sum_(x, neg_(y))); }
+__device__ __forceinline__ df2 prod_(const df2& x, const df2& y) {
+  const float2 p = mul2_(x.h, y.h);
+  return df2{p, fma2_(x.h, y.l, fma2_(x.l, y.h, fma2_(x.h, y.h, neg_(p))))};
+}
+__device__ __forceinline__ df2 rcpu_(const df2& y) {
+  float2 r0;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0.x) : "f"(y.h.x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0.y) : "f"(y.h.y));
+  const float2 p = mul2_(y.h, r0);
+  const float2 e = fma2_(neg_(y.l), r0, sub2_(sub2_(make_float2(1.f, 1.f), p), fma2_(y.h, r0, neg_(p))));
+  return df2{r0, mul2_(r0, fma2_(e, e, e))};
+}
+__device__ __forceinline__ df2 rootu_(const df2& x) {
+  float2 s0, i0;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(s0.x) : "f"(x.h.x));
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(s0.y) : "f"(x.h.y));
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(i0.x) : "f"(x.h.x));
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(i0.y) : "f"(x.h.y));
+  i0.x = x.h.x > 1.2e-38f ? i0.x : 0.f;
+  i0.y = x.h.y > 1.2e-38f ? i0.y : 0.f;
+  const float2 p = mul2_(s0, s0);
+  const float2 r = add2_(sub2_(sub2_(x.h, p), fma2_(s0, s0, neg_(p))), x.l);
+  return df2{s0, mul2_(mul2_(r, make_float2(0.5f, 0.5f)), i0)};
+}
+
 // Comparisons of normalised values.
 __device__ __forceinline__ bool operator<(const df& a, const df& b) { return a.h < b.h || (a.h == b.h && a.l < b.l); }
 __device__ __forceinline__ bool operator>(const df& a, const df& b) { return b < a; }

@@ -164,9 +164,11 @@ __device__ __forceinline__ R minmod(R a, R b) {
   return abs_le(a, b) ? a : b;
 }
 __device__ __forceinline__ df minmod(const df& a, const df& b) {
-  if (prod_nonpos(a, b)) return df(0.f, 0.f);
+  // selected, not branched: a.h b.h > 0 can only fail by underflow, below 1e-45
   const bool le = a.h > 0.f ? !(b < a) : !(a < b);
-  return le ? a : b;
+  const bool zero = prod_nonpos(a, b);
+  const float h = le ? a.h : b.h, l = le ? a.l : b.l;
+  return df(zero ? 0.f : h, zero ? 0.f : l);
 }
 
 // ------------------------------------------------------------------ Hancock predictor
@@ -199,6 +201,27 @@ __device__ __forceinline__ void hancock(const R q[5], const R dqx[5], const R dq
   qh[2] = q[2] - hdt * ((tx2 + ty2) + tz2);
   qh[3] = q[3] - hdt * ((tx3 + ty3) + tz3);
   qh[4] = q[4] - hdt * ((tx4 + ty4) + tz4);
+}
+
+// The same in double-float: each row is one sum of four products, closed by one normalisation, with
+// the velocity divergence formed once; rows (0, 1) and (2, 3) side by side in packed FP32.
+__device__ __forceinline__ void hancock(const df q[5], const df dqx[5], const df dqy[5], const df dqz[5],
+                                        const df& gamma, const df& hdt, df qh[5]) {
+  const df ir = rcpu_(q[0]);
+  const df gp = prod_(gamma, q[4]);
+  const df div = sum_(sum_(dqx[1], dqy[2]), dqz[3]);
+  const df2 u = both_(q[1]), v = both_(q[2]), w = both_(q[3]), nh = neg_(both_(hdt));
+  const df2 a = sum_(sum_(prod_(u, pair_(dqx[0], dqx[1])), prod_(v, pair_(dqy[0], dqy[1]))),
+                     sum_(prod_(w, pair_(dqz[0], dqz[1])), prod_(pair_(q[0], ir), pair_(div, dqx[4]))));
+  const df2 b = sum_(sum_(prod_(u, pair_(dqx[2], dqx[3])), prod_(v, pair_(dqy[2], dqy[3]))),
+                     sum_(prod_(w, pair_(dqz[2], dqz[3])), prod_(both_(ir), pair_(dqy[4], dqz[4]))));
+  const df c = sum_(sum_(prod_(q[1], dqx[4]), prod_(q[2], dqy[4])), sum_(prod_(q[3], dqz[4]), prod_(gp, div)));
+  const df2 qa = pair_(q[0], q[1]) + prod_(nh, a), qb = pair_(q[2], q[3]) + prod_(nh, b);
+  qh[0] = first_(qa);
+  qh[1] = second_(qa);
+  qh[2] = first_(qb);
+  qh[3] = second_(qb);
+  qh[4] = q[4] + prod_(-hdt, c);
 }
 
 template <class R>
@@ -281,6 +304,60 @@ __device__ __forceinline__ void hllc_core(const R qL[5], const R qR[5], bool zn,
   F[2] = mn * t1;
   F[3] = mn * t2;
   F[4] = ue * (Ee + pe);
+}
+
+// The same flux in double-float: the two sides side by side in packed FP32 up to S*, sums and products
+// left unnormalised inside the formulas, S* from its distance to u_L (S* - u_L = (p_R - p_L + m_R (u_L -
+// u_R)) / (m_L - m_R), which does not cancel in fast flow), and the star energy without 1/m_K: with i =
+// 1/(S_K - S*) and g = (S_K - u_K) i, E* = g E_K + (S* - u_K)(r* S* + p_K i).
+// The fluxes are returned unnormalised (they are only summed).  The kinetic sum's order is (u_n^2 +
+// u_t1^2) + u_t2^2 for every normal.
+__device__ __forceinline__ void hllc_core(const df qL[5], const df qR[5], bool, const df& gamma, const df& inv_gm1,
+                                          df F[5]) {
+  const df2 r2 = pair_(qL[0], qR[0]), u2 = pair_(qL[1], qR[1]), p2 = pair_(qL[4], qR[4]);
+  const df2 c2 = rootu_(prod_(prod_(both_(gamma), p2), rcpu_(r2)));
+  const df2 lo = u2 - c2, hi = u2 + c2;
+  const df aL = first_(lo), bL = second_(lo), aR = first_(hi), bR = second_(hi);
+  const df SL = aL <= bL ? aL : bL;
+  const df SR = aR >= bR ? aR : bR;
+  const df2 d2 = sum_(pair_(SL, SR), neg_(u2));  // S - u of either side
+  const df2 m2 = prod_(r2, d2);
+  const df du = sum_(qL[1], -qR[1]);
+  const df num = sum_(sum_(qR[4], -qL[4]), prod_(second_(m2), du));
+  const df dl = quot_(num, sum_(first_(m2), -second_(m2)));  // S* - u_L
+  const df Ss = qL[1] + dl;
+  const bool SLneg = cmp_neg(SL), SRpos = cmp_pos(SR);
+  const bool star = SLneg && SRpos;
+  const bool left = !SLneg || (SRpos && !cmp_neg(Ss));
+  const df rK = left ? qL[0] : qR[0];
+  const df uK = left ? qL[1] : qR[1];
+  const df t1 = left ? qL[2] : qR[2];
+  const df t2 = left ? qL[3] : qR[3];
+  const df pK = left ? qL[4] : qR[4];
+  const df mK = left ? first_(m2) : second_(m2);
+  const df dK = left ? first_(d2) : second_(d2);
+  const df2 tt = pair_(t1, t2);
+  const df2 sq = prod_(tt, tt);
+  const df ke = sum_(sum_(prod_(uK, uK), first_(sq)), second_(sq));
+  const df EK = norm_(sum_(prod_(pK, inv_gm1), prod_(half_(rK), ke)));
+  const df dr = sum_(dl, du);
+  const df d = norm_(left ? dl : dr);  // S* - u_K
+  const df iD = rcpu_(sum_(dK, -d));
+  const df2 rg = prod_(both_(iD), pair_(mK, dK));
+  const df rs = first_(rg), g = second_(rg);
+  const df ps = sum_(pK, prod_(mK, d));
+  const df Es = sum_(prod_(g, EK), prod_(d, sum_(prod_(rs, Ss), prod_(pK, iD))));
+  const df re = star ? rs : rK;
+  const df ue = star ? Ss : uK;
+  const df pe = star ? ps : pK;
+  const df Ee = star ? Es : EK;
+  const df mn = norm_(prod_(re, ue));
+  F[0] = mn;
+  F[1] = sum_(prod_(mn, ue), pe);
+  const df2 ft = prod_(both_(mn), tt);
+  F[2] = first_(ft);
+  F[3] = second_(ft);
+  F[4] = prod_(ue, sum_(Ee, pe));
 }
 
 template <class R>
@@ -515,8 +592,8 @@ struct PolDF {
   using S = double;
   using R = df;
   // The same recovery as PolF64, in double-float from the double state (split into float pairs on
-  // the integer pipe, split_double).
-  static __device__ __forceinline__ void recover(const double U[5], const Params& P, df q[5], unsigned& flags) {
+  // the integer pipe, split_double); ir receives 1/rho (unnormalised).
+  static __device__ __forceinline__ void recover(const double U[5], const Params& P, df q[5], df& ir, unsigned& flags) {
     df rho, mx, my, mz, E;
     split_double(U[0], rho.h, rho.l);
     split_double(U[1], mx.h, mx.l);
@@ -525,23 +602,29 @@ struct PolDF {
     split_double(U[4], E.h, E.l);
     const df rf = kc<df>(P, K_RHOF);
     if (rho < rf) { flags |= HYDRO_EBIT_RHO_FLOOR; rho = rf; }
-    const df ir = rcp_(rho);
-    const df kin = half_(((mx * mx + my * my) + mz * mz) * ir);
+    ir = rcpu_(rho);
+    const df2 mxy = pair_(mx, my), sq = prod_(mxy, mxy);
+    const df kin = norm_(prod_(sum_(sum_(first_(sq), second_(sq)), prod_(mz, mz)), half_(ir)));
     const df eint = sub_acc(E, kin);
     if (cmp_neg(eint)) flags |= HYDRO_EBIT_P_FLOOR;
-    df p = kc<df>(P, K_GM1) * eint;
+    df p = norm_(prod_(kc<df>(P, K_GM1), eint));
     if (!(isfinite(p.h) && isfinite(rho.h))) flags |= HYDRO_EBIT_NONFINITE;
     const df pf = kc<df>(P, K_PF);
+    const df2 uv = norm_(prod_(mxy, both_(ir)));
     q[0] = rho;
-    q[1] = mx * ir;
-    q[2] = my * ir;
-    q[3] = mz * ir;
+    q[1] = first_(uv);
+    q[2] = second_(uv);
+    q[3] = norm_(prod_(mz, ir));
     q[4] = p < pf ? pf : p;
+  }
+  static __device__ __forceinline__ void recover(const double U[5], const Params& P, df q[5], unsigned& flags) {
+    df ir;
+    recover(U, P, q, ir, flags);
   }
   // U_old - dtdx * div: the double-float increment made a double exactly (float_to_double) and
   // subtracted from the double state in double.
   static __device__ __forceinline__ double update(double Uold, const df& dtdx, const df& div) {
-    const df d = dtdx * div;
+    const df d = prod_(dtdx, div);
     return Uold - (float_to_double(d.h) + float_to_double(d.l));
   }
   static __device__ __forceinline__ df speed(const double U[5], const Params& P, unsigned& flags);
@@ -596,9 +679,10 @@ __device__ __forceinline__ float PolMixed::speed(const double U[5], const Params
   return ((fabsf(u) + fabsf(v)) + fabsf(w)) + 3.0f * c;
 }
 __device__ __forceinline__ df PolDF::speed(const double U[5], const Params& P, unsigned& flags) {
-  df q[5];
-  recover(U, P, q, flags);
-  return cfl_speed(q, kc<df>(P, K_GAMMA));
+  df q[5], ir;
+  recover(U, P, q, ir, flags);
+  const df c = rootu_(prod_(prod_(kc<df>(P, K_GAMMA), q[4]), ir));
+  return sum_(sum_(rabs(q[1]), rabs(q[2])), rabs(q[3])) + mulf_(c, 3.f);  // normalised: the maximum compares it
 }
 
 // ------------------------------------------------------------------ CFL candidates

@@ -74,31 +74,96 @@ struct Plane5<double, H, W> {
   }
 };
 
+// Double-float: values 0, 1 and 2, 3 side by side, high words then low words, the operands of the packed
+// FP32 instructions as they are loaded.
 template <int H, int W>
 struct Plane5<df, H, W> {
-  float4 a[H][W];  // (h0, l0, h1, l1)
-  float4 b[H][W];  // (h2, l2, h3, l3)
+  float4 a[H][W];  // (h0, h1, l0, l1)
+  float4 b[H][W];  // (h2, h3, l2, l3)
   float2 c[H][W];  // (h4, l4)
   __device__ __forceinline__ void st(int j, int i, const df v[5]) {
-    a[j][i] = make_float4(v[0].h, v[0].l, v[1].h, v[1].l);
-    b[j][i] = make_float4(v[2].h, v[2].l, v[3].h, v[3].l);
+    a[j][i] = make_float4(v[0].h, v[1].h, v[0].l, v[1].l);
+    b[j][i] = make_float4(v[2].h, v[3].h, v[2].l, v[3].l);
     c[j][i] = make_float2(v[4].h, v[4].l);
   }
   __device__ __forceinline__ void ld(int j, int i, df v[5]) const {
     const float4 t = a[j][i], u = b[j][i];
     const float2 w = c[j][i];
-    v[0] = df(t.x, t.y); v[1] = df(t.z, t.w); v[2] = df(u.x, u.y); v[3] = df(u.z, u.w);
+    v[0] = df(t.x, t.z); v[1] = df(t.y, t.w); v[2] = df(u.x, u.z); v[3] = df(u.y, u.w);
     v[4] = df(w.x, w.y);
   }
 };
+
+// Halves of five values (exact), and five sums or differences at once (double-float: values 0, 1 and 2, 3 in packed FP32).
+template <class R>
+__device__ __forceinline__ void half5(const R a[5], R r[5]) {
+#pragma unroll
+  for (int v = 0; v < 5; ++v) r[v] = half_(a[v]);
+}
+__device__ __forceinline__ void half5(const df a[5], df r[5]) {
+  const df2 s = half_(pair_(a[0], a[1])), t = half_(pair_(a[2], a[3]));
+  r[0] = first_(s); r[1] = second_(s); r[2] = first_(t); r[3] = second_(t);
+  r[4] = half_(a[4]);
+}
+template <class R>
+__device__ __forceinline__ void sub5(const R a[5], const R b[5], R r[5]) {
+#pragma unroll
+  for (int v = 0; v < 5; ++v) r[v] = a[v] - b[v];
+}
+__device__ __forceinline__ void sub5(const df a[5], const df b[5], df r[5]) {
+  const df2 s = pair_(a[0], a[1]) - pair_(b[0], b[1]), t = pair_(a[2], a[3]) - pair_(b[2], b[3]);
+  r[0] = first_(s); r[1] = second_(s); r[2] = first_(t); r[3] = second_(t);
+  r[4] = a[4] - b[4];
+}
+template <class R>
+__device__ __forceinline__ void add5(const R a[5], const R b[5], R r[5]) {
+#pragma unroll
+  for (int v = 0; v < 5; ++v) r[v] = a[v] + b[v];
+}
+__device__ __forceinline__ void add5(const df a[5], const df b[5], df r[5]) {
+  const df2 s = pair_(a[0], a[1]) + pair_(b[0], b[1]), t = pair_(a[2], a[3]) + pair_(b[2], b[3]);
+  r[0] = first_(s); r[1] = second_(s); r[2] = first_(t); r[3] = second_(t);
+  r[4] = a[4] + b[4];
+}
+// The flux divergence ((xp - xm) + (yp - ym) - zm) + zp of five fields: in two parts, the z fluxes
+// living in registers (double-float: unnormalised, the update closes it).
+template <class R>
+__device__ __forceinline__ void div_xy(const R xp[5], const R xm[5], const R yp[5], const R ym[5], R d[5]) {
+#pragma unroll
+  for (int v = 0; v < 5; ++v) d[v] = (xp[v] - xm[v]) + (yp[v] - ym[v]);
+}
+template <class R>
+__device__ __forceinline__ void div_z(const R zp[5], const R zm[5], R d[5]) {
+#pragma unroll
+  for (int v = 0; v < 5; ++v) d[v] = (d[v] - zm[v]) + zp[v];
+}
+__device__ __forceinline__ void div_xy(const df xp[5], const df xm[5], const df yp[5], const df ym[5], df d[5]) {
+#pragma unroll
+  for (int v = 0; v < 4; v += 2) {
+    const df2 t = sum_(sum_(pair_(xp[v], xp[v + 1]), neg_(pair_(xm[v], xm[v + 1]))),
+                       sum_(pair_(yp[v], yp[v + 1]), neg_(pair_(ym[v], ym[v + 1]))));
+    d[v] = first_(t);
+    d[v + 1] = second_(t);
+  }
+  d[4] = sum_(sum_(xp[4], -xm[4]), sum_(yp[4], -ym[4]));
+}
+__device__ __forceinline__ void div_z(const df zp[5], const df zm[5], df d[5]) {
+#pragma unroll
+  for (int v = 0; v < 4; v += 2) {
+    const df2 t = sum_(sum_(pair_(d[v], d[v + 1]), neg_(pair_(zm[v], zm[v + 1]))), pair_(zp[v], zp[v + 1]));
+    d[v] = first_(t);
+    d[v + 1] = second_(t);
+  }
+  d[4] = sum_(sum_(d[4], -zm[4]), zp[4]);
+}
 
 template <class Pol, int TX, int TY>
 struct TileShared {
   using R = typename Pol::R;
   Plane5<R, TY + 4, TX + 4> q[3];  // primitive planes p-1, p, p+1 (ring)
   Plane5<R, TY + 2, TX + 2> qh;    // predicted state of plane p (tile + 1 ring)
-  Plane5<R, TY + 2, TX + 2> sx;    // x slopes of plane p
-  Plane5<R, TY + 2, TX + 2> sy;    // y slopes of plane p
+  Plane5<R, TY + 2, TX + 2> sx;    // half x slopes of plane p
+  Plane5<R, TY + 2, TX + 2> sy;    // half y slopes of plane p
   Plane5<R, TY, TX + 1> fx;        // x-face fluxes of plane p, index i+1 for face i+1/2
   Plane5<R, TY + 1, TX> fy;        // y-face fluxes of plane p, index j+1 for face j+1/2
   long long yoff[TY + 4];          // y offset (y index * stride) of the halo rows
@@ -126,27 +191,30 @@ __device__ __forceinline__ R limited_t(R a, R b, int) {
 template <int LIM, class Pol, int TX, int TY>
 __device__ __forceinline__ void predict_cell(TileShared<Pol, TX, TY>& sm, int i, int j, int sm1, int s0, int sp1,
                                              const Params& prm, typename Pol::R hdt, typename Pol::R qh[5],
-                                             typename Pol::R dqz[5]) {
+                                             typename Pol::R dqz[5]) {  // dqz: half the z slopes
   using R = typename Pol::R;
   const int ci = i + 2, cj = j + 2;
-  R c[5], xm[5], xp[5], ym[5], yp[5], zm[5], zp[5], dqx[5], dqy[5];
+  R c[5], dqx[5], dqy[5], h[5];
   sm.q[s0].ld(cj, ci, c);
-  sm.q[s0].ld(cj, ci - 1, xm);
-  sm.q[s0].ld(cj, ci + 1, xp);
-  sm.q[s0].ld(cj - 1, ci, ym);
-  sm.q[s0].ld(cj + 1, ci, yp);
-  sm.q[sm1].ld(cj, ci, zm);
-  sm.q[sp1].ld(cj, ci, zp);
+  auto slope = [&](const auto& lo, int jl, int il, const auto& hi, int jh, int ih, R dq[5]) {
+    R m[5], p[5];
+    lo.ld(jl, il, m);
+    hi.ld(jh, ih, p);
+    sub5(c, m, m);
+    sub5(p, c, p);
 #pragma unroll
-  for (int v = 0; v < 5; ++v) {
-    dqx[v] = limited_t<LIM>(c[v] - xm[v], xp[v] - c[v], prm.limiter);
-    dqy[v] = limited_t<LIM>(c[v] - ym[v], yp[v] - c[v], prm.limiter);
-    dqz[v] = limited_t<LIM>(c[v] - zm[v], zp[v] - c[v], prm.limiter);
-  }
+    for (int v = 0; v < 5; ++v) dq[v] = limited_t<LIM>(m[v], p[v], prm.limiter);
+  };
+  slope(sm.q[s0], cj, ci - 1, sm.q[s0], cj, ci + 1, dqx);
+  slope(sm.q[s0], cj - 1, ci, sm.q[s0], cj + 1, ci, dqy);
+  slope(sm.q[sm1], cj, ci, sm.q[sp1], cj, ci, dqz);
   hancock(c, dqx, dqy, dqz, kc<R>(prm, K_GAMMA), hdt, qh);
   sm.qh.st(j + 1, i + 1, qh);
-  sm.sx.st(j + 1, i + 1, dqx);
-  sm.sy.st(j + 1, i + 1, dqy);
+  half5(dqx, h);
+  sm.sx.st(j + 1, i + 1, h);
+  half5(dqy, h);
+  sm.sy.st(j + 1, i + 1, h);
+  half5(dqz, dqz);
 }
 
 // Flux of the x face between tile cells (i, j) and (i+1, j) (D = 0) or the y face between
@@ -167,11 +235,8 @@ __device__ __forceinline__ void face_flux(TileShared<Pol, TX, TY>& sm, int i, in
     sm.sy.ld(lj, li, sL);
     sm.sy.ld(rj, ri, sR);
   }
-#pragma unroll
-  for (int v = 0; v < 5; ++v) {
-    qL[v] = qL[v] + half_(sL[v]);
-    qR[v] = qR[v] - half_(sR[v]);
-  }
+  add5(qL, sL, qL);
+  sub5(qR, sR, qR);
   floor_state(qL, kc<R>(prm, K_RHOF), kc<R>(prm, K_PF));
   floor_state(qR, kc<R>(prm, K_RHOF), kc<R>(prm, K_PF));
   hllc<D>(qL, qR, kc<R>(prm, K_GAMMA), kc<R>(prm, K_IGM1), F);
@@ -190,11 +255,8 @@ __device__ __forceinline__ void face_flux_dyn(TileShared<Pol, TX, TY>& sm, int d
   const auto& sl = d == 0 ? sm.sx : sm.sy;
   sl.ld(lj, li, sL);
   sl.ld(rj, ri, sR);
-#pragma unroll
-  for (int v = 0; v < 5; ++v) {
-    qL[v] = qL[v] + half_(sL[v]);
-    qR[v] = qR[v] - half_(sR[v]);
-  }
+  add5(qL, sL, qL);
+  sub5(qR, sR, qR);
   floor_state(qL, kc<R>(prm, K_RHOF), kc<R>(prm, K_PF));
   floor_state(qR, kc<R>(prm, K_RHOF), kc<R>(prm, K_PF));
   hllc_dyn(d, qL, qR, kc<R>(prm, K_GAMMA), kc<R>(prm, K_IGM1), F);
@@ -372,13 +434,10 @@ __device__ void step_tile(TileShared<Pol, TX, TY>& sm, const PatchIO<typename Po
 #pragma unroll
   for (int v = 0; v < 5; ++v) { LzPrev[v] = FzPrev[v] = Fz[v] = R(0); }
 
-  auto z_faces = [&](int p, const R qh[5], const R dqz[5]) {
+  auto z_faces = [&](int p, const R qh[5], const R hz[5]) {  // hz: half z slopes
     R Lz[5], Rz[5];
-#pragma unroll
-    for (int v = 0; v < 5; ++v) {
-      Lz[v] = qh[v] + half_(dqz[v]);
-      Rz[v] = qh[v] - half_(dqz[v]);
-    }
+    add5(qh, hz, Lz);
+    sub5(qh, hz, Rz);
     floor_state(Lz, kc<R>(prm, K_RHOF), kc<R>(prm, K_PF));
     floor_state(Rz, kc<R>(prm, K_RHOF), kc<R>(prm, K_PF));
     if (p >= z0) hllc<2>(LzPrev, Rz, gamma, kc<R>(prm, K_IGM1), Fz);
@@ -393,8 +452,8 @@ __device__ void step_tile(TileShared<Pol, TX, TY>& sm, const PatchIO<typename Po
     sm.fx.ld(tj, ti, xm);
     sm.fy.ld(tj + 1, ti, yp);
     sm.fy.ld(tj, ti, ym);
-#pragma unroll
-    for (int v = 0; v < 5; ++v) dF[v] = (xp[v] - xm[v]) + (yp[v] - ym[v]);
+    div_xy(xp, xm, yp, ym, dF);
+    div_z(Fz, FzPrev, dF);
     // the updated cell of this column, written to the output; false where the column lies outside
     // the patch (or, in the bounds-checked build, an index lies outside its array)
     auto write_cell = [&](S Un[5]) -> bool {
@@ -404,8 +463,7 @@ __device__ void step_tile(TileShared<Pol, TX, TY>& sm, const PatchIO<typename Po
       if (!index_ok(ai, in_extent, flags) || !index_ok(ao, (long long)(P.nz + 2 * P.gout) * P.osz, flags)) return false;
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const R div = (dF[v] - FzPrev[v]) + Fz[v];
-        Un[v] = Pol::update(__ldg(P.in[v] + ai), dtdx, div);
+        Un[v] = Pol::update(__ldg(P.in[v] + ai), dtdx, dF[v]);
         P.out[v][ao] = Un[v];
       }
       return true;
