@@ -171,6 +171,26 @@ __device__ __forceinline__ df minmod(const df& a, const df& b) {
   return df(zero ? 0.f : h, zero ? 0.f : l);
 }
 
+// MC alone (the same values as limited(a, b, HYDRO_MC)); double-float selected, not branched.
+template <class R>
+__device__ __forceinline__ R mc_slope(R a, R b) {
+  return limited(a, b, HYDRO_MC);
+}
+__device__ __forceinline__ df mc_pick(const df& a, const df& b, const df& m) {  // m = (a + b)/2
+  const bool pos = a.h > 0.f;
+  const bool le = pos ? !(b < a) : !(a < b);
+  const df t = df(le ? 2.f * a.h : 2.f * b.h, le ? 2.f * a.l : 2.f * b.l);
+  const bool mid = pos ? m < t : t < m;
+  const bool zero = prod_nonpos(a, b);
+  const float h = mid ? m.h : t.h, l = mid ? m.l : t.l;
+  return df(zero ? 0.f : h, zero ? 0.f : l);
+}
+__device__ __forceinline__ df mc_slope(const df& a, const df& b) { return mc_pick(a, b, half_(a + b)); }
+__device__ __forceinline__ df2 mc_slope(const df2& a, const df2& b) {
+  const df2 m = half_(a + b);
+  return pair_(mc_pick(first_(a), first_(b), first_(m)), mc_pick(second_(a), second_(b), second_(m)));
+}
+
 // ------------------------------------------------------------------ Hancock predictor
 // qh = q - hdt * (A_x dqx + A_y dqy + A_z dqz), A_d the primitive Jacobian of direction d.
 template <class R>

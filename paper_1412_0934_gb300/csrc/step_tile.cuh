@@ -185,6 +185,7 @@ __device__ __forceinline__ int ring_slot(int p) { return (p + 3) % 3; }
 template <int LIM, class R>
 __device__ __forceinline__ R limited_t(R a, R b, int) {
   if constexpr (LIM == HYDRO_MINMOD) return minmod(a, b);
+  else if constexpr (LIM == HYDRO_MC) return mc_slope(a, b);
   else return limited(a, b, LIM);
 }
 
