@@ -387,7 +387,8 @@ int hydro_autotune(hydro_ctx* ctx, const hydro_patch* in, const hydro_patch* out
                    const char* cache_path);
 
 /* Current tile configuration: *tile_id (index into the compiled tile shapes) and *zchunk (no
- * counterpart in the paper).  Compiled shapes (columns x rows of one block's tile): 0 16 x 16,
+ * counterpart in the paper).  A context that no call has tuned reports 0, 32; its hydro_step and
+ * hydro_run then choose tile and chunk per box or patch set by a cost rule (the results are the same).  Compiled shapes (columns x rows of one block's tile): 0 16 x 16,
  * 1 32 x 8, 2 8 x 8, 3 32 x 16, 4 16 x 16 with a whole SM's registers for one block; the PPM
  * kernel has one shape (16 x 16) and ignores tile_id.  hydro_set_tuning refuses tile_id outside
  * [0, HYDRO_NUM_TILES) and zchunk outside [1, 4096]. */

@@ -38,6 +38,7 @@ struct hydro_ctx {
   int ntiles = 0;
   int* d_counter = nullptr;  // 1 + HYDRO_NUM_PATCH_CLASSES tile counters
   int wl_tile = -1, wl_zchunk = -1;
+  bool wl_tuned = false;  // the work-list was built for the caller's tuning (else for the rule's)
   // tile shape per patch-shape class (-1: the context's tile_id / zchunk); the work-list of a batch
   // built per class: its entries' patches (d_cls_idx), their offsets in the work-list and counts
   int cls_tile[HYDRO_NUM_PATCH_CLASSES] = {-1, -1, -1}, cls_zc[HYDRO_NUM_PATCH_CLASSES] = {0, 0, 0};
@@ -53,8 +54,11 @@ struct hydro_ctx {
   HostPatchIO* h_cfl = nullptr;
   HostPatchIO* d_cfl = nullptr;
   size_t cfl_cap = 0;
-  // tuning
+  // tuning; until a caller sets it (hydro_set_tuning, hydro_set_class_tuning, hydro_autotune), hydro_step
+  // and hydro_run take each box's and patch set's tile shape and z chunk from the rule of default_tuning
   int tile_id = 0, zchunk = 32;
+  bool tuned = false;
+  int rule_n[3] = {0, 0, 0}, rule_tile = 0, rule_zc = 0;  // the rule's choice for the last box size
   // graph cache of hydro_run
   cudaGraphExec_t graph = nullptr;
   const void* g_a = nullptr;
@@ -62,6 +66,7 @@ struct hydro_ctx {
   int g_n = -1;
   double* g_dt = nullptr;
   int g_tile = -1, g_zc = -1;
+  bool g_tuned = false;
   // adjoint scratch
   void* d_adj = nullptr;
   size_t adj_cap = 0;
@@ -220,13 +225,109 @@ bool per_class(const hydro_ctx* c) {
 int class_tile(const hydro_ctx* c, int k) { return c->cls_tile[k] >= 0 ? c->cls_tile[k] : c->tile_id; }
 int class_zc(const hydro_ctx* c, int k) { return c->cls_tile[k] >= 0 ? c->cls_zc[k] : c->zchunk; }
 
+// ------------------------------------------------------------------ default tuning
+// The tile shape and z chunk of a box or patch set whose context has no tuning of the caller's, from a
+// cost model of the step kernels: a block marching zc planes alone on an SM takes plane * (zc + start)
+// microseconds, and k blocks resident together (at most `resident`) take share[k] times that.  With n =
+// ceil(blocks / SMs) blocks per SM the launch takes their rounds, full ones of `resident` blocks and the
+// rest.  Short chunks fill the SMs of a small box (32^3 at one 32-plane chunk of 16x16 tiles is 4 blocks)
+// and repeat two planes each; long ones serve the large boxes.  The constants are fits to steps of 16^3
+// to 512^3 boxes at 2 to 128-plane chunks; the model stays within 5% of those and picks, against the
+// fixed 16x16 tiles of 32 planes: FP64 32^3 1367 -> 97 us, double-float 64^3 359 -> 77, FP32 96^3 76 -> 46,
+// mixed 64^3 124 -> 33; 512^3 within 1% of the best of the sweep.
+struct ShapeCost {
+  int tile;
+  double plane, start;
+  int resident;
+  double share[4];
+};
+constexpr ShapeCost kCostF64[] = {{0, 41.0, 1.2, 2, {0.0, 1.0, 1.77}},
+                                  {2, 28.4, 1.25, 3, {0.0, 1.0, 1.0, 1.27}},
+                                  {3, 73.6, 1.04, 1, {0.0, 1.0}}};
+constexpr ShapeCost kCostDF[] = {{0, 10.5, 1.9, 2, {0.0, 1.0, 1.3}}, {3, 13.25, 1.8, 1, {0.0, 1.0}}};
+constexpr ShapeCost kCostF32[] = {{0, 1.95, 5.3, 3, {0.0, 1.0, 1.29, 1.76}},
+                                  {1, 1.94, 5.3, 3, {0.0, 1.0, 1.29, 1.76}},
+                                  {3, 2.5, 4.9, 1, {0.0, 1.0}}};
+constexpr ShapeCost kCostMixed[] = {{0, 3.4, 4.0, 3, {0.0, 1.0, 1.27, 1.65}},
+                                    {1, 3.38, 4.0, 3, {0.0, 1.0, 1.27, 1.65}},
+                                    {3, 4.55, 3.2, 1, {0.0, 1.0}}};
+constexpr ShapeCost kCostPpm8[] = {{0, 1.0, 4.0, 1, {0.0, 1.0}}};  // one tile shape: only the chunk is chosen
+constexpr ShapeCost kCostPpm4[] = {{0, 1.0, 4.0, 2, {0.0, 1.0, 1.3}}};
+
+double rounds(const ShapeCost& s, long long n) {
+  return (double)(n / s.resident) * s.share[s.resident] + s.share[n % s.resident];
+}
+
+void default_tuning(const hydro_ctx* c, const hydro_patch* in, int n, int* tile, int* zchunk) {
+  const ShapeCost* shapes = kCostF64;
+  int ns = 3;
+  switch (c->cfg.precision) {
+    case HYDRO_FP32: shapes = kCostF32; break;
+    case HYDRO_MIXED: shapes = kCostMixed; break;
+    case HYDRO_FP64_DF: shapes = kCostDF; ns = 2; break;
+  }
+  if (ppm(c)) {
+    shapes = (c->cfg.precision == HYDRO_FP32 || c->cfg.precision == HYDRO_MIXED) ? kCostPpm4 : kCostPpm8;
+    ns = 1;
+  }
+  int maxnz = 1;
+  for (int i = 0; i < n; ++i) maxnz = std::max(maxnz, in[i].nz);
+  double best = 1e300;
+  *tile = 0;
+  *zchunk = 32;
+  // the fixed 16x16 tiles of 32 planes first: another choice has to save 3% of their time
+  long long blocks0 = -1;  // blocks of those
+  auto consider = [&](int zc, int kinds) {
+    for (int k = 0; k < kinds; ++k) {
+      const ShapeCost& s = shapes[k];
+      const int tx = hydro::kTileX[s.tile], ty = hydro::kTileY[s.tile];
+      long long blocks = 0;
+      double planes = 0.0;  // marched by all blocks, their start planes included
+      for (int i = 0; i < n; ++i) {
+        const long long cols = (long long)((in[i].nx + tx - 1) / tx) * ((in[i].ny + ty - 1) / ty);
+        const long long chunks = (in[i].nz + zc - 1) / zc;
+        blocks += cols * chunks;
+        planes += (double)cols * (in[i].nz + chunks * s.start);
+      }
+      if (blocks0 < 0) blocks0 = blocks;
+      const long long per_sm = (blocks + c->sm_count - 1) / c->sm_count;
+      const double t = s.plane * planes / (double)blocks * rounds(s, per_sm);
+      if (t < best) {
+        best = best == 1e300 ? 0.97 * t : t;
+        *tile = s.tile;
+        *zchunk = zc;
+      }
+    }
+  };
+  consider(32, 1);
+  // Where that fills every SM four times over there is little left to balance, and differences the model
+  // does not hold (caches, uneven patches, the last tiles' tail) decide: the batched, FP64 and PPM steps
+  // keep it (4096 uneven patches, mixed: 10.8 ms, 11.6 with the model's choice; FP64 256^3 16.4 against
+  // 16.9).  Uniform boxes in double-float and float still gain 3-4% from fewer start planes.
+  if (blocks0 >= 4LL * shapes[0].resident * c->sm_count && (n > 1 || ppm(c) || c->cfg.precision == HYDRO_FP64)) return;
+  if (n == 1) {
+    // one box: every chunk count up to 64, and two-plane chunks at the least
+    for (int k = 1; k <= 64; ++k) {
+      const int zc = (maxnz + k - 1) / k;
+      if (zc > 128 && k < 64) continue;
+      consider(std::min(zc, 4096), ns);
+      if (zc <= 2) break;
+    }
+  } else {
+    for (int zc : {2, 4, 8, 16, 32}) {
+      consider(zc, ns);
+      if (zc >= maxnz) break;
+    }
+  }
+}
+
 // Upload the descriptors of (in, out) and build the tile work-list for the current tuning,
 // unless the cached set and tuning are unchanged.  With a tile shape per patch-shape class the
 // work-list holds one segment per class, each built with its class's tile shape and z chunk.
 int prepare_batch(hydro_ctx* c, const hydro_patch* in, const hydro_patch* out, int n) {
   const bool set_same = same_set(c->key_in, in, n) && same_set(c->key_out, out, n);
-  const int tile = ppm(c) ? 0 : c->tile_id;  // the PPM kernel's tiles are 16 x 16 (tile shape 0)
-  const int tx = hydro::kTileX[tile], ty = hydro::kTileY[tile];
+  // the PPM kernel's tiles are 16 x 16 (tile shape 0)
+  int tile = ppm(c) ? 0 : c->tile_id, zchunk = c->zchunk;
   const bool pc = per_class(c);
   int cls_key[2 * HYDRO_NUM_PATCH_CLASSES];
   for (int k = 0; k < HYDRO_NUM_PATCH_CLASSES; ++k) {
@@ -234,8 +335,11 @@ int prepare_batch(hydro_ctx* c, const hydro_patch* in, const hydro_patch* out, i
     cls_key[2 * k + 1] = class_zc(c, k);
   }
   if (set_same && pc == c->wl_per_class &&
-      (pc ? std::memcmp(cls_key, c->wl_cls, sizeof(cls_key)) == 0 : (c->wl_tile == tile && c->wl_zchunk == c->zchunk)))
+      (pc ? std::memcmp(cls_key, c->wl_cls, sizeof(cls_key)) == 0
+          : c->wl_tuned == c->tuned && (!c->tuned || (c->wl_tile == tile && c->wl_zchunk == zchunk))))
     return HYDRO_OK;
+  if (!c->tuned) default_tuning(c, in, n, &tile, &zchunk);
+  const int tx = hydro::kTileX[tile], ty = hydro::kTileY[tile];
   if (!set_same) {
     size_t old = c->patches_cap;
     int rc = ensure_device(&c->d_patches, &c->patches_cap, (size_t)n);
@@ -304,18 +408,19 @@ int prepare_batch(hydro_ctx* c, const hydro_patch* in, const hydro_patch* out, i
   // tile count on the host sizes the buffer; the device builds the list itself
   size_t total = 0;
   for (int i = 0; i < n; ++i)
-    total += (size_t)((in[i].nx + tx - 1) / tx) * ((in[i].ny + ty - 1) / ty) * ((in[i].nz + c->zchunk - 1) / c->zchunk);
+    total += (size_t)((in[i].nx + tx - 1) / tx) * ((in[i].ny + ty - 1) / ty) * ((in[i].nz + zchunk - 1) / zchunk);
   if (total > 0x7fffffff) return HYDRO_ERR_ARG;
   int rc = ensure_device(&c->d_counts, &c->counts_cap, (size_t)n + 1);
   if (rc) return rc;
   rc = ensure_device(&c->d_tiles, &c->tiles_cap, total);
   if (rc) return rc;
-  if (hydro::build_worklist(c->d_patches, n, tx, ty, c->zchunk, c->d_counts, c->d_tiles, c->stream) != cudaSuccess)
+  if (hydro::build_worklist(c->d_patches, n, tx, ty, zchunk, c->d_counts, c->d_tiles, c->stream) != cudaSuccess)
     return HYDRO_ERR_CUDA;
   c->launches += 3;
   c->ntiles = (int)total;
   c->wl_tile = tile;
-  c->wl_zchunk = c->zchunk;
+  c->wl_zchunk = zchunk;
+  c->wl_tuned = c->tuned;
   c->wl_per_class = false;
   return HYDRO_OK;
 }
@@ -331,9 +436,18 @@ int step_one_uniform(hydro_ctx* c, const hydro_patch& in, const hydro_patch& out
     int rc = reset_slots(c, dt_next, 1, s);
     if (rc) return rc;
   }
-  int zc = std::min(c->zchunk, in.nz);
+  int tile = c->tile_id, zc = c->zchunk;
+  if (!c->tuned) {
+    if (c->rule_n[0] != in.nx || c->rule_n[1] != in.ny || c->rule_n[2] != in.nz) {
+      default_tuning(c, &in, 1, &c->rule_tile, &c->rule_zc);
+      c->rule_n[0] = in.nx; c->rule_n[1] = in.ny; c->rule_n[2] = in.nz;
+    }
+    tile = c->rule_tile;
+    zc = c->rule_zc;
+  }
+  zc = std::min(zc, in.nz);
   cudaError_t e = ppm(c) ? c->ops->step_ppm(make_io(in, out), c->prm, dt, dt_next, zc, c->d_err, s)
-                         : c->ops->step_uniform(c->tile_id, make_io(in, out), c->prm, dt, dt_next, zc, c->d_err, s);
+                         : c->ops->step_uniform(tile, make_io(in, out), c->prm, dt, dt_next, zc, c->d_err, s);
   c->launches += 1;
   return cuda_status(e);
 }
@@ -549,11 +663,11 @@ int hydro_step(hydro_ctx* c, const hydro_patch* in, const hydro_patch* out, int 
   c->launches += 1;
   if (ppm(c))
     return cuda_status(c->ops->step_ppm_batched(c->d_patches, c->d_tiles, c->ntiles, c->d_counter, c->prm, dt_dev,
-                                                dt_next_dev, c->zchunk, c->d_err, c->sm_count, c->stream));
-  const int per_sm = c->ops->batched_blocks_per_sm(c->tile_id, c->cfg.limiter);
+                                                dt_next_dev, c->wl_zchunk, c->d_err, c->sm_count, c->stream));
+  const int per_sm = c->ops->batched_blocks_per_sm(c->wl_tile, c->cfg.limiter);
   int grid = std::max(1, std::min(c->ntiles, c->sm_count * per_sm));
-  return cuda_status(c->ops->step_batched(c->tile_id, c->d_patches, c->d_tiles, c->ntiles, c->d_counter, c->prm,
-                                          dt_dev, dt_next_dev, c->zchunk, c->d_err, grid, c->stream));
+  return cuda_status(c->ops->step_batched(c->wl_tile, c->d_patches, c->d_tiles, c->ntiles, c->d_counter, c->prm,
+                                          dt_dev, dt_next_dev, c->wl_zchunk, c->d_err, grid, c->stream));
 }
 
 // Host-buffer step of one periodic box: the state crosses the host link in z slabs on two copy
@@ -1364,7 +1478,7 @@ int hydro_run(hydro_ctx* c, const hydro_patch* a, const hydro_patch* b, int nste
   };
   if (!use_graph) return enqueue(c->stream);
   const bool hit = c->graph && c->g_a == a->U[0] && c->g_b == b->U[0] && c->g_n == nsteps && c->g_dt == dt_hist_dev &&
-                   c->g_tile == c->tile_id && c->g_zc == c->zchunk;
+                   c->g_tile == c->tile_id && c->g_zc == c->zchunk && c->g_tuned == c->tuned;
   if (!hit) {
     if (c->graph) cudaGraphExecDestroy(c->graph);
     c->graph = nullptr;
@@ -1391,6 +1505,7 @@ int hydro_run(hydro_ctx* c, const hydro_patch* a, const hydro_patch* b, int nste
     c->g_dt = dt_hist_dev;
     c->g_tile = c->tile_id;
     c->g_zc = c->zchunk;
+    c->g_tuned = c->tuned;
   }
   c->launches += nsteps + 1;
   return cuda_status(cudaGraphLaunch(c->graph, c->stream));
@@ -1407,6 +1522,7 @@ int hydro_set_tuning(hydro_ctx* c, int tile_id, int zchunk) {
   if (!c || tile_id < 0 || tile_id >= hydro::kNumTiles || zchunk < 1 || zchunk > 4096) return HYDRO_ERR_ARG;
   c->tile_id = tile_id;
   c->zchunk = zchunk;
+  c->tuned = true;
   for (int k = 0; k < HYDRO_NUM_PATCH_CLASSES; ++k) c->cls_tile[k] = -1;
   return HYDRO_OK;
 }
@@ -1456,6 +1572,7 @@ int hydro_autotune(hydro_ctx* c, const hydro_patch* in, const hydro_patch* out, 
         if (ok) {
           c->tile_id = t;
           c->zchunk = z;
+          c->tuned = true;
           for (int k = 0; k < NC; ++k) {
             c->cls_tile[k] = ct[k];
             c->cls_zc[k] = cz[k];
@@ -1467,6 +1584,8 @@ int hydro_autotune(hydro_ctx* c, const hydro_patch* in, const hydro_patch* out, 
       std::fclose(f);
     }
   }
+  const bool was_tuned = c->tuned;
+  c->tuned = true;
   for (int k = 0; k < NC; ++k) c->cls_tile[k] = -1;
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
@@ -1556,6 +1675,7 @@ int hydro_autotune(hydro_ctx* c, const hydro_patch* in, const hydro_patch* out, 
   cudaEventDestroy(e1);
   if (rc) {
     for (int k = 0; k < NC; ++k) c->cls_tile[k] = -1;
+    c->tuned = was_tuned;
     return rc;
   }
   c->tile_id = bt;
