@@ -146,7 +146,8 @@ int hydro_cfl_dt(hydro_ctx* ctx, const hydro_patch* p, int npatch, double* dt_de
  * step.  A single periodic box (npatch == 1, ng == 0) runs the uniform-grid kernel; any other
  * set (in[p] with ng == 2, or 3 in a HYDRO_PPM context) runs one persistent launch over a
  * device-built tile work-list.  The descriptors are
- * uploaded and the work-list rebuilt only when the patch set differs from the previous call's. */
+ * uploaded and the work-list built when the patch set is none of the last four calls' (a level that
+ * steps from one buffer set to another and back builds each once). */
 int hydro_step(hydro_ctx* ctx, const hydro_patch* in, const hydro_patch* out, int npatch, const double* dt_dev,
                double* dt_next_dev);
 
@@ -170,8 +171,8 @@ int hydro_step_octs(hydro_ctx* ctx, void* const gathered[5], void* const out[5],
  *                 level or one another;
  *   fine_origins: host array [npatch][3] of int (x, y, z): the fine-level index of each patch's
  *                 first interior cell (any integers: fine indices wrap with the level's period).
- * Arithmetic in the storage type.  A call with a patch set different from the previous call's
- * uploads its descriptors and synchronises the stream first. */
+ * Arithmetic in the storage type.  A call with a patch set other than the last few uploads its
+ * descriptors (enqueued on the stream). */
 int hydro_fill_ghosts(hydro_ctx* ctx, const hydro_patch* coarse, const hydro_patch* fine, const int* fine_origins,
                       int npatch);
 
@@ -192,9 +193,9 @@ int hydro_fill_ghosts_time(hydro_ctx* ctx, const hydro_patch* coarse_old, const 
  *   fine:    npatch patches, ng == 2, interiors no larger than the period and not overlapping one
  *            another (modulo the period); they must not share memory;
  *   origins: host array [npatch][3] of int: each patch's first interior cell (wrapped by the period).
- * Deterministic (each ghost cell has at most one source).  A call with a patch set different from
- * the previous call's builds its copy list on the host (a spatial hash of the interiors) and
- * synchronises the stream first. */
+ * Deterministic (each ghost cell has at most one source).  A call with a patch set other than
+ * the last few builds its copy list on the host (a spatial hash of the interiors) and uploads it
+ * (enqueued on the stream). */
 int hydro_exchange_ghosts(hydro_ctx* ctx, const hydro_patch* fine, const int* origins, int npatch, const int period[3]);
 
 /* Flux registers, refluxing and average-down: the coupling of two AMR levels (refinement ratio 2)
@@ -219,8 +220,8 @@ int hydro_exchange_ghosts(hydro_ctx* ctx, const hydro_patch* fine, const int* or
  *       are applied in turn, so the result is deterministic.
  *   hydro_average_down: the coarse cells under each fine patch's interior (fine origin and sizes
  *       even) become the mean of their eight children.
- * A call whose descriptors differ from the previous call of the same kind uploads them and
- * synchronises the stream first. */
+ * A call whose descriptors are not those of one of the last few calls of the same kind uploads them
+ * (enqueued on the stream). */
 int hydro_patch_fluxes(hydro_ctx* ctx, const hydro_patch* patches, int npatch, const double* dt_dev,
                        void* const* registers, int accumulate);
 int hydro_level_fluxes(hydro_ctx* ctx, const hydro_patch* level, const int* box_origins, const int* box_dims, int nbox,
@@ -320,8 +321,8 @@ typedef struct {
  *       81 elements per cell of each patch's interior grown by one cell per side.
  *   hydro_mhd_cfl_patches: dt_dev[p] <- the CFL dt of each patch's interior (bit-identical to the
  *       fused one).
- * Precisions and errors as hydro_mhd_step.  The descriptors are uploaded when the patch set differs
- * from the previous call's (the stream is synchronised first). */
+ * Precisions and errors as hydro_mhd_step.  The descriptors are uploaded when the patch set is
+ * none of the last few calls'. */
 int hydro_mhd_step_patches(hydro_ctx* ctx, const hydro_mhd_patch* in, const hydro_mhd_patch* out, int npatch,
                            const double* dt_dev, double* dt_next_dev);
 int hydro_mhd_cfl_patches(hydro_ctx* ctx, const hydro_mhd_patch* p, int npatch, double* dt_dev);

@@ -8,7 +8,9 @@ There is no CPU fallback: if the library is not built, or no GPU is present, cal
 A patch is built from a tensor of shape (5, nz + 2 ng, ny + 2 ng, nx + 2 ng) (fields rho, m_x,
 m_y, m_z, E; x fastest) with ``patch(U, ng, dx)``; float64 for FP64/MIXED, float32 for FP32.
 """
+import array
 import ctypes
+import itertools
 import os
 
 import torch
@@ -174,8 +176,7 @@ class MhdPatch:
 
 
 def _mhd_parray(patches):
-    patches = list(patches)
-    return (hydro_mhd_patch * len(patches))(*[p.c for p in patches]), len(patches)
+    return _struct_array(hydro_mhd_patch, list(patches))
 
 
 class Patch:
@@ -220,10 +221,17 @@ def host_patch(fields, dx):
     return Patch(fields, 0, dx, host=True)
 
 
+def _struct_array(struct, patches):
+    """C array of the patches' descriptors, and their number: the structures' bytes joined in one go (a
+    level holds thousands of patches; assigning them one by one took longer than the call's kernels)."""
+    n = len(patches)
+    if n == 1:
+        return (struct * 1)(patches[0].c), 1
+    return (struct * n).from_buffer_copy(b"".join([p.c for p in patches])) if n else (struct * 0)(), n
+
+
 def _parray(patches):
-    patches = [patches] if isinstance(patches, Patch) else list(patches)
-    arr = (hydro_patch * len(patches))(*[p.c for p in patches])
-    return arr, len(patches)
+    return _struct_array(hydro_patch, [patches] if isinstance(patches, Patch) else list(patches))
 
 
 def _ptr(t):
@@ -244,11 +252,14 @@ def _f64(t, n, what):
 
 
 def _dtypes(obj):
+    """The set of element types of a patch, a tensor, or nested lists of them."""
     if isinstance(obj, (Patch, MhdPatch, torch.Tensor)):
-        yield obj.dtype
-    elif isinstance(obj, (list, tuple)):
-        for o in obj:
-            yield from _dtypes(o)
+        return {obj.dtype}
+    if isinstance(obj, (list, tuple)):
+        if set(map(type, obj)) <= {Patch, MhdPatch, torch.Tensor}:
+            return {o.dtype for o in obj}
+        return set().union(*[_dtypes(o) for o in obj])
+    return set()
 
 
 def _same_dtype(ctx, *objs):
@@ -331,9 +342,7 @@ def hydro_fill_ghosts(ctx, coarse, fine, origins):
     """Fill the ghost layers of the fine patches (list of Patch, ng = 2) from the periodic coarse
     Patch; origins: (x, y, z) fine-level index of each patch's first interior cell."""
     f, n = _parray(fine)
-    o = (ctypes.c_int * (3 * n))(*[int(v) for xyz in origins for v in xyz])
-    if len(o) != 3 * n:
-        raise ValueError("one (x, y, z) origin per patch")
+    o = _origins(origins, n)
     _same_dtype(ctx, coarse, fine)
     _check(lib().hydro_fill_ghosts(ctx.handle, ctypes.byref(coarse.c), f, o, n), "hydro_fill_ghosts")
 
@@ -342,9 +351,7 @@ def hydro_fill_ghosts_time(ctx, coarse_old, coarse_new, theta, fine, origins):
     """hydro_fill_ghosts from the coarse level at the fraction theta of its step:
     (1 - theta) coarse_old + theta coarse_new, then prolonged."""
     f, n = _parray(fine)
-    o = (ctypes.c_int * (3 * n))(*[int(v) for xyz in origins for v in xyz])
-    if len(o) != 3 * n:
-        raise ValueError("one (x, y, z) origin per patch")
+    o = _origins(origins, n)
     _same_dtype(ctx, coarse_old, coarse_new, fine)
     _check(lib().hydro_fill_ghosts_time(ctx.handle, ctypes.byref(coarse_old.c), ctypes.byref(coarse_new.c),
                                         float(theta), f, o, n), "hydro_fill_ghosts_time")
@@ -354,9 +361,7 @@ def hydro_exchange_ghosts(ctx, fine, origins, period):
     """Ghosts of the patches (list of Patch, ng = 2) covered by a same-level interior take its
     values; origins: first interior cell (x, y, z) per patch; period: (x, y, z) of the level."""
     f, n = _parray(fine)
-    o = (ctypes.c_int * (3 * n))(*[int(v) for xyz in origins for v in xyz])
-    if len(o) != 3 * n:
-        raise ValueError("one (x, y, z) origin per patch")
+    o = _origins(origins, n)
     per = (ctypes.c_int * 3)(*[int(v) for v in period])
     _same_dtype(ctx, fine)
     _check(lib().hydro_exchange_ghosts(ctx.handle, f, o, n, per), "hydro_exchange_ghosts")
@@ -368,12 +373,29 @@ def register_size(nx, ny, nz):
 
 
 def _ints(rows):
-    flat = [int(v) for r in rows for v in r]
-    return (ctypes.c_int * len(flat))(*flat)
+    """C ints of the rows' values, in order."""
+    rows = list(rows)
+    try:
+        flat = array.array("i", list(itertools.chain.from_iterable(rows)))
+    except (TypeError, OverflowError):  # values that int() converts and an int array does not take
+        flat = [int(v) for r in rows for v in r]
+        return (ctypes.c_int * len(flat))(*flat)
+    return (ctypes.c_int * len(flat)).from_buffer(flat) if len(flat) else (ctypes.c_int * 0)()
+
+
+def _origins(origins, n):
+    """C ints of n (x, y, z) origins."""
+    o = _ints(origins)
+    if len(o) > 3 * n:
+        raise ValueError("one (x, y, z) origin per patch")
+    return o if len(o) == 3 * n else (ctypes.c_int * (3 * n))(*o)
 
 
 def _ptrs(tensors):
-    return (ctypes.c_void_p * len(tensors))(*[_ptr(t) for t in tensors])
+    tensors = list(tensors)
+    if not all([t is not None and t.is_cuda for t in tensors]):
+        return (ctypes.c_void_p * len(tensors))(*[_ptr(t) for t in tensors])
+    return (ctypes.c_void_p * len(tensors))(*[t.data_ptr() for t in tensors])
 
 
 def hydro_patch_fluxes(ctx, patches, dt, registers, accumulate=False):

@@ -18,6 +18,58 @@
 using hydro::HostPatchIO;
 using hydro::HostTileRec;
 
+// What a call derives from its descriptors (field pointers, shapes, origins, boxes) and keeps on the
+// device: descriptor copies, block tables, copy tasks, work-lists.  The last kKept sets of each kind of
+// call stay, the least recently used making room: a level's patches step from one buffer set to another
+// and back, so consecutive calls alternate between sets (with one kept set, each substep of a subcycled
+// level rebuilt its tables and drained the stream for it).
+struct SetCache {
+  static constexpr int kKept = 4;
+  struct Entry {
+    std::vector<char> key;
+    bool valid = false;
+    unsigned long long used = 0;
+    char* d = nullptr;
+    size_t cap = 0;
+    size_t off[4] = {};  // offsets of the parts in d
+    int n[10] = {};      // counts and settings of the set
+  };
+  Entry entry[kKept];
+  unsigned long long clock = 0;
+  Entry* find(const std::vector<char>& key) {
+    for (Entry& e : entry)
+      if (e.valid && e.key == key) {
+        e.used = ++clock;
+        return &e;
+      }
+    return nullptr;
+  }
+  // The entry to fill for a new key, with room for n bytes (nullptr: no memory); valid once the
+  // caller has enqueued its contents and calls done().
+  Entry* replace(size_t n) {
+    Entry* o = &entry[0];
+    for (Entry& e : entry)
+      if (e.used < o->used) o = &e;
+    o->valid = false;
+    if (o->cap < n) {
+      cudaFree(o->d);
+      o->d = nullptr;
+      o->cap = 0;
+      if (cudaMalloc(&o->d, n + n / 4) != cudaSuccess) return nullptr;
+      o->cap = n + n / 4;
+    }
+    return o;
+  }
+  void done(Entry* e, std::vector<char>&& key) {
+    e->key = std::move(key);
+    e->used = ++clock;
+    e->valid = true;
+  }
+  void free_all() {
+    for (Entry& e : entry) cudaFree(e.d);
+  }
+};
+
 struct hydro_ctx {
   hydro_config cfg;
   hydro::Params prm;
@@ -26,34 +78,19 @@ struct hydro_ctx {
   const hydro::KernelOps* ops = nullptr;
   int device = 0, sm_count = 0;
   unsigned* d_err = nullptr;
-  // batched step: cached patch set, device descriptors and work-list
-  std::vector<hydro_patch> key_in, key_out;
-  HostPatchIO* h_patches = nullptr;  // pinned staging
-  HostPatchIO* d_patches = nullptr;
-  size_t patches_cap = 0;
-  int* d_counts = nullptr;
-  size_t counts_cap = 0;
-  HostTileRec* d_tiles = nullptr;
-  size_t tiles_cap = 0;
-  int ntiles = 0;
+  // page-locked staging of uploads: two buffers in turn, each reused once its last copy has run
+  char* h_stage[2] = {nullptr, nullptr};
+  size_t h_stage_cap[2] = {0, 0};
+  cudaEvent_t ev_stage[2] = {nullptr, nullptr};
+  int stage_turn = 0;
+  // batched step: descriptors and work-list of the last patch sets
+  SetCache batch;
   int* d_counter = nullptr;  // 1 + HYDRO_NUM_PATCH_CLASSES tile counters
-  int wl_tile = -1, wl_zchunk = -1;
-  bool wl_tuned = false;  // the work-list was built for the caller's tuning (else for the rule's)
-  // tile shape per patch-shape class (-1: the context's tile_id / zchunk); the work-list of a batch
-  // built per class: its entries' patches (d_cls_idx), their offsets in the work-list and counts
+  // tile shape per patch-shape class (-1: the context's tile_id / zchunk)
   int cls_tile[HYDRO_NUM_PATCH_CLASSES] = {-1, -1, -1}, cls_zc[HYDRO_NUM_PATCH_CLASSES] = {0, 0, 0};
-  bool wl_per_class = false;
-  int wl_cls[2 * HYDRO_NUM_PATCH_CLASSES] = {};
-  int* d_cls_idx = nullptr;
-  size_t cls_idx_cap = 0;
-  int cls_off[HYDRO_NUM_PATCH_CLASSES] = {}, cls_ntiles[HYDRO_NUM_PATCH_CLASSES] = {};
   double* d_cls_dt = nullptr;  // the autotuner's per-class time steps
   size_t cls_dt_cap = 0;
-  // CFL of many patches: cached descriptors
-  std::vector<hydro_patch> cfl_key;
-  HostPatchIO* h_cfl = nullptr;
-  HostPatchIO* d_cfl = nullptr;
-  size_t cfl_cap = 0;
+  SetCache cfl_sets;  // CFL of many patches: descriptors
   // tuning; until a caller sets it (hydro_set_tuning, hydro_set_class_tuning, hydro_autotune), hydro_step
   // and hydro_run take each box's and patch set's tile shape and z chunk from the rule of default_tuning
   int tile_id = 0, zchunk = 32;
@@ -86,27 +123,12 @@ struct hydro_ctx {
   cudaEvent_t ev_ready = nullptr;
   std::vector<cudaEvent_t> ev_copied, ev_stepped, ev_halo;
   cudaEvent_t ev_begin = nullptr, ev_end = nullptr;
-  // coarse-to-fine ghost fill: uploaded patch descriptors and ghost-cell offsets of the last set
-  std::vector<hydro::HostGhostPatch> ghost_key;
-  hydro::HostGhostPatch* d_ghost = nullptr;
-  size_t ghost_cap = 0;
-  int2* d_ghost_blocks = nullptr;
-  size_t ghost_blocks_cap = 0;
-  int ghost_nblocks = 0;
-  // same-level ghost exchange: uploaded patch descriptors and copy tasks of the last set
-  std::vector<hydro::HostGhostPatch> xchg_key;
-  int xchg_period[3] = {0, 0, 0};
-  hydro::HostGhostPatch* d_xchg = nullptr;
-  size_t xchg_cap = 0;
-  hydro::HostCopyTask* d_tasks = nullptr;
-  size_t tasks_cap = 0;
-  int ntasks = 0;
-  // flux registers (patch boxes, level boxes), refluxing, average-down: descriptors and block
-  // tables of the last call of each kind (reused without an upload when unchanged)
+  // coarse-to-fine ghost fill: descriptors and block table; same-level exchange: descriptors and tasks
+  SetCache ghost_sets, xchg_sets;
+  // flux registers (patch boxes, level boxes), refluxing, average-down, MHD step and CFL on patches:
+  // descriptors and block tables
   static constexpr int kAux = 6;  // 0, 1 box fluxes; 2 reflux; 3 average-down; 4 MHD step; 5 MHD CFL
-  char* d_aux[kAux] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-  size_t aux_cap[kAux] = {0, 0, 0, 0, 0, 0};
-  std::vector<char> aux_last[kAux];
+  SetCache aux[kAux];
   // oct builder scratch: key bitmap, word prefix sums, block prefix sums
   unsigned* d_octs_scratch = nullptr;
   size_t octs_scratch_cap = 0;
@@ -188,15 +210,6 @@ HostPatchIO make_io(const hydro_patch& in, const hydro_patch& out) {
   return h;
 }
 
-bool same_patch(const hydro_patch& a, const hydro_patch& b) { return std::memcmp(&a, &b, sizeof(hydro_patch)) == 0; }
-
-bool same_set(const std::vector<hydro_patch>& key, const hydro_patch* p, int n) {
-  if ((int)key.size() != n) return false;
-  for (int i = 0; i < n; ++i)
-    if (!same_patch(key[i], p[i])) return false;
-  return true;
-}
-
 template <class T>
 int ensure_device(T** d, size_t* cap, size_t n) {
   if (*cap >= n) return HYDRO_OK;
@@ -206,6 +219,55 @@ int ensure_device(T** d, size_t* cap, size_t n) {
   if (cudaMalloc(reinterpret_cast<void**>(d), n * sizeof(T)) != cudaSuccess) return HYDRO_ERR_NOMEM;
   *cap = n;
   return HYDRO_OK;
+}
+
+template <class T>
+size_t append(std::vector<char>& bytes, const T* p, size_t n) {
+  const size_t off = (bytes.size() + 255) / 256 * 256;
+  bytes.resize(off + n * sizeof(T));
+  if (n) std::memcpy(bytes.data() + off, p, n * sizeof(T));
+  return off;
+}
+
+// Enqueue the copy of n host bytes to device memory on the context's stream, through page-locked
+// staging: the caller may free p, and the stream's order keeps earlier readers of d safe, so nothing
+// is drained.
+bool upload(hydro_ctx* c, void* d, const void* p, size_t n) {
+  if (n == 0) return true;
+  const int t = c->stage_turn ^= 1;
+  if (!c->ev_stage[t] && cudaEventCreateWithFlags(&c->ev_stage[t], cudaEventDisableTiming) != cudaSuccess) return false;
+  if (c->h_stage[t] && cudaEventSynchronize(c->ev_stage[t]) != cudaSuccess) return false;
+  if (c->h_stage_cap[t] < n) {
+    cudaFreeHost(c->h_stage[t]);
+    c->h_stage[t] = nullptr;
+    c->h_stage_cap[t] = 0;
+    const size_t cap_n = std::max<size_t>(n + n / 4, 1 << 18);
+    if (cudaMallocHost(&c->h_stage[t], cap_n) != cudaSuccess) return false;
+    c->h_stage_cap[t] = cap_n;
+  }
+  std::memcpy(c->h_stage[t], p, n);
+  return cudaMemcpyAsync(d, c->h_stage[t], n, cudaMemcpyHostToDevice, c->stream) == cudaSuccess &&
+         cudaEventRecord(c->ev_stage[t], c->stream) == cudaSuccess;
+}
+
+// An entry of `cache` for a new set of n bytes; *rc says why there is none.  Refused while the stream is
+// being captured: a graph must neither allocate nor hold the staging buffer.
+SetCache::Entry* new_entry(hydro_ctx* c, SetCache& cache, size_t n, int* rc) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  *rc = HYDRO_ERR_CUDA;
+  if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return nullptr;
+  *rc = HYDRO_ERR_NOMEM;
+  return cache.replace(std::max<size_t>(n, 256));
+}
+
+// The entry holding `bytes` on the device, uploaded unless one of the last sets has them.
+SetCache::Entry* upload_set(hydro_ctx* c, SetCache& cache, std::vector<char>&& bytes) {
+  if (SetCache::Entry* e = cache.find(bytes)) return e;
+  int rc;
+  SetCache::Entry* e = new_entry(c, cache, bytes.size(), &rc);
+  if (!e || !upload(c, e->d, bytes.data(), bytes.size())) return nullptr;
+  cache.done(e, std::move(bytes));
+  return e;
 }
 
 // Patch-shape class of a patch for the per-class tile choice (include/hydro.h): 0 an x or y edge
@@ -321,107 +383,87 @@ void default_tuning(const hydro_ctx* c, const hydro_patch* in, int n, int* tile,
   }
 }
 
+// Counts and settings of a batch entry (SetCache::Entry::n).
+enum { B_NTILES, B_TILE, B_ZCHUNK, B_PER_CLASS, B_CLS_OFF, B_CLS_NTILES = B_CLS_OFF + HYDRO_NUM_PATCH_CLASSES };
+// Its parts: descriptors, tile records, prefix-sum counts, patch indices by class.
+enum { B_PATCHES, B_TILES, B_COUNTS, B_INDEX };
+
 // Upload the descriptors of (in, out) and build the tile work-list for the current tuning,
-// unless the cached set and tuning are unchanged.  With a tile shape per patch-shape class the
+// unless one of the last sets and its tuning are the same.  With a tile shape per patch-shape class the
 // work-list holds one segment per class, each built with its class's tile shape and z chunk.
-int prepare_batch(hydro_ctx* c, const hydro_patch* in, const hydro_patch* out, int n) {
-  const bool set_same = same_set(c->key_in, in, n) && same_set(c->key_out, out, n);
+int prepare_batch(hydro_ctx* c, const hydro_patch* in, const hydro_patch* out, int n, SetCache::Entry** entry) {
+  constexpr int NC = HYDRO_NUM_PATCH_CLASSES;
   // the PPM kernel's tiles are 16 x 16 (tile shape 0)
   int tile = ppm(c) ? 0 : c->tile_id, zchunk = c->zchunk;
   const bool pc = per_class(c);
-  int cls_key[2 * HYDRO_NUM_PATCH_CLASSES];
-  for (int k = 0; k < HYDRO_NUM_PATCH_CLASSES; ++k) {
-    cls_key[2 * k] = class_tile(c, k);
-    cls_key[2 * k + 1] = class_zc(c, k);
+  std::vector<char> key(2 * (size_t)n * sizeof(hydro_patch));
+  std::memcpy(key.data(), in, (size_t)n * sizeof(hydro_patch));
+  std::memcpy(key.data() + (size_t)n * sizeof(hydro_patch), out, (size_t)n * sizeof(hydro_patch));
+  int setting[2 * NC + 2] = {};
+  for (int k = 0; k < NC && pc; ++k) {
+    setting[2 * k] = 1 + class_tile(c, k);
+    setting[2 * k + 1] = class_zc(c, k);
   }
-  if (set_same && pc == c->wl_per_class &&
-      (pc ? std::memcmp(cls_key, c->wl_cls, sizeof(cls_key)) == 0
-          : c->wl_tuned == c->tuned && (!c->tuned || (c->wl_tile == tile && c->wl_zchunk == zchunk))))
-    return HYDRO_OK;
-  if (!c->tuned) default_tuning(c, in, n, &tile, &zchunk);
-  const int tx = hydro::kTileX[tile], ty = hydro::kTileY[tile];
-  if (!set_same) {
-    size_t old = c->patches_cap;
-    int rc = ensure_device(&c->d_patches, &c->patches_cap, (size_t)n);
-    if (rc) return rc;
-    if (c->patches_cap != old || !c->h_patches) {
-      if (c->h_patches) cudaFreeHost(c->h_patches);
-      if (cudaMallocHost(&c->h_patches, c->patches_cap * sizeof(HostPatchIO)) != cudaSuccess) return HYDRO_ERR_NOMEM;
-    }
-    // the staging buffer may still be read by an earlier copy on the stream
-    if (cudaStreamSynchronize(c->stream) != cudaSuccess) return HYDRO_ERR_CUDA;
-    for (int i = 0; i < n; ++i) c->h_patches[i] = make_io(in[i], out[i]);
-    if (cudaMemcpyAsync(c->d_patches, c->h_patches, n * sizeof(HostPatchIO), cudaMemcpyHostToDevice, c->stream) !=
-        cudaSuccess)
-      return HYDRO_ERR_CUDA;
-    c->key_in.assign(in, in + n);
-    c->key_out.assign(out, out + n);
+  if (!pc && c->tuned) {
+    setting[2 * NC] = 1 + tile;
+    setting[2 * NC + 1] = zchunk;
   }
-  if (pc) {
-    // patches by class (host), the index list uploaded, then one work-list segment per class
-    std::vector<int> idx;
-    idx.reserve(n);
-    int cnt[HYDRO_NUM_PATCH_CLASSES] = {}, first[HYDRO_NUM_PATCH_CLASSES] = {};
-    size_t tiles[HYDRO_NUM_PATCH_CLASSES] = {};
-    for (int k = 0; k < HYDRO_NUM_PATCH_CLASSES; ++k) {
-      first[k] = (int)idx.size();
-      const int t = class_tile(c, k), z = class_zc(c, k), kx = hydro::kTileX[t], ky = hydro::kTileY[t];
-      for (int i = 0; i < n; ++i)
-        if (patch_class(in[i]) == k) {
-          idx.push_back(i);
-          tiles[k] += (size_t)((in[i].nx + kx - 1) / kx) * ((in[i].ny + ky - 1) / ky) * ((in[i].nz + z - 1) / z);
-        }
-      cnt[k] = (int)idx.size() - first[k];
+  append(key, setting, 2 * NC + 2);
+  if ((*entry = c->batch.find(key))) return HYDRO_OK;
+  if (!pc && !c->tuned) default_tuning(c, in, n, &tile, &zchunk);
+  // patches by class (all in class 0 without a tile shape per class) and tiles per class: the counts on
+  // the host size the buffer, the device builds the list itself
+  int t[NC], z[NC], cnt[NC] = {}, first[NC] = {};
+  size_t tiles[NC] = {}, total = 0;
+  std::vector<int> idx;
+  for (int k = 0; k < (pc ? NC : 1); ++k) {
+    t[k] = pc ? class_tile(c, k) : tile;
+    z[k] = pc ? class_zc(c, k) : zchunk;
+    const int kx = hydro::kTileX[t[k]], ky = hydro::kTileY[t[k]];
+    first[k] = (int)idx.size();
+    for (int i = 0; i < n; ++i) {
+      if (pc && patch_class(in[i]) != k) continue;
+      if (pc) idx.push_back(i);
+      ++cnt[k];
+      tiles[k] += (size_t)((in[i].nx + kx - 1) / kx) * ((in[i].ny + ky - 1) / ky) * ((in[i].nz + z[k] - 1) / z[k]);
     }
-    size_t total = 0;
-    for (int k = 0; k < HYDRO_NUM_PATCH_CLASSES; ++k) total += tiles[k];
-    if (total > 0x7fffffff) return HYDRO_ERR_ARG;
-    int rc = ensure_device(&c->d_counts, &c->counts_cap, (size_t)n + HYDRO_NUM_PATCH_CLASSES);
-    if (rc) return rc;
-    rc = ensure_device(&c->d_tiles, &c->tiles_cap, std::max<size_t>(total, 1));
-    if (rc) return rc;
-    rc = ensure_device(&c->d_cls_idx, &c->cls_idx_cap, (size_t)n);
-    if (rc) return rc;
-    if (cudaStreamSynchronize(c->stream) != cudaSuccess ||
-        cudaMemcpy(c->d_cls_idx, idx.data(), n * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess)
-      return HYDRO_ERR_CUDA;
-    size_t off = 0;
-    for (int k = 0; k < HYDRO_NUM_PATCH_CLASSES; ++k) {
-      c->cls_off[k] = (int)off;
-      c->cls_ntiles[k] = (int)tiles[k];
-      if (cnt[k]) {
-        const int t = class_tile(c, k);
-        if (hydro::build_worklist(c->d_patches, cnt[k], hydro::kTileX[t], hydro::kTileY[t], class_zc(c, k),
-                                  c->d_counts + first[k] + k, c->d_tiles + off, c->stream,
-                                  c->d_cls_idx + first[k]) != cudaSuccess)
-          return HYDRO_ERR_CUDA;
-        c->launches += 3;
-      }
-      off += tiles[k];
-    }
-    c->ntiles = (int)total;
-    c->wl_per_class = true;
-    std::memcpy(c->wl_cls, cls_key, sizeof(cls_key));
-    c->wl_tile = -1;
-    return HYDRO_OK;
+    total += tiles[k];
   }
-  // tile count on the host sizes the buffer; the device builds the list itself
-  size_t total = 0;
-  for (int i = 0; i < n; ++i)
-    total += (size_t)((in[i].nx + tx - 1) / tx) * ((in[i].ny + ty - 1) / ty) * ((in[i].nz + zchunk - 1) / zchunk);
   if (total > 0x7fffffff) return HYDRO_ERR_ARG;
-  int rc = ensure_device(&c->d_counts, &c->counts_cap, (size_t)n + 1);
-  if (rc) return rc;
-  rc = ensure_device(&c->d_tiles, &c->tiles_cap, total);
-  if (rc) return rc;
-  if (hydro::build_worklist(c->d_patches, n, tx, ty, zchunk, c->d_counts, c->d_tiles, c->stream) != cudaSuccess)
-    return HYDRO_ERR_CUDA;
-  c->launches += 3;
-  c->ntiles = (int)total;
-  c->wl_tile = tile;
-  c->wl_zchunk = zchunk;
-  c->wl_tuned = c->tuned;
-  c->wl_per_class = false;
+  std::vector<HostPatchIO> io((size_t)n);
+  for (int i = 0; i < n; ++i) io[i] = make_io(in[i], out[i]);
+  std::vector<char> bytes;
+  size_t off[4] = {};
+  off[B_PATCHES] = append(bytes, io.data(), io.size());
+  off[B_INDEX] = append(bytes, idx.data(), idx.size());
+  auto align = [](size_t x) { return (x + 255) / 256 * 256; };
+  off[B_TILES] = align(bytes.size());
+  off[B_COUNTS] = align(off[B_TILES] + total * sizeof(HostTileRec));
+  int rc;
+  SetCache::Entry* e = new_entry(c, c->batch, off[B_COUNTS] + ((size_t)n + NC) * sizeof(int), &rc);
+  if (!e) return rc;
+  if (!upload(c, e->d, bytes.data(), bytes.size())) return HYDRO_ERR_CUDA;
+  std::memcpy(e->off, off, sizeof(off));
+  e->n[B_NTILES] = (int)total;
+  e->n[B_TILE] = tile;
+  e->n[B_ZCHUNK] = zchunk;
+  e->n[B_PER_CLASS] = pc;
+  size_t done = 0;
+  for (int k = 0; k < (pc ? NC : 1); ++k) {
+    e->n[B_CLS_OFF + k] = (int)done;
+    e->n[B_CLS_NTILES + k] = (int)tiles[k];
+    if (cnt[k]) {
+      if (hydro::build_worklist(reinterpret_cast<HostPatchIO*>(e->d + off[B_PATCHES]), cnt[k], hydro::kTileX[t[k]],
+                                hydro::kTileY[t[k]], z[k], reinterpret_cast<int*>(e->d + off[B_COUNTS]) + first[k] + k,
+                                reinterpret_cast<HostTileRec*>(e->d + off[B_TILES]) + done, c->stream,
+                                pc ? reinterpret_cast<int*>(e->d + off[B_INDEX]) + first[k] : nullptr) != cudaSuccess)
+        return HYDRO_ERR_CUDA;
+      c->launches += 3;
+    }
+    done += tiles[k];
+  }
+  c->batch.done(e, std::move(key));
+  *entry = e;
   return HYDRO_OK;
 }
 
@@ -452,34 +494,6 @@ int step_one_uniform(hydro_ctx* c, const hydro_patch& in, const hydro_patch& out
   return cuda_status(e);
 }
 
-// Device copy of host descriptor bytes for a call kind: the buffer of the last call of that kind
-// when the bytes are unchanged, else a fresh upload (after the stream has drained: earlier
-// kernels may still read the buffer).  Returns the device address or nullptr.
-char* upload_aux(hydro_ctx* c, int kind, const std::vector<char>& bytes) {
-  if (c->d_aux[kind] && bytes == c->aux_last[kind]) return c->d_aux[kind];
-  if (cudaStreamSynchronize(c->stream) != cudaSuccess) return nullptr;
-  if (c->aux_cap[kind] < bytes.size() || !c->d_aux[kind]) {
-    cudaFree(c->d_aux[kind]);
-    c->d_aux[kind] = nullptr;
-    c->aux_cap[kind] = 0;
-    c->aux_last[kind].clear();
-    const size_t n = std::max<size_t>(bytes.size(), 256);
-    if (cudaMalloc(&c->d_aux[kind], n) != cudaSuccess) return nullptr;
-    c->aux_cap[kind] = n;
-  }
-  if (!bytes.empty() && cudaMemcpy(c->d_aux[kind], bytes.data(), bytes.size(), cudaMemcpyHostToDevice) != cudaSuccess)
-    return nullptr;
-  c->aux_last[kind] = bytes;
-  return c->d_aux[kind];
-}
-template <class T>
-size_t append(std::vector<char>& bytes, const T* p, size_t n) {
-  const size_t off = (bytes.size() + 255) / 256 * 256;
-  bytes.resize(off + n * sizeof(T));
-  if (n) std::memcpy(bytes.data() + off, p, n * sizeof(T));
-  return off;
-}
-
 int box_fluxes(hydro_ctx* c, int kind, const std::vector<hydro::HostBoxFluxes>& boxes, const double* dt_dev,
                int accumulate) {
   std::vector<int2> blocks;
@@ -493,8 +507,9 @@ int box_fluxes(hydro_ctx* c, int kind, const std::vector<hydro::HostBoxFluxes>& 
   std::vector<char> bytes;
   const size_t ob = append(bytes, boxes.data(), boxes.size());
   const size_t ok = append(bytes, blocks.data(), blocks.size());
-  char* d = upload_aux(c, kind, bytes);
-  if (!d) return HYDRO_ERR_CUDA;
+  const SetCache::Entry* e = upload_set(c, c->aux[kind], std::move(bytes));
+  if (!e) return HYDRO_ERR_CUDA;
+  char* d = e->d;
   c->launches += 1;
   return cuda_status(c->ops->box_fluxes(reinterpret_cast<const hydro::HostBoxFluxes*>(d + ob),
                                         reinterpret_cast<const int2*>(d + ok), (int)blocks.size(), c->prm, dt_dev,
@@ -560,12 +575,7 @@ int hydro_finalize(hydro_ctx* c) {
   if (c->capture) cudaStreamDestroy(c->capture);
   cudaFree(c->d_err);
   cudaFree(c->d_counter);
-  cudaFree(c->d_cls_idx);
   cudaFree(c->d_cls_dt);
-  cudaFree(c->d_patches);
-  cudaFree(c->d_counts);
-  cudaFree(c->d_tiles);
-  cudaFree(c->d_cfl);
   cudaFree(c->d_adj);
   if (c->s_h2d) cudaStreamSynchronize(c->s_h2d);
   if (c->s_d2h) cudaStreamSynchronize(c->s_d2h);
@@ -574,11 +584,11 @@ int hydro_finalize(hydro_ctx* c) {
   cudaFree(c->d_stage_io);
   cudaFree(c->d_stage_tiles);
   cudaFree(c->d_stage_counters);
-  cudaFree(c->d_ghost);
-  cudaFree(c->d_ghost_blocks);
-  cudaFree(c->d_xchg);
-  cudaFree(c->d_tasks);
-  for (int k = 0; k < hydro_ctx::kAux; ++k) cudaFree(c->d_aux[k]);
+  c->batch.free_all();
+  c->cfl_sets.free_all();
+  c->ghost_sets.free_all();
+  c->xchg_sets.free_all();
+  for (SetCache& s : c->aux) s.free_all();
   cudaFree(c->d_octs_scratch);
   cudaFree(c->d_mhd);
   for (cudaEvent_t e : c->ev_copied) cudaEventDestroy(e);
@@ -590,8 +600,10 @@ int hydro_finalize(hydro_ctx* c) {
   if (c->s_d2h) cudaStreamDestroy(c->s_d2h);
   if (c->s_cmp2) cudaStreamDestroy(c->s_cmp2);
   if (c->ev_ready) cudaEventDestroy(c->ev_ready);
-  if (c->h_patches) cudaFreeHost(c->h_patches);
-  if (c->h_cfl) cudaFreeHost(c->h_cfl);
+  for (int t = 0; t < 2; ++t) {
+    cudaFreeHost(c->h_stage[t]);
+    if (c->ev_stage[t]) cudaEventDestroy(c->ev_stage[t]);
+  }
   delete c;
   return HYDRO_OK;
 }
@@ -606,24 +618,19 @@ int hydro_cfl_dt(hydro_ctx* c, const hydro_patch* p, int npatch, double* dt_dev)
     c->launches += 1;
     return cuda_status(c->ops->cfl(nullptr, make_io(p[0], p[0]), 1, c->prm, dt_dev, c->d_err, c->stream));
   }
-  if (!same_set(c->cfl_key, p, npatch)) {
-    size_t old = c->cfl_cap;
-    rc = ensure_device(&c->d_cfl, &c->cfl_cap, (size_t)npatch);
-    if (rc) return rc;
-    if (c->cfl_cap != old || !c->h_cfl) {
-      if (c->h_cfl) cudaFreeHost(c->h_cfl);
-      if (cudaMallocHost(&c->h_cfl, c->cfl_cap * sizeof(HostPatchIO)) != cudaSuccess) return HYDRO_ERR_NOMEM;
-    }
-    if (cudaStreamSynchronize(c->stream) != cudaSuccess) return HYDRO_ERR_CUDA;
-    for (int i = 0; i < npatch; ++i) c->h_cfl[i] = make_io(p[i], p[i]);
-    if (cudaMemcpyAsync(c->d_cfl, c->h_cfl, npatch * sizeof(HostPatchIO), cudaMemcpyHostToDevice, c->stream) !=
-        cudaSuccess)
-      return HYDRO_ERR_CUDA;
-    c->cfl_key.assign(p, p + npatch);
+  std::vector<char> key;
+  append(key, p, (size_t)npatch);
+  SetCache::Entry* e = c->cfl_sets.find(key);
+  if (!e) {
+    std::vector<HostPatchIO> io((size_t)npatch);
+    for (int i = 0; i < npatch; ++i) io[i] = make_io(p[i], p[i]);
+    if (!(e = new_entry(c, c->cfl_sets, io.size() * sizeof(io[0]), &rc))) return rc;
+    if (!upload(c, e->d, io.data(), io.size() * sizeof(io[0]))) return HYDRO_ERR_CUDA;
+    c->cfl_sets.done(e, std::move(key));
   }
   HostPatchIO big = make_io(p[0], p[0]);
   c->launches += 1;
-  return cuda_status(c->ops->cfl(c->d_cfl, big, npatch, c->prm, dt_dev, c->d_err, c->stream));
+  return cuda_status(c->ops->cfl(reinterpret_cast<const HostPatchIO*>(e->d), big, npatch, c->prm, dt_dev, c->d_err, c->stream));
 }
 
 int hydro_step(hydro_ctx* c, const hydro_patch* in, const hydro_patch* out, int npatch, const double* dt_dev,
@@ -637,37 +644,41 @@ int hydro_step(hydro_ctx* c, const hydro_patch* in, const hydro_patch* out, int 
   if (npatch == 1 && in[0].ng == 0) return step_one_uniform(c, in[0], out[0], dt_dev, dt_next_dev, c->stream);
   for (int i = 0; i < npatch; ++i)  // ghost layers the reconstruction's stencil needs
     if (in[i].ng != (ppm(c) ? 3 : 2)) return HYDRO_ERR_ARG;
-  int rc = prepare_batch(c, in, out, npatch);
+  SetCache::Entry* e = nullptr;
+  int rc = prepare_batch(c, in, out, npatch, &e);
   if (rc) return rc;
+  const HostPatchIO* d_patches = reinterpret_cast<const HostPatchIO*>(e->d + e->off[B_PATCHES]);
+  const HostTileRec* d_tiles = reinterpret_cast<const HostTileRec*>(e->d + e->off[B_TILES]);
+  const int ntiles = e->n[B_NTILES], tile = e->n[B_TILE], zchunk = e->n[B_ZCHUNK];
   if (cudaMemsetAsync(c->d_counter, 0, (1 + HYDRO_NUM_PATCH_CLASSES) * sizeof(int), c->stream) != cudaSuccess)
     return HYDRO_ERR_CUDA;
   if (dt_next_dev) {
     rc = reset_slots(c, dt_next_dev, npatch, c->stream);
     if (rc) return rc;
   }
-  if (c->wl_per_class) {
+  if (e->n[B_PER_CLASS]) {
     // one persistent launch per class, each over its own work-list segment and counter
     for (int k = 0; k < HYDRO_NUM_PATCH_CLASSES; ++k) {
-      if (!c->cls_ntiles[k]) continue;
+      const int nt = e->n[B_CLS_NTILES + k];
+      if (!nt) continue;
       const int t = class_tile(c, k);
       const int per_sm = c->ops->batched_blocks_per_sm(t, c->cfg.limiter);
-      const int grid = std::max(1, std::min(c->cls_ntiles[k], c->sm_count * per_sm));
+      const int grid = std::max(1, std::min(nt, c->sm_count * per_sm));
       c->launches += 1;
-      cudaError_t e = c->ops->step_batched(t, c->d_patches, c->d_tiles + c->cls_off[k], c->cls_ntiles[k],
-                                           c->d_counter + 1 + k, c->prm, dt_dev, dt_next_dev, class_zc(c, k),
-                                           c->d_err, grid, c->stream);
-      if (e != cudaSuccess) return HYDRO_ERR_CUDA;
+      cudaError_t err = c->ops->step_batched(t, d_patches, d_tiles + e->n[B_CLS_OFF + k], nt, c->d_counter + 1 + k, c->prm,
+                                             dt_dev, dt_next_dev, class_zc(c, k), c->d_err, grid, c->stream);
+      if (err != cudaSuccess) return HYDRO_ERR_CUDA;
     }
     return HYDRO_OK;
   }
   c->launches += 1;
   if (ppm(c))
-    return cuda_status(c->ops->step_ppm_batched(c->d_patches, c->d_tiles, c->ntiles, c->d_counter, c->prm, dt_dev,
-                                                dt_next_dev, c->wl_zchunk, c->d_err, c->sm_count, c->stream));
-  const int per_sm = c->ops->batched_blocks_per_sm(c->wl_tile, c->cfg.limiter);
-  int grid = std::max(1, std::min(c->ntiles, c->sm_count * per_sm));
-  return cuda_status(c->ops->step_batched(c->wl_tile, c->d_patches, c->d_tiles, c->ntiles, c->d_counter, c->prm,
-                                          dt_dev, dt_next_dev, c->wl_zchunk, c->d_err, grid, c->stream));
+    return cuda_status(c->ops->step_ppm_batched(d_patches, d_tiles, ntiles, c->d_counter, c->prm, dt_dev, dt_next_dev,
+                                                zchunk, c->d_err, c->sm_count, c->stream));
+  const int per_sm = c->ops->batched_blocks_per_sm(tile, c->cfg.limiter);
+  const int grid = std::max(1, std::min(ntiles, c->sm_count * per_sm));
+  return cuda_status(c->ops->step_batched(tile, d_patches, d_tiles, ntiles, c->d_counter, c->prm, dt_dev, dt_next_dev,
+                                          zchunk, c->d_err, grid, c->stream));
 }
 
 // Host-buffer step of one periodic box: the state crosses the host link in z slabs on two copy
@@ -892,30 +903,29 @@ static int fill_ghosts_impl(hydro_ctx* c, const hydro_patch* coarse, const hydro
     }
     if (cells > 0x7fffffff) return HYDRO_ERR_ARG;
   }
-  const bool same = c->ghost_key.size() == set.size() &&
-                    std::memcmp(c->ghost_key.data(), set.data(), set.size() * sizeof(set[0])) == 0;
-  if (!same) {
+  std::vector<char> key;
+  append(key, set.data(), set.size());
+  SetCache::Entry* e = c->ghost_sets.find(key);
+  if (!e) {
     std::vector<int2> blocks;
     for (int i = 0; i < npatch; ++i)
       for (int first = 0; first < set[i].cm[0] * set[i].cm[1] * set[i].cm[2]; first += 256)
         blocks.push_back(make_int2(i, first));
     if (blocks.size() > 0x7fffffff) return HYDRO_ERR_ARG;
-    int rc = ensure_device(&c->d_ghost, &c->ghost_cap, (size_t)npatch);
-    if (rc) return rc;
-    rc = ensure_device(&c->d_ghost_blocks, &c->ghost_blocks_cap, blocks.size());
-    if (rc) return rc;
-    // the descriptors may still be read by an earlier fill on the stream
-    if (cudaStreamSynchronize(c->stream) != cudaSuccess) return HYDRO_ERR_CUDA;
-    if (cudaMemcpy(c->d_ghost, set.data(), set.size() * sizeof(set[0]), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(c->d_ghost_blocks, blocks.data(), blocks.size() * sizeof(int2), cudaMemcpyHostToDevice) != cudaSuccess)
-      return HYDRO_ERR_CUDA;
-    c->ghost_key.swap(set);
-    c->ghost_nblocks = (int)blocks.size();
+    std::vector<char> bytes = key;
+    const size_t off = append(bytes, blocks.data(), blocks.size());
+    int rc;
+    if (!(e = new_entry(c, c->ghost_sets, bytes.size(), &rc))) return rc;
+    if (!upload(c, e->d, bytes.data(), bytes.size())) return HYDRO_ERR_CUDA;
+    e->off[1] = off;
+    e->n[0] = (int)blocks.size();
+    c->ghost_sets.done(e, std::move(key));
   }
   c->launches += 1;
   const HostPatchIO old = coarse_old ? make_io(*coarse_old, *coarse_old) : make_io(C, C);
-  return cuda_status(hydro::launch_fill_ghosts(elem_size(c), c->d_ghost, c->d_ghost_blocks, c->ghost_nblocks,
-                                               make_io(C, C), coarse_old ? &old : nullptr, theta, c->stream));
+  return cuda_status(hydro::launch_fill_ghosts(elem_size(c), reinterpret_cast<const hydro::HostGhostPatch*>(e->d),
+                                               reinterpret_cast<const int2*>(e->d + e->off[1]), e->n[0], make_io(C, C),
+                                               coarse_old ? &old : nullptr, theta, c->stream));
 }
 
 int hydro_fill_ghosts(hydro_ctx* c, const hydro_patch* coarse, const hydro_patch* fine, const int* fine_origins,
@@ -974,27 +984,27 @@ static std::vector<hydro::HostCopyTask> exchange_tasks(const std::vector<hydro::
           for (int q : bins[((size_t)z * nb[1] + y) * nb[0] + x])
             if (seen[q] != a) { seen[q] = a; cand.push_back(q); }
     for (int b : cand) {
-      for (int kz = -2; kz <= 2; ++kz)
-        for (int ky = -2; ky <= 2; ++ky)
-          for (int kx = -2; kx <= 2; ++kx) {
-            const int k[3] = {kx, ky, kz};
-            int lo[3], hi[3];
-            bool empty = false, own = (b == a);
-            for (int d = 0; d < 3; ++d) {
-              const int s = org(b, d) + k[d] * per[d];
-              lo[d] = std::max(glo[d], s);
-              hi[d] = std::min(ghi[d], s + dim(b, d));
-              if (lo[d] >= hi[d]) empty = true;
-              if (k[d] != 0) own = false;
-            }
-            if (empty || own) continue;
+      // per axis, the images (shift k periods) of b's interior that meet a's ghosted box, at most a
+      // few of the five: their product instead of 125 tests per candidate
+      struct Image { int k, lo, hi, s; } im[3][5];
+      int ni[3] = {0, 0, 0};
+      for (int d = 0; d < 3; ++d)
+        for (int k = -2; k <= 2; ++k) {
+          const int s = org(b, d) + k * per[d], lo = std::max(glo[d], s), hi = std::min(ghi[d], s + dim(b, d));
+          if (lo < hi) im[d][ni[d]++] = {k, lo, hi, s};
+        }
+      for (int z = 0; z < ni[2]; ++z)
+        for (int y = 0; y < ni[1]; ++y)
+          for (int x = 0; x < ni[0]; ++x) {
+            const Image m[3] = {im[0][x], im[1][y], im[2][z]};
+            if (b == a && m[0].k == 0 && m[1].k == 0 && m[2].k == 0) continue;  // its own interior
             hydro::HostCopyTask t;
             t.dst = a;
             t.src = b;
             for (int d = 0; d < 3; ++d) {
-              t.dlo[d] = lo[d] - glo[d];
-              t.slo[d] = lo[d] - (org(b, d) + k[d] * per[d]) + 2;
-              t.n[d] = hi[d] - lo[d];
+              t.dlo[d] = m[d].lo - glo[d];
+              t.slo[d] = m[d].lo - m[d].s + 2;
+              t.n[d] = m[d].hi - m[d].lo;
             }
             tasks.push_back(t);
           }
@@ -1080,8 +1090,9 @@ int hydro_reflux(hydro_ctx* c, const hydro_patch* coarse, const int* box_origins
     ot[t] = append(bytes, tables[t].data(), tables[t].size());
     nb[t] = (int)tables[t].size();
   }
-  char* d = upload_aux(c, 2, bytes);
-  if (!d) return HYDRO_ERR_CUDA;
+  const SetCache::Entry* e = upload_set(c, c->aux[2], std::move(bytes));
+  if (!e) return HYDRO_ERR_CUDA;
+  char* d = e->d;
   const int2* dt[6];
   for (int t = 0; t < 6; ++t) dt[t] = reinterpret_cast<const int2*>(d + ot[t]);
   c->launches += 6;
@@ -1113,8 +1124,9 @@ int hydro_average_down(hydro_ctx* c, const hydro_patch* coarse, const hydro_patc
   std::vector<char> bytes;
   const size_t op = append(bytes, set.data(), set.size());
   const size_t obk = append(bytes, blocks.data(), blocks.size());
-  char* d = upload_aux(c, 3, bytes);
-  if (!d) return HYDRO_ERR_CUDA;
+  const SetCache::Entry* e = upload_set(c, c->aux[3], std::move(bytes));
+  if (!e) return HYDRO_ERR_CUDA;
+  char* d = e->d;
   c->launches += 1;
   return cuda_status(hydro::launch_average_down(elem_size(c), reinterpret_cast<const hydro::HostGhostPatch*>(d + op),
                                                 reinterpret_cast<const int2*>(d + obk), (int)blocks.size(),
@@ -1137,28 +1149,28 @@ int hydro_exchange_ghosts(hydro_ctx* c, const hydro_patch* fine, const int* orig
     for (int d = 0; d < 3; ++d) g.clo[d] = g.cm[d] = 0;
     g.sy = F.sy; g.sz = F.sz;
   }
-  const bool same = c->xchg_key.size() == set.size() &&
-                    std::memcmp(c->xchg_key.data(), set.data(), set.size() * sizeof(set[0])) == 0 &&
-                    std::memcmp(c->xchg_period, period, sizeof(c->xchg_period)) == 0;
-  if (!same) {
+  std::vector<char> key;
+  append(key, set.data(), set.size());
+  append(key, period, 3);
+  SetCache::Entry* e = c->xchg_sets.find(key);
+  if (!e) {
     const std::vector<hydro::HostCopyTask> tasks = exchange_tasks(set, period);
     if (tasks.size() > 0x7fffffff) return HYDRO_ERR_ARG;
-    int rc = ensure_device(&c->d_xchg, &c->xchg_cap, (size_t)npatch);
-    if (rc) return rc;
-    rc = ensure_device(&c->d_tasks, &c->tasks_cap, std::max<size_t>(1, tasks.size()));
-    if (rc) return rc;
-    if (cudaStreamSynchronize(c->stream) != cudaSuccess) return HYDRO_ERR_CUDA;
-    if (cudaMemcpy(c->d_xchg, set.data(), set.size() * sizeof(set[0]), cudaMemcpyHostToDevice) != cudaSuccess ||
-        (!tasks.empty() && cudaMemcpy(c->d_tasks, tasks.data(), tasks.size() * sizeof(tasks[0]),
-                                      cudaMemcpyHostToDevice) != cudaSuccess))
-      return HYDRO_ERR_CUDA;
-    c->xchg_key.swap(set);
-    std::memcpy(c->xchg_period, period, sizeof(c->xchg_period));
-    c->ntasks = (int)tasks.size();
+    std::vector<char> bytes;
+    append(bytes, set.data(), set.size());
+    const size_t off = append(bytes, tasks.data(), tasks.size());
+    int rc;
+    if (!(e = new_entry(c, c->xchg_sets, bytes.size(), &rc))) return rc;
+    if (!upload(c, e->d, bytes.data(), bytes.size())) return HYDRO_ERR_CUDA;
+    e->off[1] = off;
+    e->n[0] = (int)tasks.size();
+    c->xchg_sets.done(e, std::move(key));
   }
-  if (c->ntasks == 0) return HYDRO_OK;
+  if (e->n[0] == 0) return HYDRO_OK;
   c->launches += 1;
-  return cuda_status(hydro::launch_copy_boxes(elem_size(c), c->d_xchg, c->d_tasks, c->ntasks, c->stream));
+  return cuda_status(hydro::launch_copy_boxes(elem_size(c), reinterpret_cast<const hydro::HostGhostPatch*>(e->d),
+                                              reinterpret_cast<const hydro::HostCopyTask*>(e->d + e->off[1]), e->n[0],
+                                              c->stream));
 }
 
 int hydro_step_octs_level(hydro_ctx* c, const hydro_patch* level, const int* origins_dev, long long ngroups,
@@ -1327,8 +1339,9 @@ static int mhd_patch_tables(hydro_ctx* c, int kind, const hydro_mhd_patch* in, c
   std::vector<char> bytes;
   const size_t op = append(bytes, set.data(), set.size());
   const size_t ob = tiles ? append(bytes, recs.data(), recs.size()) : append(bytes, blocks.data(), blocks.size());
-  char* d = upload_aux(c, kind, bytes);
-  if (!d) return HYDRO_ERR_CUDA;
+  const SetCache::Entry* e = upload_set(c, c->aux[kind], std::move(bytes));
+  if (!e) return HYDRO_ERR_CUDA;
+  char* d = e->d;
   *d_patches = reinterpret_cast<const hydro::HostMhdPatch*>(d + op);
   *d_blocks = d + ob;
   *nblocks = (int)(tiles ? recs.size() : blocks.size());
