@@ -133,7 +133,7 @@ __device__ __forceinline__ df quot_(const df& x, const df& y) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(y.h));
   const float q = x.h * r0, p = y.h * q;
   const float r = ((x.h - p) - fmaf(y.h, q, -p)) + fmaf(-y.l, q, x.l);
-  return df(q, r * r0);
+  return df(q, r * fmaf(fmaf(-y.h, r0, 1.f), r0, r0));
 }
 __device__ __forceinline__ df rootu_(const df& x) {
   float s0, i0;  // independent approximations: the root's own error is squared, 1/root's only scales it

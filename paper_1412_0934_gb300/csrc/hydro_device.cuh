@@ -48,8 +48,14 @@ template <class R>
 __device__ __forceinline__ R rabs(R x) {
   return x < R(0) ? -x : x;
 }
-// Float policies use the SFU approximations (relative error a few ulp of float); double uses
-// correctly rounded IEEE operations.
+// Float policies use the SFU approximations (relative error a few ulp of float).  Double starts from the
+// SFU's 20-bit approximations and takes one third-order Newton (Householder) step, 3 to 6 operations on
+// the FP64 pipe, which bounds the double kernels, where the IEEE sequences take about ten and a branch:
+//   1/y:     e = 1 - y r0,        r = r0 (1 + e + e^2)             error below 0.5 ulp + 2^-58
+//   n/d:     q = n r, q + r (n - q d)                              below 0.6 ulp
+//   sqrt(x): s0 = x y0, e = 1 - s0 y0,  s = s0 (1 + e/2 + 3 e^2/8)  below 0.8 ulp
+// for operands and results of magnitude 2^-1020 to 2^1020 (the approximations flush beyond); a zero
+// operand's root is zero.
 __device__ __forceinline__ float rcp_(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -61,9 +67,23 @@ __device__ __forceinline__ float rsqrt_(float x) {
   return r;
 }
 __device__ __forceinline__ float div_(float a, float b) { return a * rcp_(b); }
-__device__ __forceinline__ double rsqrt_(double x) { return sqrt(x); }
-__device__ __forceinline__ double rcp_(double x) { return 1.0 / x; }
-__device__ __forceinline__ double div_(double a, double b) { return a / b; }
+__device__ __forceinline__ double rcp_(double y) {
+  double r0;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(y));
+  const double e = fma(-y, r0, 1.0);
+  return fma(r0, fma(e, e, e), r0);
+}
+__device__ __forceinline__ double div_(double n, double d) {
+  const double r = rcp_(d), q = n * r;
+  return fma(r, fma(-q, d, n), q);
+}
+__device__ __forceinline__ double rsqrt_(double x) {  // the square root (named like the float one)
+  double y0;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
+  const double s0 = x * y0, e = fma(-s0, y0, 1.0);
+  const double s = fma(s0, e * fma(e, 0.375, 0.5), s0);
+  return __double2hiint(x) >= 0x00100000 ? s : 0.0;  // zero (and what .ftz reads as zero) has root zero
+}
 
 // Constant i of the parameters in arithmetic type R.
 template <class R>
@@ -171,10 +191,24 @@ __device__ __forceinline__ df minmod(const df& a, const df& b) {
   return df(zero ? 0.f : h, zero ? 0.f : l);
 }
 
+// Float: the smaller magnitude with the product of the signs (one min.xorsign.abs) is negative exactly
+// where the signs differ, so max with 0 and the sign of a finish MinMod: three operations on the ALU
+// pipe, which bounds the float kernels together with the issue slots, in place of five.
+__device__ __forceinline__ float min_xorsign(float a, float b) {
+  float t;
+  asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(t) : "f"(a), "f"(b));
+  return t;
+}
+__device__ __forceinline__ float minmod(float a, float b) { return copysignf(fmaxf(min_xorsign(a, b), 0.f), a); }
+
 // MC alone (the same values as limited(a, b, HYDRO_MC)); double-float selected, not branched.
 template <class R>
 __device__ __forceinline__ R mc_slope(R a, R b) {
   return limited(a, b, HYDRO_MC);
+}
+__device__ __forceinline__ float mc_slope(float a, float b) {
+  const float m = fabsf(0.5f * (a + b));
+  return copysignf(fmaxf(fminf(2.f * min_xorsign(a, b), m), 0.f), a);
 }
 __device__ __forceinline__ df mc_pick(const df& a, const df& b, const df& m) {  // m = (a + b)/2
   const bool pos = a.h > 0.f;
@@ -189,6 +223,18 @@ __device__ __forceinline__ df mc_slope(const df& a, const df& b) { return mc_pic
 __device__ __forceinline__ df2 mc_slope(const df2& a, const df2& b) {
   const df2 m = half_(a + b);
   return pair_(mc_pick(first_(a), first_(b), first_(m)), mc_pick(second_(a), second_(b), second_(m)));
+}
+
+// The limiter of the run time, in the selected forms (other types: limited).
+template <class R>
+__device__ __forceinline__ R limited_sel(R a, R b, int lim) {
+  return limited(a, b, lim);
+}
+__device__ __forceinline__ float limited_sel(float a, float b, int lim) {
+  return lim == HYDRO_MINMOD ? minmod(a, b) : (lim == HYDRO_MC ? mc_slope(a, b) : 0.5f * (a + b));
+}
+__device__ __forceinline__ df limited_sel(const df& a, const df& b, int lim) {
+  return lim == HYDRO_MINMOD ? minmod(a, b) : (lim == HYDRO_MC ? mc_slope(a, b) : half_(a + b));
 }
 
 // ------------------------------------------------------------------ Hancock predictor
@@ -223,6 +269,21 @@ __device__ __forceinline__ void hancock(const R q[5], const R dqx[5], const R dq
   qh[4] = q[4] - hdt * ((tx4 + ty4) + tz4);
 }
 
+// Double: the same rows in fused multiply-adds (25 operations on the FP64 pipe, the generic form 34).
+__device__ __forceinline__ void hancock(const double q[5], const double dqx[5], const double dqy[5],
+                                        const double dqz[5], double gamma, double hdt, double qh[5]) {
+  const double ir = rcp_(q[0]);
+  const double gp = gamma * q[4];
+  const double div = (dqx[1] + dqy[2]) + dqz[3];
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    const double a = v == 0 ? q[0] : (v == 4 ? gp : ir);
+    const double b = v == 0 || v == 4 ? div : (v == 1 ? dqx[4] : (v == 2 ? dqy[4] : dqz[4]));
+    const double t = fma(a, b, fma(q[3], dqz[v], fma(q[2], dqy[v], q[1] * dqx[v])));
+    qh[v] = fma(-hdt, t, q[v]);
+  }
+}
+
 // The same in double-float: each row is one sum of four products, closed by one normalisation, with
 // the velocity divergence formed once; rows (0, 1) and (2, 3) side by side in packed FP32.
 __device__ __forceinline__ void hancock(const df q[5], const df dqx[5], const df dqy[5], const df dqz[5],
@@ -250,24 +311,41 @@ __device__ __forceinline__ void floor_state(R q[5], R rho_floor, R p_floor) {
   q[4] = cmp_lt_floor(q[4], p_floor) ? p_floor : q[4];
 }
 
+// The lesser and the greater of two wave speeds (float: one operation).
+template <class R>
+__device__ __forceinline__ R lesser(R a, R b) { return a <= b ? a : b; }
+template <class R>
+__device__ __forceinline__ R greater(R a, R b) { return a >= b ? a : b; }
+__device__ __forceinline__ float lesser(float a, float b) { return fminf(a, b); }
+__device__ __forceinline__ float greater(float a, float b) { return fmaxf(a, b); }
+// floor_state, in float by the larger of the two (a NaN stays NaN): one operation each.
+template <class R>
+__device__ __forceinline__ void floor_max(R q[5], R rho_floor, R p_floor) {
+  floor_state(q, rho_floor, p_floor);
+}
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float t;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(t) : "f"(a), "f"(b));
+  return t;
+}
+__device__ __forceinline__ void floor_max(float q[5], float rho_floor, float p_floor) {
+  q[0] = max_nan(q[0], rho_floor);
+  q[4] = max_nan(q[4], p_floor);
+}
+
 // ------------------------------------------------------------------ HLLC
 // Flux through a face between floored states, in face-normal components: q = (rho, u_n, u_t1,
 // u_t2, p); ke = u^2 + v^2 + w^2 summed in x, y, z order.  F = F_L if 0 <= S_L; F_R if S_R <= 0;
 // else F_K + S_K (U*_K - U_K) with K = L if S* >= 0 else R (Davis speeds, Batten et al. star
 // state).  Only the upwind side's physical flux is formed; branches are selected, not multiplied.
-// 1/a and 1/b.  In double, where a division is a long sequence on the FP64 pipe, both come from
-// one division, 1/a = b/(ab), 1/b = a/(ab) (the operands here are positive densities, or a mass
-// flux and a speed difference, whose products stay far inside the exponent range).  A float
-// reciprocal is one SFU instruction, and a double-float one costs about what the two extra
-// double-float products would: two reciprocals.
+// 1/a and 1/b.
 __device__ __forceinline__ void rcp2(float a, float b, float& ra, float& rb) {
   ra = rcp_(a);
   rb = rcp_(b);
 }
 __device__ __forceinline__ void rcp2(double a, double b, double& ra, double& rb) {
-  const double i = 1.0 / (a * b);
-  ra = b * i;
-  rb = a * i;
+  ra = rcp_(a);
+  rb = rcp_(b);
 }
 __device__ __forceinline__ void rcp2(const df& a, const df& b, df& ra, df& rb) {
   ra = rcp_(a);
@@ -286,9 +364,9 @@ __device__ __forceinline__ void hllc_core(const R qL[5], const R qR[5], bool zn,
   const R cR = rsqrt_(gamma * qR[4] * irR);
   const R uL = qL[1], uR = qR[1];
   const R aL = uL - cL, bL = uR - cR;
-  const R SL = aL <= bL ? aL : bL;
+  const R SL = lesser(aL, bL);
   const R aR = uL + cL, bR = uR + cR;
-  const R SR = aR >= bR ? aR : bR;
+  const R SR = greater(aR, bR);
   const R mL = qL[0] * (SL - uL);
   const R mR = qR[0] * (SR - uR);
   const R Ss = div_(qR[4] - qL[4] + uL * mL - uR * mR, mL - mR);
@@ -326,6 +404,49 @@ __device__ __forceinline__ void hllc_core(const R qL[5], const R qR[5], bool zn,
   F[4] = ue * (Ee + pe);
 }
 
+// The same flux in double, in the form of the double-float one below (S* from its distance to u_L, the
+// star energy without 1/m_K): about 75 operations on the FP64 pipe, the generic form with IEEE
+// divisions and roots about 120.
+__device__ __forceinline__ void hllc_core(const double qL[5], const double qR[5], bool, double gamma, double inv_gm1,
+                                          double F[5]) {
+  const double cL = rsqrt_(div_(gamma * qL[4], qL[0])), cR = rsqrt_(div_(gamma * qR[4], qR[0]));
+  const double uL = qL[1], uR = qR[1];
+  const double aL = uL - cL, bL = uR - cR, aR = uL + cL, bR = uR + cR;
+  const double SL = aL <= bL ? aL : bL, SR = aR >= bR ? aR : bR;
+  const double dL = SL - uL, dR = SR - uR;
+  const double mL = qL[0] * dL, mR = qR[0] * dR;
+  const double du = uL - uR;
+  const double dl = div_(fma(mR, du, qR[4] - qL[4]), mL - mR);  // S* - u_L
+  const double Ss = uL + dl;
+  const bool SLneg = cmp_neg(SL), SRpos = cmp_pos(SR);
+  const bool star = SLneg && SRpos;
+  const bool left = !SLneg || (SRpos && !cmp_neg(Ss));
+  const double rK = left ? qL[0] : qR[0];
+  const double uK = left ? uL : uR;
+  const double t1 = left ? qL[2] : qR[2];
+  const double t2 = left ? qL[3] : qR[3];
+  const double pK = left ? qL[4] : qR[4];
+  const double mK = left ? mL : mR;
+  const double dK = left ? dL : dR;
+  const double d = left ? dl : dl + du;  // S* - u_K
+  const double ke = fma(t2, t2, fma(t1, t1, uK * uK));
+  const double EK = fma(0.5 * rK, ke, pK * inv_gm1);
+  const double iD = rcp_(dK - d);
+  const double rs = mK * iD, g = dK * iD;
+  const double ps = fma(mK, d, pK);
+  const double Es = fma(d, fma(rs, Ss, pK * iD), g * EK);
+  const double re = star ? rs : rK;
+  const double ue = star ? Ss : uK;
+  const double pe = star ? ps : pK;
+  const double Ee = star ? Es : EK;
+  const double mn = re * ue;
+  F[0] = mn;
+  F[1] = fma(mn, ue, pe);
+  F[2] = mn * t1;
+  F[3] = mn * t2;
+  F[4] = ue * (Ee + pe);
+}
+
 // The same flux in double-float: the two sides side by side in packed FP32 up to S*, sums and products
 // left unnormalised inside the formulas, S* from its distance to u_L (S* - u_L = (p_R - p_L + m_R (u_L -
 // u_R)) / (m_L - m_R), which does not cancel in fast flow), and the star energy without 1/m_K: with i =
@@ -340,11 +461,11 @@ __device__ __forceinline__ void hllc_core(const df qL[5], const df qR[5], bool, 
   const df aL = first_(lo), bL = second_(lo), aR = first_(hi), bR = second_(hi);
   const df SL = aL <= bL ? aL : bL;
   const df SR = aR >= bR ? aR : bR;
-  const df2 d2 = sum_(pair_(SL, SR), neg_(u2));  // S - u of either side
-  const df2 m2 = prod_(r2, d2);
+  const df2 d2 = pair_(SL, SR) - u2;  // S - u of either side
+  const df2 m2 = norm_(prod_(r2, d2));
   const df du = sum_(qL[1], -qR[1]);
   const df num = sum_(sum_(qR[4], -qL[4]), prod_(second_(m2), du));
-  const df dl = quot_(num, sum_(first_(m2), -second_(m2)));  // S* - u_L
+  const df dl = norm_(quot_(norm_(num), first_(m2) - second_(m2)));  // S* - u_L
   const df Ss = qL[1] + dl;
   const bool SLneg = cmp_neg(SL), SRpos = cmp_pos(SR);
   const bool star = SLneg && SRpos;
@@ -362,7 +483,7 @@ __device__ __forceinline__ void hllc_core(const df qL[5], const df qR[5], bool, 
   const df EK = norm_(sum_(prod_(pK, inv_gm1), prod_(half_(rK), ke)));
   const df dr = sum_(dl, du);
   const df d = norm_(left ? dl : dr);  // S* - u_K
-  const df iD = rcpu_(sum_(dK, -d));
+  const df iD = norm_(rcpu_(dK - d));
   const df2 rg = prod_(both_(iD), pair_(mK, dK));
   const df rs = first_(rg), g = second_(rg);
   const df ps = sum_(pK, prod_(mK, d));
@@ -373,11 +494,11 @@ __device__ __forceinline__ void hllc_core(const df qL[5], const df qR[5], bool, 
   const df Ee = star ? Es : EK;
   const df mn = norm_(prod_(re, ue));
   F[0] = mn;
-  F[1] = sum_(prod_(mn, ue), pe);
+  F[1] = norm_(prod_(mn, ue)) + pe;
   const df2 ft = prod_(both_(mn), tt);
   F[2] = first_(ft);
   F[3] = second_(ft);
-  F[4] = prod_(ue, sum_(Ee, pe));
+  F[4] = prod_(ue, Ee + pe);
 }
 
 template <class R>
@@ -481,7 +602,7 @@ struct PolF64 {
   static __device__ __forceinline__ void recover(const double U[5], const Params& P, double q[5], unsigned& flags) {
     double rho = U[0];
     if (rho < P.rho_floor) { flags |= HYDRO_EBIT_RHO_FLOOR; rho = P.rho_floor; }
-    const double ir = 1.0 / rho;
+    const double ir = rcp_(rho);
     const double kin = 0.5 * (U[1] * U[1] + U[2] * U[2] + U[3] * U[3]) * ir;
     const double eint = U[4] - kin;
     if (eint < 0.0) flags |= HYDRO_EBIT_P_FLOOR;
@@ -527,7 +648,7 @@ struct PolF32 {
     const float eint = d + (de - 0.5f * kl);
     if (eint < 0.f) flags |= HYDRO_EBIT_P_FLOOR;
     float p = P.kf[K_GM1] * eint;
-    if (!(isfinite(p) && isfinite(rho))) flags |= HYDRO_EBIT_NONFINITE;
+    if (!isfinite(p)) flags |= HYDRO_EBIT_NONFINITE;  // (a density that is not finite leaves none finite)
     const float pf = P.kf[K_PF];
     q[0] = rho;
     q[1] = mx * ir;
@@ -545,7 +666,7 @@ struct PolF32 {
     const float u = U[1] * ir, v = U[2] * ir, w = U[3] * ir;
     const float eint = U[4] - 0.5f * rho * ((u * u + v * v) + w * w);
     float p = P.kf[K_GM1] * eint;
-    if (!(isfinite(p) && isfinite(rho))) flags |= HYDRO_EBIT_NONFINITE;
+    if (!isfinite(p)) flags |= HYDRO_EBIT_NONFINITE;
     const float pf = P.kf[K_PF];
     p = p < pf ? pf : p;
     const float c = rsqrt_(P.kf[K_GAMMA] * p * ir);
@@ -593,7 +714,7 @@ struct PolMixed {
     const float eint = d + ((de + el) - 0.5f * kl);
     if (eint < 0.f) flags |= HYDRO_EBIT_P_FLOOR;
     float p = P.kf[K_GM1] * eint;
-    if (!(isfinite(p) && isfinite(rh))) flags |= HYDRO_EBIT_NONFINITE;
+    if (!isfinite(p)) flags |= HYDRO_EBIT_NONFINITE;  // (a density that is not finite leaves none finite)
     const float pf = P.kf[K_PF];
     q[0] = rh;
     q[1] = xh * ir;
@@ -612,7 +733,7 @@ struct PolDF {
   using S = double;
   using R = df;
   // The same recovery as PolF64, in double-float from the double state (split into float pairs on
-  // the integer pipe, split_double); ir receives 1/rho (unnormalised).
+  // the integer pipe, split_double); ir receives 1/rho.
   static __device__ __forceinline__ void recover(const double U[5], const Params& P, df q[5], df& ir, unsigned& flags) {
     df rho, mx, my, mz, E;
     split_double(U[0], rho.h, rho.l);
@@ -622,9 +743,9 @@ struct PolDF {
     split_double(U[4], E.h, E.l);
     const df rf = kc<df>(P, K_RHOF);
     if (rho < rf) { flags |= HYDRO_EBIT_RHO_FLOOR; rho = rf; }
-    ir = rcpu_(rho);
+    ir = norm_(rcpu_(rho));
     const df2 mxy = pair_(mx, my), sq = prod_(mxy, mxy);
-    const df kin = norm_(prod_(sum_(sum_(first_(sq), second_(sq)), prod_(mz, mz)), half_(ir)));
+    const df kin = norm_(prod_(norm_(sum_(sum_(first_(sq), second_(sq)), prod_(mz, mz))), half_(ir)));
     const df eint = sub_acc(E, kin);
     if (cmp_neg(eint)) flags |= HYDRO_EBIT_P_FLOOR;
     df p = norm_(prod_(kc<df>(P, K_GM1), eint));

@@ -5,7 +5,7 @@
 //   edges qL = q_{i-h}, qR = q_{i+h}, then: both set to q_i at a local extremum
 //   ((qR - q)(q - qL) <= 0); else with D = qR - qL, Q6 = 6 (q - (qL + qR)/2): qL = 3q - 2qR if
 //   D Q6 > D^2, qR = 3q - 2qL if -D^2 > D Q6.
-// Only the distances l = q - qL and r = qR - q are formed, from differences alone:
+// In double and double-float only the distances l = q - qL and r = qR - q are formed, from differences alone:
 //   l = (q_i - q_{i-1})/2 + (dq_i - dq_{i-1})/6,   r = (q_{i+1} - q_i)/2 - (dq_{i+1} - dq_i)/6,
 // both 0 where l r <= 0; there D = l + r and Q6 = 3 (l - r), so the two steepness tests are |l| > 2|r|
 // (then l = 2r) and |r| > 2|l| (then r = 2l).  Half the operations of the edge form, none of its
@@ -95,37 +95,64 @@ __device__ __forceinline__ void ppm_edge(const df2& ba, const df2& cb, const df2
   ppm_limit(l[1], r[1]);
 }
 
-// The same for the five values of consecutive cells a, b, c, d, e (double-float: values 0, 1 and 2, 3
-// in packed FP32).
+// The same for the five values of consecutive cells a, b, c, d, e, and the centre slopes D = l + r
+// (double-float: values 0, 1 and 2, 3 in packed FP32).
 template <class R>
 __device__ __forceinline__ void ppm_edges5(const R a[5], const R b[5], const R c[5], const R d[5], const R e[5],
-                                           R sixth, R l[5], R r[5]) {
+                                           R sixth, R l[5], R r[5], R D[5]) {
 #pragma unroll
   for (int v = 0; v < 5; ++v) ppm_edge(b[v] - a[v], c[v] - b[v], d[v] - c[v], e[v] - d[v], sixth, l[v], r[v]);
+  add5(l, r, D);
+}
+// Float forms the edges themselves (Colella & Woodward's constraints as printed): mixed precision keeps
+// the roundings of its float arithmetic in a double state, so they are part of its results.
+__device__ __forceinline__ void ppm_edges5(const float a[5], const float b[5], const float c[5], const float d[5],
+                                           const float e[5], float sixth, float l[5], float r[5], float D[5]) {
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    const float sb = mc_slope(b[v] - a[v], c[v] - b[v]), sc = mc_slope(c[v] - b[v], d[v] - c[v]),
+                sd = mc_slope(d[v] - c[v], e[v] - d[v]);
+    float qL = (b[v] + half_(c[v] - b[v])) - (sc - sb) * sixth;
+    float qR = (c[v] + half_(d[v] - c[v])) - (sd - sc) * sixth;
+    if (prod_nonpos(qR - c[v], c[v] - qL)) {
+      qL = qR = c[v];
+    } else {
+      const float S = qR - qL, Q6 = mulf_(c[v] - half_(qL + qR), 6.f);
+      const float SQ = S * Q6, SS = S * S;
+      if (SQ > SS)
+        qL = mulf_(c[v], 3.f) - twice_(qR);
+      else if (-SS > SQ)
+        qR = mulf_(c[v], 3.f) - twice_(qL);
+    }
+    D[v] = qR - qL;
+    l[v] = c[v] - qL;
+    r[v] = qR - c[v];
+  }
 }
 __device__ __forceinline__ void ppm_edges5(const df a[5], const df b[5], const df c[5], const df d[5], const df e[5],
-                                           df sixth, df l[5], df r[5]) {
+                                           df sixth, df l[5], df r[5], df D[5]) {
 #pragma unroll
   for (int v = 0; v < 4; v += 2) {
     const df2 A = pair_(a[v], a[v + 1]), B = pair_(b[v], b[v + 1]), C = pair_(c[v], c[v + 1]),
-              D = pair_(d[v], d[v + 1]), E = pair_(e[v], e[v + 1]);
-    ppm_edge(B - A, C - B, D - C, E - D, sixth, l + v, r + v);
+              G = pair_(d[v], d[v + 1]), E = pair_(e[v], e[v + 1]);
+    ppm_edge(B - A, C - B, G - C, E - G, sixth, l + v, r + v);
   }
   ppm_edge(b[4] - a[4], c[4] - b[4], d[4] - c[4], e[4] - d[4], sixth, l[4], r[4]);
+  add5(l, r, D);
 }
 
 // Edge distances of tile cell (i, j) of the middle plane along axis d (0 x, 1 y, 2 z); q: the cell's
 // own values.  sl: ring slots of planes p-2 .. p+2.
 template <class R, int TX, int TY>
 __device__ __forceinline__ void ppm_axis(const PpmShared<R, TX, TY>& sm, const int sl[5], int i, int j, int d,
-                                         const R q[5], R sixth, R l[5], R r[5]) {
+                                         const R q[5], R sixth, R l[5], R r[5], R D[5]) {
   const int X = i + kPpmHalo, Y = j + kPpmHalo, dx = d == 0, dy = d == 1;
   R a[5], b[5], e[5], f[5];
   sm.q[d == 2 ? sl[0] : sl[2]].ld(Y - 2 * dy, X - 2 * dx, a);
   sm.q[d == 2 ? sl[1] : sl[2]].ld(Y - dy, X - dx, b);
   sm.q[d == 2 ? sl[3] : sl[2]].ld(Y + dy, X + dx, e);
   sm.q[d == 2 ? sl[4] : sl[2]].ld(Y + 2 * dy, X + 2 * dx, f);
-  ppm_edges5(a, b, q, e, f, sixth, l, r);
+  ppm_edges5(a, b, q, e, f, sixth, l, r, D);
 }
 
 // Edge distances of tile cell (i, j) along x, y and z, and the Hancock-predicted state qh.
@@ -135,10 +162,7 @@ __device__ __forceinline__ void ppm_cell(const PpmShared<R, TX, TY>& sm, const i
   R q[5], D[3][5];
   sm.q[sl[2]].ld(j + kPpmHalo, i + kPpmHalo, q);
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    ppm_axis(sm, sl, i, j, d, q, sixth, l[d], r[d]);
-    add5(l[d], r[d], D[d]);
-  }
+  for (int d = 0; d < 3; ++d) ppm_axis(sm, sl, i, j, d, q, sixth, l[d], r[d], D[d]);
   hancock(q, D[0], D[1], D[2], gamma, hdt, qh);
 }
 
@@ -159,9 +183,8 @@ __device__ __forceinline__ void ppm_cell_axes(const PpmShared<df, TX, TY>& sm, c
 #pragma unroll 1
   for (int d = 0; d < 3; ++d) {
     df l[5], r[5], D[5];
-    ppm_axis(sm, sl, i, j, d, q, sixth, l, r);
+    ppm_axis(sm, sl, i, j, d, q, sixth, l, r, D);
     out(d, l, r);
-    add5(l, r, D);
     // Hancock terms of axis d (normal velocity q[1 + d]), as in hancock()
     const df un = d == 0 ? q[1] : (d == 1 ? q[2] : q[3]);
     const df Dn = d == 0 ? D[1] : (d == 1 ? D[2] : D[3]);
@@ -291,15 +314,17 @@ __device__ __forceinline__ void ppm_tile(PpmShared<typename Pol::R, TX, TY>& sm,
           ql[v] = zhi[v];
           qr[v] = zlo[v];
         }
-        floor_state(ql, rf, pf);
-        floor_state(qr, rf, pf);
+        floor_max(ql, rf, pf);
+        floor_max(qr, rf, pf);
         hllc<2>(ql, qr, gamma, igm1, F);
         if (p > z0 && own) {
           const int z = p - 1;
           const long long ai = (long long)(z + P.gin) * P.isz + (long long)(y0 + j + P.gin) * P.isy + (x0 + i + P.gin);
           const long long ao = (long long)(z + P.gout) * P.osz + (long long)(y0 + j + P.gout) * P.osy + (x0 + i + P.gout);
           S Un[5];
-          div_z(F, fzb, dxy);
+          R dz[5];
+          sub5(F, fzb, dz);
+          add5(dxy, dz, dxy);
 #pragma unroll
           for (int v = 0; v < 5; ++v) {
             Un[v] = Pol::update(__ldg(P.in[v] + ai), dtdx, dxy[v]);
@@ -434,8 +459,8 @@ __device__ __forceinline__ void ppm_tile(PpmShared<typename Pol::R, TX, TY>& sm,
           sm.wy[1].ld(fy, fx, ql);
           sm.wy[0].ld(fy + 1, fx, qr);
         }
-        floor_state(ql, rf, pf);
-        floor_state(qr, rf, pf);
+        floor_max(ql, rf, pf);
+        floor_max(qr, rf, pf);
         hllc_dyn(d, ql, qr, gamma, igm1, F);
         if (d == 0) sm.fx.st(fy, fx, F);
         else sm.fy.st(fy, fx, F);
@@ -465,8 +490,8 @@ __device__ __forceinline__ void ppm_tile(PpmShared<typename Pol::R, TX, TY>& sm,
           sm.wy[1].ld(fy, fx, ql);
           sm.wy[0].ld(fy + 1, fx, qr);
         }
-        floor_state(ql, rf, pf);
-        floor_state(qr, rf, pf);
+        floor_max(ql, rf, pf);
+        floor_max(qr, rf, pf);
         hllc_dyn(d, ql, qr, gamma, igm1, F);
         if (d == 0) sm.fx.st(fy, fx, F);
         else sm.fy.st(fy, fx, F);
@@ -477,8 +502,8 @@ __device__ __forceinline__ void ppm_tile(PpmShared<typename Pol::R, TX, TY>& sm,
         R ql[5], qr[5], F[5];
         sm.wx[1].ld(fy, fx, ql);
         sm.wx[0].ld(fy, fx + 1, qr);
-        floor_state(ql, rf, pf);
-        floor_state(qr, rf, pf);
+        floor_max(ql, rf, pf);
+        floor_max(qr, rf, pf);
         hllc<0>(ql, qr, gamma, igm1, F);
         sm.fx.st(fy, fx, F);
       }
@@ -487,8 +512,8 @@ __device__ __forceinline__ void ppm_tile(PpmShared<typename Pol::R, TX, TY>& sm,
         R ql[5], qr[5], F[5];
         sm.wy[1].ld(fy, fx, ql);
         sm.wy[0].ld(fy + 1, fx, qr);
-        floor_state(ql, rf, pf);
-        floor_state(qr, rf, pf);
+        floor_max(ql, rf, pf);
+        floor_max(qr, rf, pf);
         hllc<1>(ql, qr, gamma, igm1, F);
         sm.fy.st(fy, fx, F);
       }

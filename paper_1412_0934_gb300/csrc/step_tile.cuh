@@ -94,17 +94,19 @@ struct Plane5<df, H, W> {
   }
 };
 
-// Halves of five values (exact), and five sums or differences at once (double-float: values 0, 1 and 2, 3 in packed FP32).
+// Slopes as they are kept for the face states: halved in double-float, whose additions take two plain
+// operands; as they are elsewhere, where the half is free in a fused multiply-add (side5).
 template <class R>
-__device__ __forceinline__ void half5(const R a[5], R r[5]) {
+__device__ __forceinline__ void keep5(const R a[5], R r[5]) {
 #pragma unroll
-  for (int v = 0; v < 5; ++v) r[v] = half_(a[v]);
+  for (int v = 0; v < 5; ++v) r[v] = a[v];
 }
-__device__ __forceinline__ void half5(const df a[5], df r[5]) {
+__device__ __forceinline__ void keep5(const df a[5], df r[5]) {
   const df2 s = half_(pair_(a[0], a[1])), t = half_(pair_(a[2], a[3]));
   r[0] = first_(s); r[1] = second_(s); r[2] = first_(t); r[3] = second_(t);
   r[4] = half_(a[4]);
 }
+// Five sums or differences at once (float and double-float: values 0, 1 and 2, 3 in packed FP32).
 template <class R>
 __device__ __forceinline__ void sub5(const R a[5], const R b[5], R r[5]) {
 #pragma unroll
@@ -113,6 +115,12 @@ __device__ __forceinline__ void sub5(const R a[5], const R b[5], R r[5]) {
 __device__ __forceinline__ void sub5(const df a[5], const df b[5], df r[5]) {
   const df2 s = pair_(a[0], a[1]) - pair_(b[0], b[1]), t = pair_(a[2], a[3]) - pair_(b[2], b[3]);
   r[0] = first_(s); r[1] = second_(s); r[2] = first_(t); r[3] = second_(t);
+  r[4] = a[4] - b[4];
+}
+__device__ __forceinline__ void sub5(const float a[5], const float b[5], float r[5]) {
+  const float2 s = sub2_(make_float2(a[0], a[1]), make_float2(b[0], b[1]));
+  const float2 t = sub2_(make_float2(a[2], a[3]), make_float2(b[2], b[3]));
+  r[0] = s.x; r[1] = s.y; r[2] = t.x; r[3] = t.y;
   r[4] = a[4] - b[4];
 }
 template <class R>
@@ -125,36 +133,44 @@ __device__ __forceinline__ void add5(const df a[5], const df b[5], df r[5]) {
   r[0] = first_(s); r[1] = second_(s); r[2] = first_(t); r[3] = second_(t);
   r[4] = a[4] + b[4];
 }
-// The flux divergence ((xp - xm) + (yp - ym) - zm) + zp of five fields: in two parts, the z fluxes
-// living in registers (double-float: unnormalised, the update closes it).
+__device__ __forceinline__ void add5(const float a[5], const float b[5], float r[5]) {
+  const float2 s = add2_(make_float2(a[0], a[1]), make_float2(b[0], b[1]));
+  const float2 t = add2_(make_float2(a[2], a[3]), make_float2(b[2], b[3]));
+  r[0] = s.x; r[1] = s.y; r[2] = t.x; r[3] = t.y;
+  r[4] = a[4] + b[4];
+}
+// Face states of a cell: q + slope/2 (SIGN 1) or q - slope/2 (SIGN -1) from the kept slopes.
+template <int SIGN, class R>
+__device__ __forceinline__ void side5(const R q[5], const R s[5], R r[5]) {
+#pragma unroll
+  for (int v = 0; v < 5; ++v) r[v] = SIGN > 0 ? q[v] + half_(s[v]) : q[v] - half_(s[v]);
+}
+template <int SIGN>
+__device__ __forceinline__ void side5(const float q[5], const float s[5], float r[5]) {
+  const float2 h = make_float2(SIGN * 0.5f, SIGN * 0.5f);
+  const float2 a = fma2_(make_float2(s[0], s[1]), h, make_float2(q[0], q[1]));
+  const float2 b = fma2_(make_float2(s[2], s[3]), h, make_float2(q[2], q[3]));
+  r[0] = a.x; r[1] = a.y; r[2] = b.x; r[3] = b.y;
+  r[4] = fmaf(s[4], SIGN * 0.5f, q[4]);
+}
+template <int SIGN>
+__device__ __forceinline__ void side5(const df q[5], const df s[5], df r[5]) {
+  if constexpr (SIGN > 0) add5(q, s, r);
+  else sub5(q, s, r);
+}
+// The flux divergence ((xp - xm) + (yp - ym) - zm) + zp of five fields, in two parts: the z fluxes live
+// in registers.
 template <class R>
 __device__ __forceinline__ void div_xy(const R xp[5], const R xm[5], const R yp[5], const R ym[5], R d[5]) {
-#pragma unroll
-  for (int v = 0; v < 5; ++v) d[v] = (xp[v] - xm[v]) + (yp[v] - ym[v]);
+  R a[5], b[5];
+  sub5(xp, xm, a);
+  sub5(yp, ym, b);
+  add5(a, b, d);
 }
 template <class R>
 __device__ __forceinline__ void div_z(const R zp[5], const R zm[5], R d[5]) {
-#pragma unroll
-  for (int v = 0; v < 5; ++v) d[v] = (d[v] - zm[v]) + zp[v];
-}
-__device__ __forceinline__ void div_xy(const df xp[5], const df xm[5], const df yp[5], const df ym[5], df d[5]) {
-#pragma unroll
-  for (int v = 0; v < 4; v += 2) {
-    const df2 t = sum_(sum_(pair_(xp[v], xp[v + 1]), neg_(pair_(xm[v], xm[v + 1]))),
-                       sum_(pair_(yp[v], yp[v + 1]), neg_(pair_(ym[v], ym[v + 1]))));
-    d[v] = first_(t);
-    d[v + 1] = second_(t);
-  }
-  d[4] = sum_(sum_(xp[4], -xm[4]), sum_(yp[4], -ym[4]));
-}
-__device__ __forceinline__ void div_z(const df zp[5], const df zm[5], df d[5]) {
-#pragma unroll
-  for (int v = 0; v < 4; v += 2) {
-    const df2 t = sum_(sum_(pair_(d[v], d[v + 1]), neg_(pair_(zm[v], zm[v + 1]))), pair_(zp[v], zp[v + 1]));
-    d[v] = first_(t);
-    d[v + 1] = second_(t);
-  }
-  d[4] = sum_(sum_(d[4], -zm[4]), zp[4]);
+  sub5(d, zm, d);
+  add5(d, zp, d);
 }
 
 template <class Pol, int TX, int TY>
@@ -162,8 +178,8 @@ struct TileShared {
   using R = typename Pol::R;
   Plane5<R, TY + 4, TX + 4> q[3];  // primitive planes p-1, p, p+1 (ring)
   Plane5<R, TY + 2, TX + 2> qh;    // predicted state of plane p (tile + 1 ring)
-  Plane5<R, TY + 2, TX + 2> sx;    // half x slopes of plane p
-  Plane5<R, TY + 2, TX + 2> sy;    // half y slopes of plane p
+  Plane5<R, TY + 2, TX + 2> sx;    // kept x slopes of plane p
+  Plane5<R, TY + 2, TX + 2> sy;    // kept y slopes of plane p
   Plane5<R, TY, TX + 1> fx;        // x-face fluxes of plane p, index i+1 for face i+1/2
   Plane5<R, TY + 1, TX> fy;        // y-face fluxes of plane p, index j+1 for face j+1/2
   long long yoff[TY + 4];          // y offset (y index * stride) of the halo rows
@@ -171,6 +187,7 @@ struct TileShared {
   int pairok[(TX + 4) / 2];        // halo columns 2k, 2k+1 adjacent in memory, the first even
   R red[TX * TY / 32];
   int tile;
+  PatchIO<typename Pol::S> io;     // batched kernel: the current patch
 };
 
 __device__ __forceinline__ int wrapi(int x, int n) {
@@ -192,7 +209,7 @@ __device__ __forceinline__ R limited_t(R a, R b, int) {
 template <int LIM, class Pol, int TX, int TY>
 __device__ __forceinline__ void predict_cell(TileShared<Pol, TX, TY>& sm, int i, int j, int sm1, int s0, int sp1,
                                              const Params& prm, typename Pol::R hdt, typename Pol::R qh[5],
-                                             typename Pol::R dqz[5]) {  // dqz: half the z slopes
+                                             typename Pol::R dqz[5]) {  // dqz: the kept z slopes
   using R = typename Pol::R;
   const int ci = i + 2, cj = j + 2;
   R c[5], dqx[5], dqy[5], h[5];
@@ -211,11 +228,11 @@ __device__ __forceinline__ void predict_cell(TileShared<Pol, TX, TY>& sm, int i,
   slope(sm.q[sm1], cj, ci, sm.q[sp1], cj, ci, dqz);
   hancock(c, dqx, dqy, dqz, kc<R>(prm, K_GAMMA), hdt, qh);
   sm.qh.st(j + 1, i + 1, qh);
-  half5(dqx, h);
+  keep5(dqx, h);
   sm.sx.st(j + 1, i + 1, h);
-  half5(dqy, h);
+  keep5(dqy, h);
   sm.sy.st(j + 1, i + 1, h);
-  half5(dqz, dqz);
+  keep5(dqz, dqz);
 }
 
 // Flux of the x face between tile cells (i, j) and (i+1, j) (D = 0) or the y face between
@@ -236,10 +253,10 @@ __device__ __forceinline__ void face_flux(TileShared<Pol, TX, TY>& sm, int i, in
     sm.sy.ld(lj, li, sL);
     sm.sy.ld(rj, ri, sR);
   }
-  add5(qL, sL, qL);
-  sub5(qR, sR, qR);
-  floor_state(qL, kc<R>(prm, K_RHOF), kc<R>(prm, K_PF));
-  floor_state(qR, kc<R>(prm, K_RHOF), kc<R>(prm, K_PF));
+  side5<1>(qL, sL, qL);
+  side5<-1>(qR, sR, qR);
+  floor_max(qL, kc<R>(prm, K_RHOF), kc<R>(prm, K_PF));
+  floor_max(qR, kc<R>(prm, K_RHOF), kc<R>(prm, K_PF));
   hllc<D>(qL, qR, kc<R>(prm, K_GAMMA), kc<R>(prm, K_IGM1), F);
 }
 
@@ -256,10 +273,10 @@ __device__ __forceinline__ void face_flux_dyn(TileShared<Pol, TX, TY>& sm, int d
   const auto& sl = d == 0 ? sm.sx : sm.sy;
   sl.ld(lj, li, sL);
   sl.ld(rj, ri, sR);
-  add5(qL, sL, qL);
-  sub5(qR, sR, qR);
-  floor_state(qL, kc<R>(prm, K_RHOF), kc<R>(prm, K_PF));
-  floor_state(qR, kc<R>(prm, K_RHOF), kc<R>(prm, K_PF));
+  side5<1>(qL, sL, qL);
+  side5<-1>(qR, sR, qR);
+  floor_max(qL, kc<R>(prm, K_RHOF), kc<R>(prm, K_PF));
+  floor_max(qR, kc<R>(prm, K_RHOF), kc<R>(prm, K_PF));
   hllc_dyn(d, qL, qR, kc<R>(prm, K_GAMMA), kc<R>(prm, K_IGM1), F);
 }
 
@@ -435,12 +452,12 @@ __device__ void step_tile(TileShared<Pol, TX, TY>& sm, const PatchIO<typename Po
 #pragma unroll
   for (int v = 0; v < 5; ++v) { LzPrev[v] = FzPrev[v] = Fz[v] = R(0); }
 
-  auto z_faces = [&](int p, const R qh[5], const R hz[5]) {  // hz: half z slopes
+  auto z_faces = [&](int p, const R qh[5], const R sz[5]) {  // sz: kept z slopes
     R Lz[5], Rz[5];
-    add5(qh, hz, Lz);
-    sub5(qh, hz, Rz);
-    floor_state(Lz, kc<R>(prm, K_RHOF), kc<R>(prm, K_PF));
-    floor_state(Rz, kc<R>(prm, K_RHOF), kc<R>(prm, K_PF));
+    side5<1>(qh, sz, Lz);
+    side5<-1>(qh, sz, Rz);
+    floor_max(Lz, kc<R>(prm, K_RHOF), kc<R>(prm, K_PF));
+    floor_max(Rz, kc<R>(prm, K_RHOF), kc<R>(prm, K_PF));
     if (p >= z0) hllc<2>(LzPrev, Rz, gamma, kc<R>(prm, K_IGM1), Fz);
 #pragma unroll
     for (int v = 0; v < 5; ++v) LzPrev[v] = Lz[v];
@@ -726,7 +743,14 @@ __global__ void __launch_bounds__(TX* TY, (min_blocks<Pol, TX * TY, MINB>())) k_
     const int t = sm.tile;
     if (t >= ntiles) break;
     const TileRec r = tiles[t];
-    const PatchIO<typename Pol::S> P = patches[r.patch];
+    // the patch's descriptor in shared memory: its ten pointers in registers made the float kernels spill
+    // (4096 uneven patches, mixed: 11.1 ms, 10.6 from here)
+    static_assert(sizeof(sm.io) % 8 == 0 && sizeof(sm.io) / 8 <= 32, "one word per lane of the first warp");
+    if (threadIdx.x < sizeof(sm.io) / 8)
+      reinterpret_cast<long long*>(&sm.io)[threadIdx.x] =
+          reinterpret_cast<const long long*>(patches + r.patch)[threadIdx.x];
+    __syncthreads();
+    const PatchIO<typename Pol::S>& P = sm.io;
     if (r.x0 < 0 || r.y0 < 0 || r.z0 < 0 || r.x0 >= P.nx || r.y0 >= P.ny || r.z0 >= P.nz) {
       flags |= HYDRO_EBIT_BAD_TILE;
       continue;
