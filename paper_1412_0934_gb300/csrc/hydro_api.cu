@@ -132,6 +132,9 @@ struct hydro_ctx {
   // oct builder scratch: key bitmap, word prefix sums, block prefix sums
   unsigned* d_octs_scratch = nullptr;
   size_t octs_scratch_cap = 0;
+  // oct step through the table: the list's cubes (OctCubes)
+  char* d_cubes = nullptr;
+  size_t cubes_cap = 0;
   // MHD step scratch: constants, face states, fluxes
   char* d_mhd = nullptr;
   size_t mhd_cap = 0;
@@ -590,6 +593,7 @@ int hydro_finalize(hydro_ctx* c) {
   c->xchg_sets.free_all();
   for (SetCache& s : c->aux) s.free_all();
   cudaFree(c->d_octs_scratch);
+  cudaFree(c->d_cubes);
   cudaFree(c->d_mhd);
   for (cudaEvent_t e : c->ev_copied) cudaEventDestroy(e);
   for (cudaEvent_t e : c->ev_stepped) cudaEventDestroy(e);
@@ -1223,9 +1227,34 @@ int hydro_step_octs_table(hydro_ctx* c, void* const in[5], void* const out[5], i
       const uintptr_t a = reinterpret_cast<uintptr_t>(out[v]), b = reinterpret_cast<uintptr_t>(in[u]);
       if (a < b + bytes && b < a + bytes) return HYDRO_ERR_ARG;
     }
+  // A long list: its 4^3 cubes of octs are found first and stepped as boxes of 8^3 cells.  Lists too short
+  // for one cube per SM keep the one-oct kernel, as does a captured call or one whose scratch cannot be
+  // allocated.
+  const bool cubes_pay = ngroups >= 64LL * c->sm_count && ngroups <= 0x7fffffffLL - 64;
+  hydro::OctCubes cubes;
+  bool use = false;
+  if (cubes_pay) {
+    const size_t ints = 2 + (size_t)ngroups / 64 + (size_t)ngroups, need = ints * sizeof(int) + (size_t)ngroups;
+    use = need <= c->cubes_cap;
+    if (!use) {
+      cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+      use = cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
+            ensure_device(&c->d_cubes, &c->cubes_cap, need) == HYDRO_OK;
+      if (!use) cudaGetLastError();  // the allocation's failure is handled here
+    }
+    if (use) {
+      cubes.counts = reinterpret_cast<int*>(c->d_cubes);
+      cubes.start = cubes.counts + 2;
+      cubes.left = cubes.start + ngroups / 64;
+      cubes.max_cubes = (int)(ngroups / 64);
+      cubes.covered = reinterpret_cast<unsigned char*>(cubes.left + ngroups);
+      if (hydro::find_oct_cubes(list_dev, ngroups, nbr_dev, noct, cubes, c->stream) != cudaSuccess) return HYDRO_ERR_CUDA;
+      c->launches += 3;
+    }
+  }
   c->launches += 1;
-  return cuda_status(
-      c->ops->octs_table(in, nbr_dev, noct, list_dev, out, ngroups, dx, c->prm, dt_dev, c->d_err, c->stream));
+  return cuda_status(c->ops->octs_table(in, nbr_dev, noct, list_dev, out, ngroups, dx, c->prm, dt_dev, c->d_err,
+                                        use ? &cubes : nullptr, c->stream));
 }
 
 // Arguments of the MHD calls: a periodic box of nine contiguous fields in a context with a PLM

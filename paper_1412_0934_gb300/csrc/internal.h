@@ -64,6 +64,17 @@ struct HostBoxFluxes {
   double dx;
 };
 
+// The 4^3-oct cubes of an oct list (device arrays): min(counts[0], max_cubes) cubes, cube b the 64 entries
+// from start[b]; counts[1] octs outside them, left[].  max_cubes = ngroups / 64, which only a list that
+// repeats octs can exceed (runs that overlap): the rest stay in left[].
+struct OctCubes {
+  int max_cubes;
+  int* counts;
+  int* start;
+  int* left;
+  unsigned char* covered;  // [ngroups]
+};
+
 struct KernelOps {
   // Uniform periodic grid (npatch == 1, gin == 0).
   cudaError_t (*step_uniform)(int tile, const HostPatchIO& P, const Params& prm, const double* dt, double* dt_next,
@@ -85,9 +96,10 @@ struct KernelOps {
                             const Params& prm, const double* dt, unsigned* err, cudaStream_t s);
   // Oct groups of oct-major storage read through a neighbour table; group g steps oct list[g] and
   // writes its 8 cells in place of that oct in out.
+  // cubes: nullptr, or the runs of the list found by find_oct_cubes, stepped as boxes of 8^3 cells.
   cudaError_t (*octs_table)(void* const in[5], const int* nbr, int noct, const int* list, void* const out[5],
                             long long ngroups, double dx, const Params& prm, const double* dt, unsigned* err,
-                            cudaStream_t s);
+                            const OctCubes* cubes, cudaStream_t s);
   // Adjoint of one periodic step.
   cudaError_t (*adjoint)(const HostPatchIO& U, const HostPatchIO& lam, void* const lam_out[5], const Params& prm,
                          const double* dt, void* scratch, size_t scratch_bytes, unsigned* err, cudaStream_t s);
@@ -162,6 +174,11 @@ cudaError_t launch_fill_ghosts(int elem_size, const HostGhostPatch* d_patches, c
 cudaError_t launch_octs_build(const int* pos, int noct, const int dims[3], unsigned* bitmap, unsigned* word_prefix,
                               unsigned* block_prefix, size_t nwords, int* order, int* nbr, unsigned* err,
                               cudaStream_t s);
+
+// Finds the runs of 64 list entries that are a 4^3 cube of octs in Morton order and whose 27 neighbour
+// entries per oct all agree with the cube's 6^3 neighbourhood, and lists the other entries; ngroups < 2^31.
+cudaError_t find_oct_cubes(const int* list, long long ngroups, const int* nbr, int noct, const OctCubes& cubes,
+                           cudaStream_t s);
 
 // Ideal MHD with GLM cleaning on a periodic box (mhd.cu): nine fields (rho, m, E, B, psi), each
 // nx*ny*nz contiguous, x fastest; any precision.  The step needs mhd_scratch_bytes (elem_size: bytes

@@ -6,6 +6,7 @@
 #pragma once
 #include "adjoint.cuh"
 #include "internal.h"
+#include "oct_cube.cuh"
 #include "step_ppm.cuh"
 #include "step_tile.cuh"
 
@@ -165,10 +166,13 @@ cudaError_t launch_cfl(const HostPatchIO* d_patches, const HostPatchIO& single, 
 }
 
 // ------------------------------------------------------------------ oct groups
-// One warp per group.  The 80 cells of the 6^3 stencil that the step reads are recovered into
-// shared memory; the 32 cells next to the oct's faces (the oct and the 24 outside neighbours
-// across its faces) are predicted; the 36 faces of the oct get HLLC fluxes; 8 lanes update the
-// oct.  Local coordinates run from -2 to 3 (stored at +2).
+// One warp per batch of groups.  Per group, the 80 cells of the 6^3 stencil that the step reads are
+// recovered into shared memory; the 32 cells next to the oct's faces (the oct and the 24 outside
+// neighbours across its faces) are predicted; 32 of the oct's 36 faces get their HLLC fluxes, one per
+// lane.  The other four (the upper z faces) and the oct's 8 updates would leave most lanes idle, so
+// they wait in shared memory for the batch's end: 8 groups' 32 left faces make one full round and their
+// 64 updates two (float; 4 groups in 8-byte arithmetic, whose scratch is twice as large).  A group of
+// its own took two face rounds and one update round.  Local coordinates run from -2 to 3 (stored at +2).
 __device__ __forceinline__ bool oct_needed(int x, int y, int z) {
   const int ox = (x < 0 || x > 1), oy = (y < 0 || y > 1), oz = (z < 0 || z > 1);
   const int nout = ox + oy + oz;
@@ -197,15 +201,18 @@ __device__ __forceinline__ int oct_eindex(int x, int y, int z) {
 }
 
 constexpr int kOctWarps = 4;
+template <class Pol>
+constexpr int oct_batch() { return 4; }
 
 template <class Pol>
 struct OctSmem {
   using R = typename Pol::R;
-  R q[kOctWarps][5][216];
+  R q[kOctWarps][5][80];      // needed cells in the order of need[]
   R qh[kOctWarps][5][32];
-  R sl[kOctWarps][3][5][32];
-  R f[kOctWarps][5][36];
-  short need[80];
+  R sl[kOctWarps][3][5][32];  // kept slopes
+  R f[kOctWarps][oct_batch<Pol>()][5][36];
+  R left[kOctWarps][oct_batch<Pol>()][10][4];  // lower and upper states of the upper z faces
+  short need[80], at[216];    // needed cell -> stencil cell, and back
 };
 
 // Where a group's 6^3 stencil comes from and where its 8 cells go.  OctGathered: the caller's
@@ -216,13 +223,19 @@ struct OctSmem {
 // steps oct list[g] and writes it in place of that oct.
 template <class S>
 struct OctGathered {
+  static constexpr bool kGathered = true;
   const S* f[5];
   __device__ __forceinline__ bool begin(long long, unsigned&) const { return true; }
   __device__ __forceinline__ long long cell(long long g, int c) const { return g * 216 + c; }
-  __device__ __forceinline__ long long out_cell(long long g, int e) const { return g * 8 + e; }
+  // input and output index of cell e of group g's oct (any lane's own group, already found valid)
+  __device__ __forceinline__ void own(long long g, int e, long long& in, long long& out) const {
+    in = g * 216 + ((e >> 2) + 2) * 36 + (((e >> 1) & 1) + 2) * 6 + (e & 1) + 2;
+    out = g * 8 + e;
+  }
 };
 template <class S>
 struct OctLevel {
+  static constexpr bool kGathered = false;
   const S* f[5];
   int nx, ny, nz;
   long long sy, sz;
@@ -247,10 +260,19 @@ struct OctLevel {
     z += z < 0 ? nz : (z >= nz ? -nz : 0);
     return z * sz + y * sy + x;
   }
-  __device__ __forceinline__ long long out_cell(long long g, int e) const { return g * 8 + e; }
+  __device__ __forceinline__ void own(long long g, int e, long long& in, long long& out) const {
+    int x = __ldg(origins + 3 * g) + (e & 1), y = __ldg(origins + 3 * g + 1) + ((e >> 1) & 1),
+        z = __ldg(origins + 3 * g + 2) + (e >> 2);
+    x -= x >= nx ? nx : 0;
+    y -= y >= ny ? ny : 0;
+    z -= z >= nz ? nz : 0;
+    in = z * sz + y * sy + x;
+    out = g * 8 + e;
+  }
 };
 template <class S>
 struct OctTable {
+  static constexpr bool kGathered = false;
   const S* f[5];
   const int* nbr;   // [noct][27]: oct at offset (dx, dy, dz) in entry ((dz+1)*3 + dy+1)*3 + dx+1
   const int* list;  // [ngroups]: the octs to step
@@ -275,30 +297,35 @@ struct OctTable {
     const int n = __ldg(nbr + 27LL * oct + ((z >> 1) * 3 + (y >> 1)) * 3 + (x >> 1));
     return 8LL * n + ((z & 1) * 2 + (y & 1)) * 2 + (x & 1);
   }
-  __device__ __forceinline__ long long out_cell(long long, int e) const { return 8LL * oct + e; }
+  __device__ __forceinline__ void own(long long g, int e, long long& in, long long& out) const {
+    in = out = 8LL * __ldg(list + g) + e;
+  }
 };
 
-// Resident blocks per SM: six (24 warps) for float arithmetic, measured fastest against the
-// register budget of the prefetched next group; four for 8-byte arithmetic, whose larger
-// registers would otherwise spill.
-template <class Pol>
-constexpr int oct_min_blocks() { return sizeof(typename Pol::R) >= 8 ? 4 : 6; }
+// Resident blocks per SM: as many as the batch's scratch leaves room for, in float arithmetic six (80
+// registers), five for the gathered buffer, whose prefetch spills at 80 (262144 groups, mixed: 392 us
+// against 403; the whole level through its table: 3.34 ms at six, 3.47 at five).
+template <class Pol, class Src>
+constexpr int oct_min_blocks() { return sizeof(typename Pol::R) >= 8 ? 3 : (Src::kGathered ? 5 : 6); }
 
 template <class Pol, class Src>
-__global__ void __launch_bounds__(32 * kOctWarps, oct_min_blocks<Pol>()) k_octs(Src src, typename Pol::S* o0, typename Pol::S* o1,
+__global__ void __launch_bounds__(32 * kOctWarps, (oct_min_blocks<Pol, Src>())) k_octs(Src src, typename Pol::S* o0, typename Pol::S* o1,
                                                          typename Pol::S* o2, typename Pol::S* o3,
-                                                         typename Pol::S* o4, long long ngroups, double dx, Params prm,
+                                                         typename Pol::S* o4, long long ngroups, const int* count, int batch, double dx,
+                                                         Params prm,
                                                          const double* dt_dev, unsigned* err) {
   using S = typename Pol::S;
   using R = typename Pol::R;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   auto& sm = *reinterpret_cast<OctSmem<Pol>*>(smem_raw);
   S* gout[5] = {o0, o1, o2, o3, o4};
+  if (count) ngroups = *count;  // groups left by the cube kernel
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
     int n = 0;
     for (int c = 0; c < 216; ++c) {
       const int x = c % 6 - 2, y = (c / 6) % 6 - 2, z = c / 36 - 2;
+      sm.at[c] = (short)n;
       if (oct_needed(x, y, z)) sm.need[n++] = (short)c;
     }
   }
@@ -313,8 +340,32 @@ __global__ void __launch_bounds__(32 * kOctWarps, oct_min_blocks<Pol>()) k_octs(
   const R gamma = kc<R>(prm, K_GAMMA), igm1 = kc<R>(prm, K_IGM1);
   const R rf = kc<R>(prm, K_RHOF), pf = kc<R>(prm, K_PF);
   unsigned flags = 0;
+  // This lane's predicted cell and its six neighbours among the needed cells, and its face.
+  int pc, pn[3][2];
+  {
+    int x, y, z;
+    oct_ecell(lane, x, y, z);
+    const int c = (z + 2) * 36 + (y + 2) * 6 + (x + 2);
+    pc = sm.at[c];
+    pn[0][0] = sm.at[c - 1]; pn[0][1] = sm.at[c + 1];
+    pn[1][0] = sm.at[c - 6]; pn[1][1] = sm.at[c + 6];
+    pn[2][0] = sm.at[c - 36]; pn[2][1] = sm.at[c + 36];
+  }
+  // The upper z faces' normal, 2, kept from the compiler: the flux of a run-time normal rounds as the
+  // other faces' (a fixed one contracts its kinetic sum differently).
+  int dz = 2;
+  asm("" : "+r"(dz));
+  // face between cells at coordinate s-1 and s along d; (a, b) the transverse coordinates
+  const int fd = lane / 12;
+  int eL, eR;
+  {
+    const int m = lane % 12, s = m >> 2, a = m & 1, b = (m >> 1) & 1;
+    const int lx = fd == 0 ? s - 1 : a, ly = fd == 1 ? s - 1 : (fd == 0 ? a : b), lz = fd == 2 ? s - 1 : b;
+    eL = oct_eindex(lx, ly, lz);
+    eR = oct_eindex(lx + (fd == 0), ly + (fd == 1), lz + (fd == 2));
+  }
   // The needed cells of the next group are loaded into registers while this group is computed.
-  const long long gstride = (long long)gridDim.x * kOctWarps;
+  const long long bstride = (long long)gridDim.x * kOctWarps * batch;
   S pre[3][5];
   Src nxt = src;  // source state of the prefetched group
   bool nxt_ok = false;
@@ -331,106 +382,292 @@ __global__ void __launch_bounds__(32 * kOctWarps, oct_min_blocks<Pol>()) k_octs(
       }
     }
   };
-  long long g = (long long)blockIdx.x * kOctWarps + w;
-  if (g < ngroups) fetch(g);
-  for (; g < ngroups; g += gstride) {
-    const Src cur = nxt;
-    const bool ok = nxt_ok;
-    if (!ok) {  // (warp-uniform: one warp per group)
-      if (g + gstride < ngroups) fetch(g + gstride);
-      continue;
-    }
+  long long g0 = ((long long)blockIdx.x * kOctWarps + w) * batch;
+  if (g0 < ngroups) fetch(g0);
+  for (; g0 < ngroups; g0 += bstride) {
+    const int nb = (int)(ngroups - g0 < batch ? ngroups - g0 : batch);
+    unsigned valid = 0;  // groups of the batch to update (warp-uniform)
+    for (int b = 0; b < nb; ++b) {
+      const bool ok = nxt_ok;
+      if (ok) {
 #pragma unroll
-    for (int t = 0; t < 3; ++t) {
-      const int k = lane + 32 * t;
-      if (k < 80) {
-        R q[5];
-        Pol::recover(pre[t], prm, q, flags);
-        const int c = sm.need[k];
+        for (int t = 0; t < 3; ++t) {
+          const int k = lane + 32 * t;
+          if (k < 80) {
+            R q[5];
+            Pol::recover(pre[t], prm, q, flags);
 #pragma unroll
-        for (int v = 0; v < 5; ++v) sm.q[w][v][c] = q[v];
+            for (int v = 0; v < 5; ++v) sm.q[w][v][k] = q[v];
+          }
+        }
       }
-    }
-    if (g + gstride < ngroups) fetch(g + gstride);
-    __syncwarp();
-    {
-      int x, y, z;
-      oct_ecell(lane, x, y, z);
-      const int c = (z + 2) * 36 + (y + 2) * 6 + (x + 2);
-      R q0[5], dqx[5], dqy[5], dqz[5], qh[5];
+      const long long gn = b + 1 < nb ? g0 + b + 1 : g0 + bstride;
+      if (gn < ngroups) fetch(gn);
+      if (!ok) continue;
+      valid |= 1u << b;
+      __syncwarp();
+      {
+        R q0[5], dq[3][5], qh[5];
+#pragma unroll
+        for (int v = 0; v < 5; ++v) q0[v] = sm.q[w][v][pc];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          R m[5], p[5];
+#pragma unroll
+          for (int v = 0; v < 5; ++v) {
+            m[v] = sm.q[w][v][pn[d][0]];
+            p[v] = sm.q[w][v][pn[d][1]];
+          }
+          sub5(q0, m, m);
+          sub5(p, q0, p);
+#pragma unroll
+          for (int v = 0; v < 5; ++v) dq[d][v] = limited_sel(m[v], p[v], prm.limiter);
+        }
+        hancock(q0, dq[0], dq[1], dq[2], gamma, hdt, qh);
+#pragma unroll
+        for (int v = 0; v < 5; ++v) sm.qh[w][v][lane] = qh[v];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          keep5(dq[d], dq[d]);
+#pragma unroll
+          for (int v = 0; v < 5; ++v) sm.sl[w][d][v][lane] = dq[d][v];
+        }
+        // the states of the upper z faces: cells 4-7 below them, 28-31 above
+        if (lane >= 4 && lane < 8) {
+          side5<1>(qh, dq[2], qh);
+#pragma unroll
+          for (int v = 0; v < 5; ++v) sm.left[w][b][v][lane - 4] = qh[v];
+        } else if (lane >= 28) {
+          side5<-1>(qh, dq[2], qh);
+#pragma unroll
+          for (int v = 0; v < 5; ++v) sm.left[w][b][5 + v][lane - 28] = qh[v];
+        }
+      }
+      __syncwarp();
+      R qL[5], qR[5], F[5], sL[5], sR[5];
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const R* Q = sm.q[w][v];
-        const R cc = Q[c];
-        q0[v] = cc;
-        dqx[v] = limited(cc - Q[c - 1], Q[c + 1] - cc, prm.limiter);
-        dqy[v] = limited(cc - Q[c - 6], Q[c + 6] - cc, prm.limiter);
-        dqz[v] = limited(cc - Q[c - 36], Q[c + 36] - cc, prm.limiter);
+        qL[v] = sm.qh[w][v][eL];
+        qR[v] = sm.qh[w][v][eR];
+        sL[v] = sm.sl[w][fd][v][eL];
+        sR[v] = sm.sl[w][fd][v][eR];
       }
-      hancock(q0, dqx, dqy, dqz, gamma, hdt, qh);
+      side5<1>(qL, sL, qL);
+      side5<-1>(qR, sR, qR);
+      floor_max(qL, rf, pf);
+      floor_max(qR, rf, pf);
+      hllc_dyn(fd, qL, qR, gamma, igm1, F);
 #pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        sm.qh[w][v][lane] = qh[v];
-        sm.sl[w][0][v][lane] = dqx[v];
-        sm.sl[w][1][v][lane] = dqy[v];
-        sm.sl[w][2][v][lane] = dqz[v];
-      }
+      for (int v = 0; v < 5; ++v) sm.f[w][b][v][lane] = F[v];
+      __syncwarp();
     }
-    __syncwarp();
-    for (int fi = lane; fi < 36; fi += 32) {
-      const int d = fi / 12, m = fi % 12, s = m >> 2, a = m & 1, b = (m >> 1) & 1;
-      // face between cells at coordinate s-1 and s along d; (a, b) the transverse coordinates
-      int lx, ly, lz;
-      if (d == 0) { lx = s - 1; ly = a; lz = b; }
-      else if (d == 1) { lx = a; ly = s - 1; lz = b; }
-      else { lx = a; ly = b; lz = s - 1; }
-      const int eL = oct_eindex(lx, ly, lz);
-      const int eR = oct_eindex(lx + (d == 0), ly + (d == 1), lz + (d == 2));
+    // the upper z faces of the batch, four per group
+    if (lane < 4 * nb && (valid >> (lane >> 2) & 1)) {
+      const int b = lane >> 2, m = lane & 3;
       R qL[5], qR[5], F[5];
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        qL[v] = sm.qh[w][v][eL] + half_(sm.sl[w][d][v][eL]);
-        qR[v] = sm.qh[w][v][eR] - half_(sm.sl[w][d][v][eR]);
+        qL[v] = sm.left[w][b][v][m];
+        qR[v] = sm.left[w][b][5 + v][m];
       }
-      floor_state(qL, rf, pf);
-      floor_state(qR, rf, pf);
-      hllc_dyn(d, qL, qR, gamma, igm1, F);
+      floor_max(qL, rf, pf);
+      floor_max(qR, rf, pf);
+      hllc_dyn(dz, qL, qR, gamma, igm1, F);
 #pragma unroll
-      for (int v = 0; v < 5; ++v) sm.f[w][v][fi] = F[v];
+      for (int v = 0; v < 5; ++v) sm.f[w][b][v][32 + m] = F[v];
     }
     __syncwarp();
-    if (lane < 8) {
-      const int x = lane & 1, y = (lane >> 1) & 1, z = (lane >> 2) & 1;
-      const int c = (z + 2) * 36 + (y + 2) * 6 + (x + 2);
-      const int fxm = 0 * 12 + (x * 4 + y + 2 * z), fxp = fxm + 4;
-      const int fym = 1 * 12 + (y * 4 + x + 2 * z), fyp = fym + 4;
-      const int fzm = 2 * 12 + (z * 4 + x + 2 * y), fzp = fzm + 4;
+    // updates, one cell per lane
+    for (int u = lane; u < 8 * nb; u += 32) {
+      const int b = u >> 3, e = u & 7;
+      if (!(valid >> b & 1)) continue;
+      const int x = e & 1, y = (e >> 1) & 1, z = e >> 2;
+      const int fx = x * 4 + y + 2 * z, fy = 12 + y * 4 + x + 2 * z, fz = 24 + z * 4 + x + 2 * y;
+      R a[6][5], div[5];
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const R* F = sm.f[w][v];
-        const R div = ((F[fxp] - F[fxm]) + (F[fyp] - F[fym])) + (F[fzp] - F[fzm]);
-        gout[v][cur.out_cell(g, lane)] = Pol::update(__ldg(cur.f[v] + cur.cell(g, c)), dtdx, div);
+        const R* F = sm.f[w][b][v];
+        a[0][v] = F[fx + 4];
+        a[1][v] = F[fx];
+        a[2][v] = F[fy + 4];
+        a[3][v] = F[fy];
+        a[4][v] = F[fz + 4];
+        a[5][v] = F[fz];
       }
+#pragma unroll
+      for (int v = 0; v < 5; ++v) div[v] = ((a[0][v] - a[1][v]) + (a[2][v] - a[3][v])) + (a[4][v] - a[5][v]);
+      long long in, out;
+      src.own(g0 + b, e, in, out);
+#pragma unroll
+      for (int v = 0; v < 5; ++v) gout[v][out] = Pol::update(__ldg(src.f[v] + in), dtdx, div[v]);
     }
     __syncwarp();
   }
   flush_flags(flags, err);
 }
 
+// ------------------------------------------------------------------ cubes of octs
+// A run of 64 list entries that are the octs of a 4^3 cube in Morton order (found by find_oct_cubes) is
+// stepped as one box of 8^3 cells by one block: a listed oct on its own recovers 80 cells, predicts 32
+// and solves 36 faces for its 8 cells; the cube recovers 1376, predicts 896 and solves 1728 for its 512,
+// a third of the work per cell.  Every cell and face takes the operations of k_octs, so the same bits.
+// Four phases over shared memory: recover, predict (each cell's states at its faces), fluxes (in the
+// place of the recovered cells), updates.  256 threads and two blocks per SM in float arithmetic, 512
+// and one in 8-byte, whose scratch fills the SM.
+constexpr int kCubeN = 8, kCubeQ = 12;
+template <class R>
+constexpr int cube_threads() { return sizeof(R) >= 8 ? 512 : 256; }
+
+template <class R>
+struct CubeSmem {
+  R q[5][kCubeQ * kCubeQ * kCubeQ];  // recovered cells (stored at +2); then the fluxes, [axis][9][64]
+  R st[6][5][512];                   // states at the cells' low and high faces, 2 axis + high
+  R shell[6][5][64];                 // states toward the cube of the cells beyond its six sides
+  int ids[216];                      // octs of the 6^3 neighbourhood
+  static_assert(3 * 9 * 64 <= kCubeQ * kCubeQ * kCubeQ, "the fluxes fit in the place of the cells");
+};
+
+template <class Pol>
+__global__ void __launch_bounds__(cube_threads<typename Pol::R>(), sizeof(typename Pol::R) >= 8 ? 1 : 2)
+    k_oct_cubes(OctTable<typename Pol::S> src, typename Pol::S* o0, typename Pol::S* o1, typename Pol::S* o2,
+                typename Pol::S* o3, typename Pol::S* o4, OctCubes cubes, double dx, Params prm, const double* dt_dev,
+                unsigned* err) {
+  using S = typename Pol::S;
+  using R = typename Pol::R;
+  constexpr int NT = cube_threads<R>();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  auto& sm = *reinterpret_cast<CubeSmem<R>*>(smem_raw);
+  S* gout[5] = {o0, o1, o2, o3, o4};
+  const double dt = dt_dev[0];
+  if (!(dt > 0.0 && dt <= 1e300)) return;  // k_octs, launched after this kernel, raises the flag
+  const R hdt = (R)(0.5 * dt / dx);
+  const R dtdx = (R)(dt / dx);
+  const R gamma = kc<R>(prm, K_GAMMA), igm1 = kc<R>(prm, K_IGM1);
+  const R rf = kc<R>(prm, K_RHOF), pf = kc<R>(prm, K_PF);
+  const int tid = threadIdx.x, n = min(cubes.counts[0], cubes.max_cubes);
+  unsigned flags = 0;
+  for (int b = blockIdx.x; b < n; b += gridDim.x) {
+    const int* member = src.list + cubes.start[b];
+    __syncthreads();  // the previous cube's updates are done with the neighbourhood
+    for (int t = tid; t < 216; t += NT) sm.ids[t] = cube_oct(member, src.nbr, t);
+    __syncthreads();
+    // ---- recover: eight consecutive threads read an oct's eight cells
+    for (int t = tid; t < 1728; t += NT) {
+      const int o = t >> 3, e = t & 7;
+      const int x = 2 * (o % 6) + (e & 1) - 2, y = 2 * (o / 6 % 6) + ((e >> 1) & 1) - 2, z = 2 * (o / 36) + (e >> 2) - 2;
+      const int nout = (x < 0 || x > 7) + (y < 0 || y > 7) + (z < 0 || z > 7);
+      const bool far = x == -2 || x == 9 || y == -2 || y == 9 || z == -2 || z == 9;
+      if (nout > 2 || (nout == 2 && far)) continue;
+      const long long a = 8LL * sm.ids[o] + e;
+      S U[5];
+      R q[5];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) U[v] = __ldg(src.f[v] + a);
+      Pol::recover(U, prm, q, flags);
+      const int c = ((z + 2) * kCubeQ + y + 2) * kCubeQ + x + 2;
+#pragma unroll
+      for (int v = 0; v < 5; ++v) sm.q[v][c] = q[v];
+    }
+    __syncthreads();
+    // ---- predict: the 512 cells and the 384 beyond the six sides
+    for (int t = tid; t < 896; t += NT) {
+      const int f = (t - 512) >> 6, m = t & 63;  // side (t >= 512)
+      int x = t & 7, y = (t >> 3) & 7, z = t >> 6;
+      if (t >= 512) {
+        const int w = f & 1 ? 8 : -1, lo = m & 7, hi = m >> 3;
+        x = f < 2 ? w : lo;
+        y = f < 2 ? lo : (f < 4 ? w : hi);
+        z = f < 4 ? hi : w;
+      }
+      const int c = ((z + 2) * kCubeQ + y + 2) * kCubeQ + x + 2;
+      R q0[5], dq[3][5], qh[5];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) q0[v] = sm.q[v][c];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const int o = d == 0 ? 1 : (d == 1 ? kCubeQ : kCubeQ * kCubeQ);
+        R l[5], h[5];
+#pragma unroll
+        for (int v = 0; v < 5; ++v) {
+          l[v] = sm.q[v][c - o];
+          h[v] = sm.q[v][c + o];
+        }
+        sub5(q0, l, l);
+        sub5(h, q0, h);
+#pragma unroll
+        for (int v = 0; v < 5; ++v) dq[d][v] = limited_sel(l[v], h[v], prm.limiter);
+      }
+      hancock(q0, dq[0], dq[1], dq[2], gamma, hdt, qh);
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        R lo[5], hi[5];
+        keep5(dq[d], dq[d]);
+        side5<-1>(qh, dq[d], lo);
+        side5<1>(qh, dq[d], hi);
+        if (t < 512) {
+#pragma unroll
+          for (int v = 0; v < 5; ++v) {
+            sm.st[2 * d][v][t] = lo[v];
+            sm.st[2 * d + 1][v][t] = hi[v];
+          }
+        } else if (d == (f >> 1)) {
+#pragma unroll
+          for (int v = 0; v < 5; ++v) sm.shell[f][v][m] = f & 1 ? lo[v] : hi[v];
+        }
+      }
+    }
+    __syncthreads();
+    // ---- fluxes: face s (0 .. 8) of column m along axis d, between cells s - 1 and s
+    for (int t = tid; t < 1728; t += NT) {
+      const int d = t / 576, s = t / 64 % 9, m = t & 63, lo = m & 7, hi = m >> 3;
+      const int step = d == 0 ? 1 : (d == 1 ? 8 : 64);
+      const int c = s * step + (d == 0 ? 8 * lo + 64 * hi : (d == 1 ? lo + 64 * hi : m));  // cell s of the column
+      R qL[5], qR[5], F[5];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) {
+        qL[v] = s > 0 ? sm.st[2 * d + 1][v][c - step] : sm.shell[2 * d][v][m];
+        qR[v] = s < 8 ? sm.st[2 * d][v][c] : sm.shell[2 * d + 1][v][m];
+      }
+      floor_max(qL, rf, pf);
+      floor_max(qR, rf, pf);
+      hllc_dyn(d, qL, qR, gamma, igm1, F);
+#pragma unroll
+      for (int v = 0; v < 5; ++v) sm.q[v][t] = F[v];
+    }
+    __syncthreads();
+    // ---- updates, eight consecutive threads to an oct
+    for (int t = tid; t < 512; t += NT) {
+      const int o = t >> 3, e = t & 7;
+      const int x = 2 * (o & 3) + (e & 1), y = 2 * ((o >> 2) & 3) + ((e >> 1) & 1), z = 2 * (o >> 4) + (e >> 2);
+      const int fx = x * 64 + y + 8 * z, fy = 576 + y * 64 + x + 8 * z, fz = 1152 + z * 64 + x + 8 * y;
+      const long long a = 8LL * sm.ids[((o >> 4) + 1) * 36 + (((o >> 2) & 3) + 1) * 6 + (o & 3) + 1] + e;
+#pragma unroll
+      for (int v = 0; v < 5; ++v) {
+        const R* F = sm.q[v];
+        const R div = ((F[fx + 64] - F[fx]) + (F[fy + 64] - F[fy])) + (F[fz + 64] - F[fz]);
+        gout[v][a] = Pol::update(__ldg(src.f[v] + a), dtdx, div);
+      }
+    }
+  }
+  flush_flags(flags, err);
+}
+
 template <class Pol, class Src>
 cudaError_t launch_octs_src(const Src& src, void* const out[5], long long ngroups, double dx, const Params& prm,
-                            const double* dt, unsigned* err, cudaStream_t s) {
+                            const double* dt, unsigned* err, cudaStream_t s, const int* count = nullptr) {
   using S = typename Pol::S;
   const size_t smem = sizeof(OctSmem<Pol>);
   static PerDeviceOnce attr;
   cudaError_t e = attr.call(
       [&] { return cudaFuncSetAttribute(k_octs<Pol, Src>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); });
   if (e != cudaSuccess) return e;
-  long long blocks = (ngroups + kOctWarps - 1) / kOctWarps;
-  const long long cap = 152LL * 64;
-  if (blocks > cap) blocks = cap;
+  // groups per batch: full batches once every resident warp has one, fewer on a small list
+  const long long warps = 152LL * oct_min_blocks<Pol, Src>() * kOctWarps;
+  const int batch = (int)std::min<long long>(oct_batch<Pol>(), std::max<long long>(1, ngroups / warps));
+  const long long per_block = (long long)kOctWarps * batch;
+  const long long blocks = std::min((ngroups + per_block - 1) / per_block, 152LL * 64);
   k_octs<Pol, Src><<<(unsigned)blocks, 32 * kOctWarps, smem, s>>>(src, (S*)out[0], (S*)out[1], (S*)out[2], (S*)out[3],
-                                                                   (S*)out[4], ngroups, dx, prm, dt, err);
+                                                                   (S*)out[4], ngroups, count, batch, dx, prm, dt, err);
   return cudaGetLastError();
 }
 
@@ -459,7 +696,7 @@ cudaError_t launch_octs_level(const HostPatchIO& level, const int* origins, void
 template <class Pol>
 cudaError_t launch_octs_table(void* const in[5], const int* nbr, int noct, const int* list, void* const out[5],
                               long long ngroups, double dx, const Params& prm, const double* dt, unsigned* err,
-                              cudaStream_t s) {
+                              const OctCubes* cubes, cudaStream_t s) {
   using S = typename Pol::S;
   OctTable<S> src;
   for (int v = 0; v < 5; ++v) src.f[v] = static_cast<const S*>(in[v]);
@@ -467,7 +704,20 @@ cudaError_t launch_octs_table(void* const in[5], const int* nbr, int noct, const
   src.list = list;
   src.noct = noct;
   src.oct = 0;
-  return launch_octs_src<Pol>(src, out, ngroups, dx, prm, dt, err, s);
+  if (!cubes) return launch_octs_src<Pol>(src, out, ngroups, dx, prm, dt, err, s);
+  const size_t smem = sizeof(CubeSmem<typename Pol::R>);
+  static PerDeviceOnce attr;
+  cudaError_t e = attr.call([&] {
+    return cudaFuncSetAttribute(k_oct_cubes<Pol>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  });
+  if (e != cudaSuccess) return e;
+  const int blocks = (int)std::min<long long>(152 * (sizeof(typename Pol::R) >= 8 ? 1 : 2), ngroups / 64);
+  k_oct_cubes<Pol><<<blocks, cube_threads<typename Pol::R>(), smem, s>>>(
+      src, (S*)out[0], (S*)out[1], (S*)out[2], (S*)out[3], (S*)out[4], *cubes, dx, prm, dt, err);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  src.list = cubes->left;  // the octs outside the cubes
+  return launch_octs_src<Pol>(src, out, ngroups, dx, prm, dt, err, s, cubes->counts + 1);
 }
 
 // ------------------------------------------------------------------ primitive <-> conservative
@@ -632,7 +882,7 @@ __global__ void __launch_bounds__(256) k_box_fluxes(const HostBoxFluxes* boxes, 
       q_at(x - (e == 0), y - (e == 1), z - (e == 2), m);
       q_at(x + (e == 0), y + (e == 1), z + (e == 2), p);
 #pragma unroll
-      for (int v = 0; v < 5; ++v) dq[e][v] = limited(c[v] - m[v], p[v] - c[v], prm.limiter);
+      for (int v = 0; v < 5; ++v) dq[e][v] = limited_sel(c[v] - m[v], p[v] - c[v], prm.limiter);
     }
     hancock(c, dq[0], dq[1], dq[2], kc<R>(prm, K_GAMMA), hdt, qh);
 #pragma unroll

@@ -16,6 +16,7 @@
 #include <cuda_runtime.h>
 
 #include "internal.h"
+#include "oct_cube.cuh"
 
 namespace hydro {
 namespace {
@@ -156,7 +157,75 @@ __global__ void __launch_bounds__(864) k_oct_nbr(const int* pos, int noct, int3 
   nbr[27LL * i + n] = out;
 }
 
+// One warp per 32 list positions.  Each lane first compares its position's octs at the offsets 1, 2, 4
+// (the neighbours inside the first 2^3) and 8, 16, 32 (those of the next 2^3 cubes) with the table; the
+// few positions that agree are checked by the whole warp: the 216 octs of the neighbourhood are read
+// through the members, and every member's 27 entries must be the neighbourhood's, so that a step through
+// either gives the same values whatever the table holds.
+constexpr int kFindWarps = 4;
+__global__ void __launch_bounds__(32 * kFindWarps) k_find_cubes(const int* list, int ngroups, const int* nbr, int noct,
+                                                                OctCubes cubes) {
+  __shared__ int ids[kFindWarps][216];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int p = (blockIdx.x * kFindWarps + w) * 32 + lane;
+  auto beside = [&](int q, int entry, int r) {  // list[r] is list[q]'s neighbour `entry`
+    const int o = __ldg(list + q);
+    return (unsigned)o < (unsigned)noct && __ldg(nbr + 27LL * o + entry) == __ldg(list + r);
+  };
+  const bool maybe = p + 63 < ngroups && beside(p, 14, p + 1) && beside(p, 16, p + 2) && beside(p, 22, p + 4) &&
+                     beside(p + 1, 14, p + 8) && beside(p + 2, 16, p + 16) && beside(p + 4, 22, p + 32);
+  unsigned todo = __ballot_sync(0xffffffffu, maybe);
+  while (todo) {
+    const int b = p - lane + __ffs(todo) - 1;
+    todo &= todo - 1;
+    bool ok = (unsigned)__ldg(list + b + lane) < (unsigned)noct && (unsigned)__ldg(list + b + 32 + lane) < (unsigned)noct;
+    if (!__all_sync(0xffffffffu, ok)) continue;
+    for (int t = lane; t < 216; t += 32) {
+      const int o = cube_oct(list + b, nbr, t);
+      ids[w][t] = o;
+      ok = ok && (unsigned)o < (unsigned)noct;
+    }
+    __syncwarp();
+    // member m of the 4^3 (row-major), its entry n
+    for (int t = lane; t < 64 * 27 && ok; t += 32) {
+      const int m = t / 27, n = t - 27 * m, i = m & 3, j = (m >> 2) & 3, k = m >> 4;
+      const int o = ids[w][((k + 1) * 6 + j + 1) * 6 + i + 1];
+      ok = __ldg(nbr + 27LL * o + n) == ids[w][((k + n / 9) * 6 + j + n / 3 % 3) * 6 + i + n % 3];
+    }
+    ok = __all_sync(0xffffffffu, ok);
+    if (!ok) continue;
+    int at = 0;
+    if (lane == 0) at = atomicAdd(cubes.counts, 1);
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (at >= cubes.max_cubes) continue;
+    if (lane == 0) cubes.start[at] = b;
+    cubes.covered[b + lane] = 1;
+    cubes.covered[b + 32 + lane] = 1;
+  }
+}
+
+__global__ void __launch_bounds__(256) k_left_octs(const int* list, int ngroups, OctCubes cubes) {
+  const int p = blockIdx.x * 256 + threadIdx.x, lane = threadIdx.x & 31;
+  const bool left = p < ngroups && !cubes.covered[p];
+  const unsigned who = __ballot_sync(0xffffffffu, left);
+  int base = 0;
+  if (lane == 0 && who) base = atomicAdd(cubes.counts + 1, __popc(who));
+  base = __shfl_sync(0xffffffffu, base, 0);
+  if (left) cubes.left[base + __popc(who & ((1u << lane) - 1u))] = list[p];
+}
+
 }  // namespace
+
+cudaError_t find_oct_cubes(const int* list, long long ngroups, const int* nbr, int noct, const OctCubes& cubes,
+                           cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(cubes.counts, 0, 2 * sizeof(int), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(cubes.covered, 0, (size_t)ngroups, s);
+  if (e != cudaSuccess) return e;
+  const int n = (int)ngroups;
+  k_find_cubes<<<(n + 32 * kFindWarps - 1) / (32 * kFindWarps), 32 * kFindWarps, 0, s>>>(list, n, nbr, noct, cubes);
+  k_left_octs<<<(n + 255) / 256, 256, 0, s>>>(list, n, cubes);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_octs_build(const int* pos, int noct, const int dims[3], unsigned* bitmap, unsigned* word_prefix,
                               unsigned* block_prefix, size_t nwords, int* order, int* nbr, unsigned* err,
