@@ -1202,12 +1202,23 @@ int hydro_octs_build(hydro_ctx* c, const int* pos_dev, int noct, const int dims[
   }
   const size_t nwords = std::max<size_t>(1, ((size_t)1 << (3 * bits)) >> 5);
   const size_t nblocks = (nwords + 1023) / 1024;
-  int rc = ensure_device(&c->d_octs_scratch, &c->octs_scratch_cap, 2 * nwords + nblocks);
+  // Octs by key as well, where the key space is at most eight times the octs (a refined half of a level
+  // per axis): beyond, clearing it costs more than the table's rank lookups; nor does a first call under
+  // capture, or one without the memory, grow the scratch for it.
+  const size_t base = 2 * nwords + nblocks, with_slots = base + 32 * nwords;
+  bool slots = nbr_dev && 32 * nwords <= 8 * (size_t)noct;
+  if (slots && c->octs_scratch_cap < with_slots) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    slots = cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
+            ensure_device(&c->d_octs_scratch, &c->octs_scratch_cap, with_slots) == HYDRO_OK;
+    if (!slots) cudaGetLastError();
+  }
+  int rc = ensure_device(&c->d_octs_scratch, &c->octs_scratch_cap, base);
   if (rc) return rc;
   unsigned* bitmap = c->d_octs_scratch;
   c->launches += nbr_dev ? 5 : 4;
   return cuda_status(hydro::launch_octs_build(pos_dev, noct, dims, bitmap, bitmap + nwords, bitmap + 2 * nwords,
-                                              nwords, order_dev, nbr_dev, c->d_err, c->stream));
+                                              nwords, slots ? reinterpret_cast<int*>(bitmap + base) : nullptr, order_dev, nbr_dev, c->d_err, c->stream));
 }
 
 int hydro_step_octs_table(hydro_ctx* c, void* const in[5], void* const out[5], int noct, const int* nbr_dev,

@@ -170,9 +170,9 @@ cudaError_t launch_fill_ghosts(int elem_size, const HostGhostPatch* d_patches, c
 
 // Morton order and neighbour table of a level's octs (octs_build.cu).  Scratch: bitmap and
 // word_prefix of nwords words, block_prefix of (nwords + 1023) / 1024 words; nwords = max(1, 8^b / 32)
-// for keys below 8^b.
+// for keys below 8^b.  slot: nullptr, or 32 nwords ints for the octs' indices by key.
 cudaError_t launch_octs_build(const int* pos, int noct, const int dims[3], unsigned* bitmap, unsigned* word_prefix,
-                              unsigned* block_prefix, size_t nwords, int* order, int* nbr, unsigned* err,
+                              unsigned* block_prefix, size_t nwords, int* slot, int* order, int* nbr, unsigned* err,
                               cudaStream_t s);
 
 // Finds the runs of 64 list entries that are a 4^3 cube of octs in Morton order and whose 27 neighbour

@@ -319,14 +319,21 @@ __global__ void __launch_bounds__(32 * kOctWarps, (oct_min_blocks<Pol, Src>())) 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   auto& sm = *reinterpret_cast<OctSmem<Pol>*>(smem_raw);
   S* gout[5] = {o0, o1, o2, o3, o4};
-  if (count) ngroups = *count;  // groups left by the cube kernel
+  if (count) {  // groups left by the cube kernel: often none, and then only block 0 stays, to check dt
+    ngroups = *count;
+    if (blockIdx.x > 0 && (long long)blockIdx.x * kOctWarps * batch >= ngroups) return;
+  }
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (threadIdx.x == 0) {
+  // needed cells numbered in stencil order: a ballot per 32 cells, the first warp's lanes together
+  if (threadIdx.x < 32) {
     int n = 0;
-    for (int c = 0; c < 216; ++c) {
-      const int x = c % 6 - 2, y = (c / 6) % 6 - 2, z = c / 36 - 2;
-      sm.at[c] = (short)n;
-      if (oct_needed(x, y, z)) sm.need[n++] = (short)c;
+    for (int c = lane; c < 224; c += 32) {
+      const bool needed = c < 216 && oct_needed(c % 6 - 2, (c / 6) % 6 - 2, c / 36 - 2);
+      const unsigned who = __ballot_sync(0xffffffffu, needed);
+      const int k = n + __popc(who & ((1u << lane) - 1u));
+      if (c < 216) sm.at[c] = (short)k;
+      if (needed) sm.need[k] = (short)c;
+      n += __popc(who);
     }
   }
   __syncthreads();
@@ -512,11 +519,11 @@ __global__ void __launch_bounds__(32 * kOctWarps, (oct_min_blocks<Pol, Src>())) 
 // and solves 36 faces for its 8 cells; the cube recovers 1376, predicts 896 and solves 1728 for its 512,
 // a third of the work per cell.  Every cell and face takes the operations of k_octs, so the same bits.
 // Four phases over shared memory: recover, predict (each cell's states at its faces), fluxes (in the
-// place of the recovered cells), updates.  256 threads and two blocks per SM in float arithmetic, 512
-// and one in 8-byte, whose scratch fills the SM.
-constexpr int kCubeN = 8, kCubeQ = 12;
-template <class R>
-constexpr int cube_threads() { return sizeof(R) >= 8 ? 512 : 256; }
+// place of the recovered cells), updates.  512 threads; two blocks per SM in float arithmetic, one in
+// 8-byte, whose scratch fills the SM (2097152 octs, mixed, order and table built too: 1.96 ms, 2.09 with
+// 256 threads, 2.04 with 384).
+constexpr int kCubeThreads = 512;
+constexpr int kCubeQ = 12;  // cells per axis with the two beyond each side
 
 template <class R>
 struct CubeSmem {
@@ -528,13 +535,13 @@ struct CubeSmem {
 };
 
 template <class Pol>
-__global__ void __launch_bounds__(cube_threads<typename Pol::R>(), sizeof(typename Pol::R) >= 8 ? 1 : 2)
+__global__ void __launch_bounds__(kCubeThreads, sizeof(typename Pol::R) >= 8 ? 1 : 2)
     k_oct_cubes(OctTable<typename Pol::S> src, typename Pol::S* o0, typename Pol::S* o1, typename Pol::S* o2,
                 typename Pol::S* o3, typename Pol::S* o4, OctCubes cubes, double dx, Params prm, const double* dt_dev,
                 unsigned* err) {
   using S = typename Pol::S;
   using R = typename Pol::R;
-  constexpr int NT = cube_threads<R>();
+  constexpr int NT = kCubeThreads;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   auto& sm = *reinterpret_cast<CubeSmem<R>*>(smem_raw);
   S* gout[5] = {o0, o1, o2, o3, o4};
@@ -712,7 +719,7 @@ cudaError_t launch_octs_table(void* const in[5], const int* nbr, int noct, const
   });
   if (e != cudaSuccess) return e;
   const int blocks = (int)std::min<long long>(152 * (sizeof(typename Pol::R) >= 8 ? 1 : 2), ngroups / 64);
-  k_oct_cubes<Pol><<<blocks, cube_threads<typename Pol::R>(), smem, s>>>(
+  k_oct_cubes<Pol><<<blocks, kCubeThreads, smem, s>>>(
       src, (S*)out[0], (S*)out[1], (S*)out[2], (S*)out[3], (S*)out[4], *cubes, dx, prm, dt, err);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
