@@ -404,19 +404,24 @@ __device__ __forceinline__ void hllc_core(const R qL[5], const R qR[5], bool zn,
   F[4] = ue * (Ee + pe);
 }
 
+// S* - u_L (the reverse step forms its S* with it too, and selects the same branches).
+__device__ __forceinline__ double contact_offset(const double qL[5], const double qR[5], double mR, double du,
+                                                 double den) {
+  return div_(fma(mR, du, qR[4] - qL[4]), den);
+}
 // The same flux in double, in the form of the double-float one below (S* from its distance to u_L, the
 // star energy without 1/m_K): about 75 operations on the FP64 pipe, the generic form with IEEE
 // divisions and roots about 120.
 __device__ __forceinline__ void hllc_core(const double qL[5], const double qR[5], bool, double gamma, double inv_gm1,
                                           double F[5]) {
-  const double cL = rsqrt_(div_(gamma * qL[4], qL[0])), cR = rsqrt_(div_(gamma * qR[4], qR[0]));
+  const double cL = rsqrt_(gamma * qL[4] * rcp_(qL[0])), cR = rsqrt_(gamma * qR[4] * rcp_(qR[0]));
   const double uL = qL[1], uR = qR[1];
   const double aL = uL - cL, bL = uR - cR, aR = uL + cL, bR = uR + cR;
   const double SL = aL <= bL ? aL : bL, SR = aR >= bR ? aR : bR;
   const double dL = SL - uL, dR = SR - uR;
   const double mL = qL[0] * dL, mR = qR[0] * dR;
   const double du = uL - uR;
-  const double dl = div_(fma(mR, du, qR[4] - qL[4]), mL - mR);  // S* - u_L
+  const double dl = contact_offset(qL, qR, mR, du, mL - mR);  // S* - u_L
   const double Ss = uL + dl;
   const bool SLneg = cmp_neg(SL), SRpos = cmp_pos(SR);
   const bool star = SLneg && SRpos;

@@ -13,8 +13,9 @@
 // The rest is the PLM step with the parabola's centre slope D in the Hancock predictor and face
 // states q_h + (qR - q), q_h + (qL - q) in place of q_h +- dq/2.  The stencil radius is 3.
 //
-// Kernel layout: one thread per column of a TX x TY tile marching up z (as the PLM kernel), on a
-// periodic box (indices wrapped) or on a patch carrying three ghost layers filled by the caller.
+// Kernel layout in float arithmetic: one thread per column of a TX x TY tile marching up z (as the PLM
+// kernel), on a periodic box (indices wrapped) or on a patch carrying three ghost layers filled by the
+// caller; 8-byte arithmetic splits each plane's work over 512 threads (PpmWideShared, below).
 // Shared memory holds a ring of five recovered planes (p-2 .. p+2) over the tile and three halo
 // cells each side, the x- and y-face states of plane p (the tile's cells and one ring cell beyond
 // each edge) and the x and y fluxes of plane p.  The z reconstruction of a column reads its own
@@ -143,8 +144,8 @@ __device__ __forceinline__ void ppm_edges5(const df a[5], const df b[5], const d
 
 // Edge distances of tile cell (i, j) of the middle plane along axis d (0 x, 1 y, 2 z); q: the cell's
 // own values.  sl: ring slots of planes p-2 .. p+2.
-template <class R, int TX, int TY>
-__device__ __forceinline__ void ppm_axis(const PpmShared<R, TX, TY>& sm, const int sl[5], int i, int j, int d,
+template <class R, class Sh>
+__device__ __forceinline__ void ppm_axis(const Sh& sm, const int sl[5], int i, int j, int d,
                                          const R q[5], R sixth, R l[5], R r[5], R D[5]) {
   const int X = i + kPpmHalo, Y = j + kPpmHalo, dx = d == 0, dy = d == 1;
   R a[5], b[5], e[5], f[5];
@@ -166,48 +167,13 @@ __device__ __forceinline__ void ppm_cell(const PpmShared<R, TX, TY>& sm, const i
   hancock(q, D[0], D[1], D[2], gamma, hdt, qh);
 }
 
-// The same reconstruction and prediction with the three axes in a loop, for double-float arithmetic,
-// whose inlined edge reconstructions would overflow the instruction cache: one copy of the five
-// reconstructions serves all axes, the Hancock terms are summed axis by axis, and the edge distances
-// go where the caller wants them: out(d, l, r) for axis d.
-template <int TX, int TY, class Out>
-__device__ __forceinline__ void ppm_cell_axes(const PpmShared<df, TX, TY>& sm, const int sl[5], int i, int j,
-                                              const df& gamma, const df& hdt, const df& sixth, df qh[5], Out out) {
-  df q[5];
-  sm.q[sl[2]].ld(j + kPpmHalo, i + kPpmHalo, q);
-  const df ir = rcpu_(q[0]);
-  const df gp = prod_(gamma, q[4]);
-  const df none(0.f, 0.f);
-  df2 ta = both_(none), tb = ta;
-  df tc = none;
-#pragma unroll 1
-  for (int d = 0; d < 3; ++d) {
-    df l[5], r[5], D[5];
-    ppm_axis(sm, sl, i, j, d, q, sixth, l, r, D);
-    out(d, l, r);
-    // Hancock terms of axis d (normal velocity q[1 + d]), as in hancock()
-    const df un = d == 0 ? q[1] : (d == 1 ? q[2] : q[3]);
-    const df Dn = d == 0 ? D[1] : (d == 1 ? D[2] : D[3]);
-    const df2 u2 = both_(un);
-    ta = sum_(ta, sum_(prod_(u2, pair_(D[0], D[1])), prod_(pair_(q[0], d == 0 ? ir : none), pair_(Dn, D[4]))));
-    tb = sum_(tb, sum_(prod_(u2, pair_(D[2], D[3])), prod_(pair_(d == 1 ? ir : none, d == 2 ? ir : none), both_(D[4]))));
-    tc = sum_(tc, sum_(prod_(un, D[4]), prod_(gp, Dn)));
-  }
-  const df2 nh = neg_(both_(hdt)), qa = pair_(q[0], q[1]) + prod_(nh, ta), qb = pair_(q[2], q[3]) + prod_(nh, tb);
-  qh[0] = first_(qa);
-  qh[1] = second_(qa);
-  qh[2] = first_(qb);
-  qh[3] = second_(qb);
-  qh[4] = q[4] + prod_(-hdt, tc);
-}
-
 // Resident blocks per SM: the 8-byte ring and face arrays take ~165 KB of shared memory.
 template <class Pol>
 constexpr int ppm_min_blocks() { return sizeof(typename Pol::R) >= 8 ? 1 : 2; }
 
 // Block-wide maximum of v (all threads call); the result is valid in thread 0.
-template <class R, int TX, int TY>
-__device__ __forceinline__ R ppm_block_max(PpmShared<R, TX, TY>& sm, R v) {
+template <class R, class Sh>
+__device__ __forceinline__ R ppm_block_max(Sh& sm, R v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     R w = shfl_xor_(v, o);
@@ -217,7 +183,7 @@ __device__ __forceinline__ R ppm_block_max(PpmShared<R, TX, TY>& sm, R v) {
   if ((threadIdx.x & 31) == 0) sm.red[threadIdx.x >> 5] = v;
   __syncthreads();
   if (threadIdx.x == 0)
-    for (int w = 1; w < TX * TY / 32; ++w) v = sm.red[w] > v ? sm.red[w] : v;
+    for (int w = 1; w < (int)(blockDim.x / 32); ++w) v = sm.red[w] > v ? sm.red[w] : v;
   return v;
 }
 
@@ -231,7 +197,6 @@ __device__ __forceinline__ void ppm_tile(PpmShared<typename Pol::R, TX, TY>& sm,
   using S = typename Pol::S;
   using R = typename Pol::R;
   constexpr int QX = TX + 2 * kPpmHalo, QY = TY + 2 * kPpmHalo, NT = TX * TY;
-  constexpr bool kCompactPpm = std::is_same<R, df>::value;  // double-float arithmetic
   const int tid = threadIdx.x;
   const bool periodic = P.gin == 0;
   __syncthreads();  // the previous tile's last reads of the index tables are done
@@ -272,20 +237,6 @@ __device__ __forceinline__ void ppm_tile(PpmShared<typename Pol::R, TX, TY>& sm,
   else if (tid < 2 * TY) { rk = 1; ri = TX; rj = tid - TY; }
   else if (tid < 2 * TY + TX) { rk = 2; ri = tid - 2 * TY; rj = -1; }
   else if (tid < 2 * TY + 2 * TX) { rk = 3; ri = tid - 2 * TY - TX; rj = TY; }
-
-  // Split barriers (ids 1-3), in double-float arithmetic, whose block is alone on its SM: the
-  // ring cells belong to the first NR threads, whole warps, which signal barrier 1 once their tile
-  // cells are predicted, predict the ring, signal barrier 3 and take the faces between ring and
-  // tile after barrier 2; the other warps wait for every tile cell (barrier 1), signal barrier 2,
-  // take the faces between two tile cells and, once the ring cells no longer read plane p-2
-  // (barrier 3), load plane p+3 into its slot.  The ring cells' full reconstructions then overlap
-  // the interior faces instead of holding the other warps at one block barrier (+4.5% at 512^3).
-  // Float arithmetic keeps one block barrier per phase: with two resident blocks the other block
-  // fills the waits, and the split (FP32 -6.5%, the batched mixed step -5%) or one call site for
-  // the tile and ring reconstructions (FP32 -10%) cost more.
-  constexpr int NR = 2 * (TX + TY), NIX = (TX - 1) * TY, NIF = NIX + TX * (TY - 1);
-  constexpr bool kSplit = kCompactPpm && NR % 32 == 0 && NR < NT;
-  const bool ringw = tid < NR;
 
   R zhi[5], fzb[5], dxy[5];  // z-high face state, z flux below, x/y flux difference: plane p-1
 #pragma unroll
@@ -341,67 +292,7 @@ __device__ __forceinline__ void ppm_tile(PpmShared<typename Pol::R, TX, TY>& sm,
 #pragma unroll
       for (int v = 0; v < 5; ++v) zhi[v] = znew[v];
     };
-    if constexpr (kCompactPpm) {
-      // double-float: the tile cell (it 0) and this thread's ring cell (it 1) through one inlined
-      // copy of the reconstruction; the x/y edge offsets are stored and completed with qh after it
-      for (int it = 0; it < 2; ++it) {
-        if (it == 1 && !(xy && rk >= 0)) break;
-        const int ci = it == 0 ? i : ri, cj = it == 0 ? j : rj;
-        R qh[5];
-        ppm_cell_axes(sm, sl, ci, cj, gamma, hdt, sixth, qh, [&](int d, const R l[5], const R r[5]) {
-          if (it == 0) {
-            if (d == 2) {
-#pragma unroll
-              for (int v = 0; v < 5; ++v) {
-                zlo[v] = l[v];
-                znew[v] = r[v];
-              }
-            } else if (xy && d == 0) {
-              sm.wx[0].st(j, i + 1, l);
-              sm.wx[1].st(j, i + 1, r);
-            } else if (xy) {
-              sm.wy[0].st(j + 1, i, l);
-              sm.wy[1].st(j + 1, i, r);
-            }
-          } else if (d == (rk >> 1)) {
-            if (rk == 0) sm.wx[1].st(rj, 0, r);
-            else if (rk == 1) sm.wx[0].st(rj, TX + 1, l);
-            else if (rk == 2) sm.wy[1].st(0, ri, r);
-            else sm.wy[0].st(TY + 1, ri, l);
-          }
-        });
-        // the edge distances stored above become face states, q_h - l and q_h + r
-        auto low = [&](auto& w, int y, int x) {
-          R t[5];
-          w.ld(y, x, t);
-          sub5(qh, t, t);
-          w.st(y, x, t);
-        };
-        auto high = [&](auto& w, int y, int x) {
-          R t[5];
-          w.ld(y, x, t);
-          add5(qh, t, t);
-          w.st(y, x, t);
-        };
-        if (it == 0) {
-          sub5(qh, zlo, zlo);
-          add5(qh, znew, znew);
-          if (xy) {
-            low(sm.wx[0], j, i + 1);
-            high(sm.wx[1], j, i + 1);
-            low(sm.wy[0], j + 1, i);
-            high(sm.wy[1], j + 1, i);
-          }
-        } else if (rk == 0) high(sm.wx[1], rj, 0);
-        else if (rk == 1) low(sm.wx[0], rj, TX + 1);
-        else if (rk == 2) high(sm.wy[1], 0, ri);
-        else low(sm.wy[0], TY + 1, ri);
-        if (it == 0) {
-          zface_update();
-          if (kSplit && xy && ringw) bar_arrive(1, NT);
-        }
-      }
-    } else {
+    {
       R l[3][5], r[3][5], qh[5];
       ppm_cell(sm, sl, i, j, gamma, hdt, sixth, l, r, qh);
       sub5(qh, l[2], zlo);
@@ -417,7 +308,7 @@ __device__ __forceinline__ void ppm_tile(PpmShared<typename Pol::R, TX, TY>& sm,
         sm.wy[1].st(j + 1, i, r[1]);
       }
     }
-    if (!kCompactPpm && xy && rk >= 0) {
+    if (xy && rk >= 0) {
       R l[3][5], r[3][5], qh[5], w[5];
       ppm_cell(sm, sl, ri, rj, gamma, hdt, sixth, l, r, qh);
 #pragma unroll
@@ -428,75 +319,9 @@ __device__ __forceinline__ void ppm_tile(PpmShared<typename Pol::R, TX, TY>& sm,
       else if (rk == 2) sm.wy[1].st(0, ri, w);
       else sm.wy[0].st(TY + 1, ri, w);
     }
-    if constexpr (!kCompactPpm) zface_update();
-    if (kSplit && xy) {
-      if (ringw) {
-        bar_arrive(3, NT);
-        bar_sync(2, NT);
-      } else {
-        bar_sync(1, NT);
-        bar_arrive(2, NT);
-      }
-      // faces f < NIF between two tile cells (x, then y) by the other warps; face NIF + tid
-      // between this thread's ring cell and the tile by a ring thread; one HLLC call site
-      const int fend = ringw ? NIF + tid + 1 : NIF;
-      for (int f = ringw ? NIF + tid : tid - NR; f < fend; f += NT - NR) {
-        int d, fx, fy;
-        if (f < NIX) {
-          d = 0; fy = f / (TX - 1); fx = f - fy * (TX - 1) + 1;
-        } else if (f < NIF) {
-          const int g = f - NIX;
-          d = 1; fy = g / TX; fx = g - fy * TX; fy += 1;
-        } else if (rk == 0) { d = 0; fx = 0; fy = rj; }
-        else if (rk == 1) { d = 0; fx = TX; fy = rj; }
-        else if (rk == 2) { d = 1; fx = ri; fy = 0; }
-        else { d = 1; fx = ri; fy = TY; }
-        R ql[5], qr[5], F[5];
-        if (d == 0) {
-          sm.wx[1].ld(fy, fx, ql);
-          sm.wx[0].ld(fy, fx + 1, qr);
-        } else {
-          sm.wy[1].ld(fy, fx, ql);
-          sm.wy[0].ld(fy + 1, fx, qr);
-        }
-        floor_max(ql, rf, pf);
-        floor_max(qr, rf, pf);
-        hllc_dyn(d, ql, qr, gamma, igm1, F);
-        if (d == 0) sm.fx.st(fy, fx, F);
-        else sm.fy.st(fy, fx, F);
-      }
-      if (!ringw) {
-        bar_sync(3, NT);
-        load_plane(p + kPpmHalo, sl[0], tid - NR, NT - NR);  // (p < z1 on an x/y plane)
-      }
-      __syncthreads();  // fluxes and plane p+3 in place
-      if (xy) xy_div();
-      continue;
-    }
+    zface_update();
     __syncthreads();  // face states written; ring slot of plane p-2 free
-    if (kCompactPpm && xy) {
-      // double-float: x and y faces through one inlined copy of HLLC (runtime normal)
-      constexpr int NXF = (TX + 1) * TY;
-      for (int f = tid; f < NXF + TX * (TY + 1); f += NT) {
-        const int d = f < NXF ? 0 : 1;
-        const int g = d == 0 ? f : f - NXF;
-        const int w = d == 0 ? TX + 1 : TX;
-        const int fy = g / w, fx = g - fy * w;
-        R ql[5], qr[5], F[5];
-        if (d == 0) {
-          sm.wx[1].ld(fy, fx, ql);
-          sm.wx[0].ld(fy, fx + 1, qr);
-        } else {
-          sm.wy[1].ld(fy, fx, ql);
-          sm.wy[0].ld(fy + 1, fx, qr);
-        }
-        floor_max(ql, rf, pf);
-        floor_max(qr, rf, pf);
-        hllc_dyn(d, ql, qr, gamma, igm1, F);
-        if (d == 0) sm.fx.st(fy, fx, F);
-        else sm.fy.st(fy, fx, F);
-      }
-    } else if (xy) {
+    if (xy) {
       for (int f = tid; f < (TX + 1) * TY; f += NT) {
         const int fy = f / (TX + 1), fx = f - fy * (TX + 1);
         R ql[5], qr[5], F[5];
@@ -524,14 +349,246 @@ __device__ __forceinline__ void ppm_tile(PpmShared<typename Pol::R, TX, TY>& sm,
   }
 }
 
+// ------------------------------------------------------------------ 8-byte tile
+// Double-float and double run the same tile with 512 threads.  One thread per column left 8 warps per SM
+// (the five-plane ring fills the SM's shared memory) with ~11000 dependent instructions each per plane:
+// the double-float kernel waited on latencies at 36% of its issue slots.  Here a plane takes three phases between block
+// barriers, and the first two split a cell's work:
+//   A  the edge reconstructions, one (cell, axis) per thread: 768 of the tile's cells and, where plane
+//      p's x and y faces are needed, 192 of the ring's; edge distances to shared memory
+//   B  the first 256 threads: predictor, face states, z face p - 1/2 and the update of plane p - 1;
+//      the others: the ring cells' predictor and face states, and the load of plane p + 3 into the
+//      slot of plane p - 2
+//   C  the 544 x and y faces
+// 191x203x187 double-float step: 7.7 -> 4.0 ms; 96^3 double (FP64 pipe): 2.83 -> 2.46 ms.
+template <class R, int TX, int TY>
+struct PpmWideShared {
+  static constexpr int QX = TX + 2 * kPpmHalo, QY = TY + 2 * kPpmHalo;
+  Plane5<R, QY, QX> q[5];       // ring of recovered planes
+  Plane5<R, TY, TX + 2> wx[2];  // x faces: [low/high] edge distances, then states, at (y, x + 1)
+  Plane5<R, TY + 2, TX> wy[2];  // y faces, at (y + 1, x)
+  Plane5<R, TY, TX> wz[2];      // z edge distances of the tile's cells
+  Plane5<R, 3, 2 * (TX + TY)> slope;  // the ring cells' centre slopes, [axis][ring cell]
+  Plane5<R, TY, TX + 1> fx;
+  Plane5<R, TY + 1, TX> fy;
+  int sx[QX], sy[QY];
+  R red[2 * TX * TY / 32];
+  int tile;
+};
+
+template <class Pol, int TX, int TY>
+__device__ __forceinline__ void ppm_tile(PpmWideShared<typename Pol::R, TX, TY>& sm, const PatchIO<double>& P, int x0,
+                                         int y0, int z0, int z1, const Params& prm, double dtv, bool want_cfl,
+                                         unsigned& flags, typename Pol::R& smax) {
+  using R = typename Pol::R;
+  constexpr int QX = TX + 2 * kPpmHalo, QY = TY + 2 * kPpmHalo, NC = TX * TY, NT = 2 * NC, NR = 2 * (TX + TY);
+  static_assert(NC % 32 == 0 && NR % 32 == 0 && NR <= NC, "whole warps per axis and per role");
+  const int tid = threadIdx.x;
+  const bool periodic = P.gin == 0;
+  __syncthreads();  // the previous tile's last reads of the index tables are done
+  for (int k = tid; k < QX; k += NT)
+    sm.sx[k] = periodic ? wrap_index(x0 + k - kPpmHalo, P.nx) : min(x0 + k - kPpmHalo + P.gin, P.nx + 2 * P.gin - 1);
+  for (int k = tid; k < QY; k += NT)
+    sm.sy[k] = periodic ? wrap_index(y0 + k - kPpmHalo, P.ny) : min(y0 + k - kPpmHalo + P.gin, P.ny + 2 * P.gin - 1);
+  __syncthreads();
+  const R gamma = kc<R>(prm, K_GAMMA), igm1 = kc<R>(prm, K_IGM1), sixth = kc<R>(prm, K_SIXTH);
+  const R rf = kc<R>(prm, K_RHOF), pf = kc<R>(prm, K_PF);
+  const R hdt = (R)(0.5 * dtv / P.dx);
+  const R dtdx = (R)(dtv / P.dx);
+  auto load_plane = [&](int z, int s, int first, int stride) {
+    const long long zo = (long long)(periodic ? wrap_index(z, P.nz) : z + P.gin) * P.isz;
+    for (int c = first; c < QX * QY; c += stride) {
+      const int y = c / QX, x = c - y * QX;
+      const long long a = zo + (long long)sm.sy[y] * P.isy + sm.sx[x];
+      double U[5];
+      R q[5];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) U[v] = __ldg(P.in[v] + a);
+      Pol::recover(U, prm, q, flags);
+      sm.q[s].st(y, x, q);
+    }
+  };
+  // ring cell r: x-low, x-high, y-low, y-high sides in turn
+  auto ring_cell = [&](int r, int& side, int& i, int& j) {
+    if (r < TY) { side = 0; i = -1; j = r; }
+    else if (r < 2 * TY) { side = 1; i = TX; j = r - TY; }
+    else if (r < 2 * TY + TX) { side = 2; i = r - 2 * TY; j = -1; }
+    else { side = 3; i = r - 2 * TY - TX; j = TY; }
+  };
+  for (int k = 0; k < 5; ++k) load_plane(z0 - kPpmHalo + k, k, tid, NT);  // slot of plane z: (z - z0 + 3) mod 5
+  __syncthreads();
+
+  const int i = tid % TX, j = (tid % NC) / TX;  // column of the first NC threads
+  const bool column = tid < NC, own = column && x0 + i < P.nx && y0 + j < P.ny;
+  R zhi[5], fzb[5];  // z-high face state of plane p-1 and z flux below it
+#pragma unroll
+  for (int v = 0; v < 5; ++v) zhi[v] = fzb[v] = R(0);
+  for (int p = z0 - 1; p <= z1; ++p) {
+    const int base = p - z0 + 1;
+    int sl[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) sl[k] = (base + k) % 5;
+    const bool xy = p >= z0 && p < z1;  // plane p is updated: its x and y faces are needed
+    // ---- A
+    for (int t = tid; t < 3 * (xy ? NC + NR : NC); t += NT) {
+      const bool ring = t >= 3 * NC;
+      const int d = ring ? (t - 3 * NC) / NR : t / NC, c = ring ? (t - 3 * NC) % NR : t % NC;
+      int ci = c % TX, cj = c / TX, side = 0;
+      if (ring) ring_cell(c, side, ci, cj);
+      R q[5], l[5], r[5], D[5];
+      sm.q[sl[2]].ld(cj + kPpmHalo, ci + kPpmHalo, q);
+      ppm_axis(sm, sl, ci, cj, d, q, sixth, l, r, D);
+      if (ring) {
+        sm.slope.st(d, c, D);
+        if (d == (side >> 1)) {
+          if (side == 0) sm.wx[1].st(cj, 0, r);
+          else if (side == 1) sm.wx[0].st(cj, TX + 1, l);
+          else if (side == 2) sm.wy[1].st(0, ci, r);
+          else sm.wy[0].st(TY + 1, ci, l);
+        }
+      } else if (d == 0) {
+        sm.wx[0].st(cj, ci + 1, l);
+        sm.wx[1].st(cj, ci + 1, r);
+      } else if (d == 1) {
+        sm.wy[0].st(cj + 1, ci, l);
+        sm.wy[1].st(cj + 1, ci, r);
+      } else {
+        sm.wz[0].st(cj, ci, l);
+        sm.wz[1].st(cj, ci, r);
+      }
+    }
+    __syncthreads();
+    // ---- B
+    auto low = [&](const R qh[5], auto& w, int y, int x) {  // edge distance -> face state
+      R t[5];
+      w.ld(y, x, t);
+      sub5(qh, t, t);
+      w.st(y, x, t);
+    };
+    auto high = [&](const R qh[5], auto& w, int y, int x) {
+      R t[5];
+      w.ld(y, x, t);
+      add5(qh, t, t);
+      w.st(y, x, t);
+    };
+    if (column) {
+      R q[5], D[3][5], l[5], qh[5];
+      sm.q[sl[2]].ld(j + kPpmHalo, i + kPpmHalo, q);
+      sm.wx[0].ld(j, i + 1, l);
+      sm.wx[1].ld(j, i + 1, D[0]);
+      add5(l, D[0], D[0]);
+      sm.wy[0].ld(j + 1, i, l);
+      sm.wy[1].ld(j + 1, i, D[1]);
+      add5(l, D[1], D[1]);
+      sm.wz[0].ld(j, i, l);
+      sm.wz[1].ld(j, i, D[2]);
+      add5(l, D[2], D[2]);
+      hancock(q, D[0], D[1], D[2], gamma, hdt, qh);
+      if (xy) {
+        low(qh, sm.wx[0], j, i + 1);
+        high(qh, sm.wx[1], j, i + 1);
+        low(qh, sm.wy[0], j + 1, i);
+        high(qh, sm.wy[1], j + 1, i);
+      }
+      R zlo[5], znew[5];
+      sm.wz[0].ld(j, i, zlo);
+      sm.wz[1].ld(j, i, znew);
+      sub5(qh, zlo, zlo);
+      add5(qh, znew, znew);
+      if (p > z0 - 1) {
+        R F[5];
+        floor_max(zhi, rf, pf);
+        floor_max(zlo, rf, pf);
+        hllc<2>(zhi, zlo, gamma, igm1, F);
+        if (p > z0) {
+          R xp[5], xm[5], yp[5], ym[5], div[5];  // plane p-1's x and y fluxes
+          sm.fx.ld(j, i + 1, xp);
+          sm.fx.ld(j, i, xm);
+          sm.fy.ld(j + 1, i, yp);
+          sm.fy.ld(j, i, ym);
+          div_xy(xp, xm, yp, ym, div);
+          sub5(F, fzb, xp);
+          add5(div, xp, div);
+          if (own) {
+            const int z = p - 1;
+            const long long ai = (long long)(z + P.gin) * P.isz + (long long)(y0 + j + P.gin) * P.isy + (x0 + i + P.gin);
+            const long long ao = (long long)(z + P.gout) * P.osz + (long long)(y0 + j + P.gout) * P.osy + (x0 + i + P.gout);
+            double Un[5];
+#pragma unroll
+            for (int v = 0; v < 5; ++v) {
+              Un[v] = Pol::update(__ldg(P.in[v] + ai), dtdx, div[v]);
+              P.out[v][ao] = Un[v];
+            }
+            if (want_cfl) {
+              const R sp = Pol::speed(Un, prm, flags);
+              smax = sp > smax ? sp : smax;
+            }
+          }
+        }
+#pragma unroll
+        for (int v = 0; v < 5; ++v) fzb[v] = F[v];
+      }
+#pragma unroll
+      for (int v = 0; v < 5; ++v) zhi[v] = znew[v];
+    } else {
+      const int u = tid - NC;
+      if (xy && u < NR) {
+        int side, ci, cj;
+        ring_cell(u, side, ci, cj);
+        R q[5], D[3][5], qh[5];
+        sm.q[sl[2]].ld(cj + kPpmHalo, ci + kPpmHalo, q);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) sm.slope.ld(d, u, D[d]);
+        hancock(q, D[0], D[1], D[2], gamma, hdt, qh);
+        if (side == 0) high(qh, sm.wx[1], cj, 0);
+        else if (side == 1) low(qh, sm.wx[0], cj, TX + 1);
+        else if (side == 2) high(qh, sm.wy[1], 0, ci);
+        else low(qh, sm.wy[0], TY + 1, ci);
+      }
+      // the threads without a ring cell come first, where some take a cell more
+      if (p < z1) load_plane(p + kPpmHalo, sl[0], NC - 1 - u, NC);
+    }
+    __syncthreads();
+    // ---- C
+    if (xy) {
+      constexpr int NXF = (TX + 1) * TY;
+      for (int f = tid; f < NXF + TX * (TY + 1); f += NT) {
+        const int d = f < NXF ? 0 : 1, g = d == 0 ? f : f - NXF, w = d == 0 ? TX + 1 : TX;
+        const int fy = g / w, fx = g - fy * w;
+        R ql[5], qr[5], F[5];
+        if (d == 0) {
+          sm.wx[1].ld(fy, fx, ql);
+          sm.wx[0].ld(fy, fx + 1, qr);
+        } else {
+          sm.wy[1].ld(fy, fx, ql);
+          sm.wy[0].ld(fy + 1, fx, qr);
+        }
+        floor_max(ql, rf, pf);
+        floor_max(qr, rf, pf);
+        hllc_dyn(d, ql, qr, gamma, igm1, F);
+        if (d == 0) sm.fx.st(fy, fx, F);
+        else sm.fy.st(fy, fx, F);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// The tile's shared memory and block size by policy.
+template <class Pol, int TX, int TY>
+using PpmTileShared = typename std::conditional<sizeof(typename Pol::R) >= 8, PpmWideShared<typename Pol::R, TX, TY>,
+                                                PpmShared<typename Pol::R, TX, TY>>::type;
+template <class Pol, int TX, int TY>
+constexpr int ppm_threads() { return sizeof(typename Pol::R) >= 8 ? 2 * TX * TY : TX * TY; }
+
 // Periodic box: one tile per block, tiles from the block index.
 template <class Pol, int TX, int TY>
-__global__ void __launch_bounds__(TX * TY, ppm_min_blocks<Pol>())
+__global__ void __launch_bounds__((ppm_threads<Pol, TX, TY>()), ppm_min_blocks<Pol>())
     k_step_ppm(PatchIO<typename Pol::S> P, Params prm, const double* dt_dev, double* dt_next, int zchunk,
                unsigned* err) {
   using R = typename Pol::R;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  auto& sm = *reinterpret_cast<PpmShared<R, TX, TY>*>(smem_raw);
+  auto& sm = *reinterpret_cast<PpmTileShared<Pol, TX, TY>*>(smem_raw);
   const double dt = dt_dev[0];
   if (!(dt > 0.0 && dt <= 1e300)) {
     if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) atomicOr(err, HYDRO_EBIT_BAD_DT);
@@ -552,12 +609,12 @@ __global__ void __launch_bounds__(TX * TY, ppm_min_blocks<Pol>())
 // Patches with three ghost layers: a persistent grid taking tiles from the device work-list by an
 // atomic counter (as the PLM batched kernel); per-patch dt, dx and dt_next.
 template <class Pol, int TX, int TY>
-__global__ void __launch_bounds__(TX * TY, ppm_min_blocks<Pol>())
+__global__ void __launch_bounds__((ppm_threads<Pol, TX, TY>()), ppm_min_blocks<Pol>())
     k_step_ppm_batched(const PatchIO<typename Pol::S>* patches, const TileRec* tiles, int ntiles, int* counter,
                        Params prm, const double* dt_dev, double* dt_next, int zchunk, unsigned* err) {
   using R = typename Pol::R;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  auto& sm = *reinterpret_cast<PpmShared<R, TX, TY>*>(smem_raw);
+  auto& sm = *reinterpret_cast<PpmTileShared<Pol, TX, TY>*>(smem_raw);
   unsigned flags = 0;
   for (;;) {
     __syncthreads();
@@ -592,7 +649,7 @@ static_assert(kTileX[0] == kPpmTX && kTileY[0] == kPpmTY, "the PPM work-list is 
 
 template <class Pol>
 cudaError_t ppm_attr(const void* fn) {
-  const size_t smem = sizeof(PpmShared<typename Pol::R, kPpmTX, kPpmTY>);
+  const size_t smem = sizeof(PpmTileShared<Pol, kPpmTX, kPpmTY>);
   return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
@@ -602,9 +659,9 @@ cudaError_t launch_ppm(const HostPatchIO& P, const Params& prm, const double* dt
   static PerDeviceOnce attr;
   cudaError_t ea = attr.call([&] { return ppm_attr<Pol>(reinterpret_cast<const void*>(k_step_ppm<Pol, kPpmTX, kPpmTY>)); });
   if (ea != cudaSuccess) return ea;
-  const size_t smem = sizeof(PpmShared<typename Pol::R, kPpmTX, kPpmTY>);
+  const size_t smem = sizeof(PpmTileShared<Pol, kPpmTX, kPpmTY>);
   dim3 grid((P.nx + kPpmTX - 1) / kPpmTX, (P.ny + kPpmTY - 1) / kPpmTY, (P.nz + zchunk - 1) / zchunk);
-  k_step_ppm<Pol, kPpmTX, kPpmTY><<<grid, kPpmTX * kPpmTY, smem, s>>>(to_dev<Pol>(P), prm, dt, dt_next, zchunk, err);
+  k_step_ppm<Pol, kPpmTX, kPpmTY><<<grid, ppm_threads<Pol, kPpmTX, kPpmTY>(), smem, s>>>(to_dev<Pol>(P), prm, dt, dt_next, zchunk, err);
   return cudaGetLastError();
 }
 
@@ -617,12 +674,12 @@ cudaError_t launch_ppm_batched(const HostPatchIO* d_patches, const HostTileRec* 
   static PerDeviceOnce attr;
   cudaError_t ea = attr.call([&] { return ppm_attr<Pol>(reinterpret_cast<const void*>(fn)); });
   if (ea != cudaSuccess) return ea;
-  const size_t smem = sizeof(PpmShared<typename Pol::R, kPpmTX, kPpmTY>);
+  const size_t smem = sizeof(PpmTileShared<Pol, kPpmTX, kPpmTY>);
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kPpmTX * kPpmTY, smem) != cudaSuccess || per_sm < 1)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, ppm_threads<Pol, kPpmTX, kPpmTY>(), smem) != cudaSuccess || per_sm < 1)
     per_sm = 1;
   const int grid = std::max(1, std::min(ntiles, sm_count * per_sm));
-  fn<<<grid, kPpmTX * kPpmTY, smem, s>>>(reinterpret_cast<const PatchIO<typename Pol::S>*>(d_patches),
+  fn<<<grid, ppm_threads<Pol, kPpmTX, kPpmTY>(), smem, s>>>(reinterpret_cast<const PatchIO<typename Pol::S>*>(d_patches),
                                          reinterpret_cast<const TileRec*>(d_tiles), ntiles, d_counter, prm, dt,
                                          dt_next, zchunk, err);
   return cudaGetLastError();
