@@ -46,8 +46,14 @@ __device__ __forceinline__ void hllc_core_adj(const R qL[5], const R qR[5], R ke
   // ---- forward recomputation (the values that select branches exactly as hllc_core forms them)
   R irL, irR;
   rcp2(qL[0], qR[0], irL, irR);
-  const R cL = rsqrt_(gamma * qL[4] * irL);
-  const R cR = rsqrt_(gamma * qR[4] * irR);
+  R cL, cR;
+  if constexpr (std::is_same<R, double>::value) {
+    cL = sound_speed(gamma * qL[4], qL[0]);
+    cR = sound_speed(gamma * qR[4], qR[0]);
+  } else {
+    cL = rsqrt_(gamma * qL[4] * irL);
+    cR = rsqrt_(gamma * qR[4] * irR);
+  }
   const R uL = qL[1], uR = qR[1];
   const R aL = uL - cL, bL = uR - cR;
   const bool selL = aL <= bL;

@@ -175,17 +175,24 @@ __device__ __forceinline__ df2 norm_(const df2& x) {
   const float2 s = add2_(x.h, x.l);
   return df2{s, sub2_(x.l, sub2_(s, x.h))};
 }
+__device__ __forceinline__ df2 two_sum2_(const float2& a, const float2& b) {
+  const float2 s = add2_(a, b), t = sub2_(s, a);
+  return df2{s, add2_(sub2_(a, sub2_(s, t)), sub2_(b, t))};
+}
 __device__ __forceinline__ df2 sum_(const df2& x, const df2& y) {
-  const float2 s = add2_(x.h, y.h);
-  const float2 b = sub2_(s, x.h);
-  const float2 e = add2_(sub2_(x.h, sub2_(s, b)), sub2_(y.h, b));
-  return df2{s, add2_(e, add2_(x.l, y.l))};
+  const df2 s = two_sum2_(x.h, y.h);
+  return df2{s.h, add2_(s.l, add2_(x.l, y.l))};
 }
 __device__ __forceinline__ df2 operator+(const df2& x, const df2& y) { return norm_(sum_(x, y)); }
 __device__ __forceinline__ df2 operator-(const df2& x, const df2& y) { return norm_(sum_(x, neg_(y))); }
 __device__ __forceinline__ df2 prod_(const df2& x, const df2& y) {
   const float2 p = mul2_(x.h, y.h);
   return df2{p, fma2_(x.h, y.l, fma2_(x.l, y.h, fma2_(x.h, y.h, neg_(p))))};
+}
+__device__ __forceinline__ df2 add_acc(const df2& x, const df2& y) {  // the accurate sum
+  const df2 s = two_sum2_(x.h, y.h), t = two_sum2_(x.l, y.l);
+  const df2 v = norm_(df2{s.h, add2_(s.l, t.h)});
+  return norm_(df2{v.h, add2_(v.l, t.l)});
 }
 __device__ __forceinline__ df2 rcpu_(const df2& y) {
   float2 r0;
@@ -206,6 +213,21 @@ __device__ __forceinline__ df2 rootu_(const df2& x) {
   const float2 p = mul2_(s0, s0);
   const float2 r = add2_(sub2_(sub2_(x.h, p), fma2_(s0, s0, neg_(p))), x.l);
   return df2{s0, mul2_(mul2_(r, make_float2(0.5f, 0.5f)), i0)};
+}
+
+// sqrt(t/r), as one Newton correction of t rsqrt(t r): one SFU approximation per value where the
+// reciprocal and the root took three, and no quotient.
+__device__ __forceinline__ df2 rootq_(const df2& t, const df2& r) {
+  const float2 x = mul2_(t.h, r.h);
+  float2 y0;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y0.x) : "f"(x.x));
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y0.y) : "f"(x.y));
+  y0.x = x.x > 1.2e-38f ? y0.x : 0.f;  // zero (and what .ftz reads as zero) has root zero
+  y0.y = x.y > 1.2e-38f ? y0.y : 0.f;
+  const float2 s0 = mul2_(t.h, y0), p = mul2_(s0, s0);
+  const df2 w = prod_(df2{p, fma2_(s0, s0, neg_(p))}, r);  // s0^2 r
+  const float2 e = add2_(sub2_(sub2_(t.h, w.h), w.l), t.l);  // t - s0^2 r
+  return df2{s0, mul2_(mul2_(e, make_float2(0.5f, 0.5f)), y0)};
 }
 
 // Comparisons of normalised values.

@@ -404,6 +404,16 @@ __device__ __forceinline__ void hllc_core(const R qL[5], const R qR[5], bool zn,
   F[4] = ue * (Ee + pe);
 }
 
+// sqrt(t/r) as t rsqrt(t r): one approximation and the third-order step for both the root and the
+// quotient (zero where t r is zero, or flushed to it).
+__device__ __forceinline__ double sound_speed(double t, double r) {
+  const double x = t * r;
+  double y0;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
+  const double s0 = t * y0, e = fma(-(x * y0), y0, 1.0);
+  const double s = fma(s0, e * fma(e, 0.375, 0.5), s0);
+  return __double2hiint(x) >= 0x00100000 ? s : 0.0;
+}
 // S* - u_L (the reverse step forms its S* with it too, and selects the same branches).
 __device__ __forceinline__ double contact_offset(const double qL[5], const double qR[5], double mR, double du,
                                                  double den) {
@@ -414,7 +424,7 @@ __device__ __forceinline__ double contact_offset(const double qL[5], const doubl
 // divisions and roots about 120.
 __device__ __forceinline__ void hllc_core(const double qL[5], const double qR[5], bool, double gamma, double inv_gm1,
                                           double F[5]) {
-  const double cL = rsqrt_(gamma * qL[4] * rcp_(qL[0])), cR = rsqrt_(gamma * qR[4] * rcp_(qR[0]));
+  const double cL = sound_speed(gamma * qL[4], qL[0]), cR = sound_speed(gamma * qR[4], qR[0]);
   const double uL = qL[1], uR = qR[1];
   const double aL = uL - cL, bL = uR - cR, aR = uL + cL, bR = uR + cR;
   const double SL = aL <= bL ? aL : bL, SR = aR >= bR ? aR : bR;
@@ -461,7 +471,7 @@ __device__ __forceinline__ void hllc_core(const double qL[5], const double qR[5]
 __device__ __forceinline__ void hllc_core(const df qL[5], const df qR[5], bool, const df& gamma, const df& inv_gm1,
                                           df F[5]) {
   const df2 r2 = pair_(qL[0], qR[0]), u2 = pair_(qL[1], qR[1]), p2 = pair_(qL[4], qR[4]);
-  const df2 c2 = rootu_(prod_(prod_(both_(gamma), p2), rcpu_(r2)));
+  const df2 c2 = rootq_(prod_(both_(gamma), p2), r2);
   const df2 lo = u2 - c2, hi = u2 + c2;
   const df aL = first_(lo), bL = second_(lo), aR = first_(hi), bR = second_(hi);
   const df SL = aL <= bL ? aL : bL;
@@ -766,6 +776,31 @@ struct PolDF {
   static __device__ __forceinline__ void recover(const double U[5], const Params& P, df q[5], unsigned& flags) {
     df ir;
     recover(U, P, q, ir, flags);
+  }
+  // Two cells at once, side by side in packed FP32: the same operations lane by lane.
+  static __device__ __forceinline__ void recover2(const double U0[5], const double U1[5], const Params& P, df q0[5],
+                                                  df q1[5], unsigned& flags) {
+    df a[5], b[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      split_double(U0[v], a[v].h, a[v].l);
+      split_double(U1[v], b[v].h, b[v].l);
+    }
+    const df rf = kc<df>(P, K_RHOF), pf = kc<df>(P, K_PF);
+    if (a[0] < rf) { flags |= HYDRO_EBIT_RHO_FLOOR; a[0] = rf; }
+    if (b[0] < rf) { flags |= HYDRO_EBIT_RHO_FLOOR; b[0] = rf; }
+    const df2 ir = norm_(rcpu_(pair_(a[0], b[0])));
+    const df2 mx = pair_(a[1], b[1]), my = pair_(a[2], b[2]), mz = pair_(a[3], b[3]);
+    const df2 kin = norm_(prod_(norm_(sum_(sum_(prod_(mx, mx), prod_(my, my)), prod_(mz, mz))), half_(ir)));
+    const df2 eint = add_acc(pair_(a[4], b[4]), neg_(kin));
+    if (cmp_neg(first_(eint)) || cmp_neg(second_(eint))) flags |= HYDRO_EBIT_P_FLOOR;
+    const df2 p = norm_(prod_(both_(kc<df>(P, K_GM1)), eint));
+    if (!(isfinite(p.h.x) && isfinite(p.h.y) && isfinite(a[0].h) && isfinite(b[0].h))) flags |= HYDRO_EBIT_NONFINITE;
+    const df2 u = norm_(prod_(mx, ir)), v = norm_(prod_(my, ir)), w = norm_(prod_(mz, ir));
+    q0[0] = a[0]; q0[1] = first_(u); q0[2] = first_(v); q0[3] = first_(w);
+    q0[4] = first_(p) < pf ? pf : first_(p);
+    q1[0] = b[0]; q1[1] = second_(u); q1[2] = second_(v); q1[3] = second_(w);
+    q1[4] = second_(p) < pf ? pf : second_(p);
   }
   // U_old - dtdx * div: the double-float increment made a double exactly (float_to_double) and
   // subtracted from the double state in double.

@@ -397,13 +397,21 @@ __device__ void step_tile(TileShared<Pol, TX, TY>& sm, const PatchIO<typename Po
       }
     }
   };
+  constexpr bool kPairRecover = std::is_same<R, df>::value;
   auto store_pair = [&](int slot, int c, const S U0[5], const S U1[5]) {
     const int cy = c / QP, cx = 2 * (c - cy * QP);
     R q[5];
-    Pol::recover(U0, prm, q, flags);
-    sm.q[slot].st(cy, cx, q);
-    Pol::recover(U1, prm, q, flags);
-    sm.q[slot].st(cy, cx + 1, q);
+    if constexpr (kPairRecover) {
+      R q1[5];
+      Pol::recover2(U0, U1, prm, q, q1, flags);
+      sm.q[slot].st(cy, cx, q);
+      sm.q[slot].st(cy, cx + 1, q1);
+    } else {
+      Pol::recover(U0, prm, q, flags);
+      sm.q[slot].st(cy, cx, q);
+      Pol::recover(U1, prm, q, flags);
+      sm.q[slot].st(cy, cx + 1, q);
+    }
   };
   auto load_plane = [&](int z) {
     const int slot = ring_slot(z);
