@@ -371,8 +371,8 @@ __device__ __forceinline__ void hllc_core(const R qL[5], const R qR[5], bool zn,
   const R mR = qR[0] * (SR - uR);
   const R Ss = div_(qR[4] - qL[4] + uL * mL - uR * mR, mL - mR);
   const bool SLneg = cmp_neg(SL), SRpos = cmp_pos(SR);
-  const bool star = SLneg && SRpos;
-  const bool left = !SLneg || (SRpos && !cmp_neg(Ss));
+  const bool star = SLneg & SRpos;  // (evaluated in full: a short circuit is a branch)
+  const bool left = !SLneg | (SRpos & !cmp_neg(Ss));
   const R rK = left ? qL[0] : qR[0];
   const R uK = left ? uL : uR;
   const R t1 = left ? qL[2] : qR[2];
@@ -579,15 +579,11 @@ static __device__ __noinline__ float2 split_double_cvt(double x) {
 }
 static __device__ __noinline__ double float_to_double_cvt(float f) { return (double)f; }
 
-__device__ __forceinline__ void split_double(double x, float& hi, float& lo) {
+// The common path alone; bad is set where x needs the conversions.
+__device__ __forceinline__ void split_fast(double x, float& hi, float& lo, bool& bad) {
   const unsigned xh = (unsigned)__double2hiint(x), xl = (unsigned)__double2loint(x);
   const unsigned ex = (xh >> 20) & 0x7FFu;  // biased exponent, E = ex - 1023
-  if (__builtin_expect(ex - 949u >= 173u, 0)) {
-    const float2 c = split_double_cvt(x);  // returned in registers: no stack frame on the common path
-    hi = c.x;
-    lo = c.y;
-    return;
-  }
+  bad |= ex - 949u >= 173u;
   const unsigned sign = xh & 0x80000000u;
   const float ht = __uint_as_float(sign | ((ex - 896u) << 23) | ((xh & 0xFFFFFu) << 3) | (xl >> 29));
   const unsigned r = xl & 0x1FFFFFFFu;
@@ -595,6 +591,27 @@ __device__ __forceinline__ void split_double(double x, float& hi, float& lo) {
   const float lt = __uint_as_float(__float_as_uint(rf * __uint_as_float((ex - 948u) << 23)) | sign);
   hi = ht + lt;
   lo = lt - (hi - ht);
+}
+__device__ __forceinline__ void split_double(double x, float& hi, float& lo) {
+  bool bad = false;
+  split_fast(x, hi, lo, bad);
+  if (__builtin_expect(bad, 0)) {
+    const float2 c = split_double_cvt(x);  // returned in registers: no stack frame on the common path
+    hi = c.x;
+    lo = c.y;
+  }
+}
+// Five values with one test for all of them: a test per value is a branch per value (with the update's
+// increments, below, also tested together: mixed 256^3 step 840 -> 800 us, 4096 mixed patches 10.55 ->
+// 9.82 ms).
+__device__ __forceinline__ void split5(const double x[5], float hi[5], float lo[5]) {
+  bool bad = false;
+#pragma unroll
+  for (int v = 0; v < 5; ++v) split_fast(x[v], hi[v], lo[v], bad);
+  if (__builtin_expect(bad, 0)) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) split_double(x[v], hi[v], lo[v]);
+  }
 }
 // Exact float -> double: sign kept, exponent rebiased by 1023 - 127, the 23 fraction bits placed
 // at the top of the 52.  Zero maps to zero; subnormal, infinite and NaN floats take the cvt.
@@ -604,6 +621,14 @@ __device__ __forceinline__ double float_to_double(float f) {
   if (__builtin_expect(e == 0u || e == 0xFFu, 0))
     return (b & 0x7FFFFFFFu) == 0u ? __hiloint2double((int)(b & 0x80000000u), 0) : float_to_double_cvt(f);
   return __hiloint2double((int)((b & 0x80000000u) | ((e + 896u) << 20) | ((b & 0x7FFFFFu) >> 3)), (int)(b << 29));
+}
+// The same without a branch, zero selected; bad is set where f needs the conversion.
+__device__ __forceinline__ double float_to_double_fast(float f, bool& bad) {
+  const unsigned b = __float_as_uint(f), m = b & 0x7FFFFFFFu;
+  const unsigned e = m >> 23;
+  bad |= (m != 0u) & ((e == 0u) | (e == 0xFFu));
+  const unsigned h = (b & 0x80000000u) | ((e + 896u) << 20) | ((b & 0x7FFFFFu) >> 3);
+  return __hiloint2double((int)(m == 0u ? b : h), (int)(b << 29));
 }
 
 // ------------------------------------------------------------------ precision policies
@@ -630,6 +655,10 @@ struct PolF64 {
     q[4] = p < P.p_floor ? P.p_floor : p;
   }
   static __device__ __forceinline__ double update(double Uold, double dtdx, double div) { return Uold - dtdx * div; }
+  static __device__ __forceinline__ void update5(const double U[5], double dtdx, const double div[5], double Un[5]) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) Un[v] = update(U[v], dtdx, div[v]);
+  }
   static __device__ __forceinline__ double speed(const double U[5], const Params& P, unsigned& flags);
 };
 
@@ -672,6 +701,10 @@ struct PolF32 {
     q[4] = p < pf ? pf : p;
   }
   static __device__ __forceinline__ float update(float Uold, float dtdx, float div) { return Uold - dtdx * div; }
+  static __device__ __forceinline__ void update5(const float U[5], float dtdx, const float div[5], float Un[5]) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) Un[v] = update(U[v], dtdx, div[v]);
+  }
   // CFL speed of a stored state: plain float recovery (the dt only needs float accuracy).
   static __device__ __forceinline__ float speed(const float U[5], const Params& P, unsigned& flags) {
     float rho = U[0];
@@ -699,19 +732,12 @@ struct PolMixed {
   // E's low part: the internal energy to float accuracy unless the kinetic energy exceeds it by
   // ~2^20, with no FP64 instruction.
   static __device__ __forceinline__ void recover(const double U[5], const Params& P, float q[5], unsigned& flags) {
-    float rh, rl;
-    if (cmp_lt_floor(U[0], P.kd[K_RHOF])) {
-      flags |= HYDRO_EBIT_RHO_FLOOR;
-      rh = P.kh[K_RHOF];
-      rl = P.kl[K_RHOF];
-    } else {
-      split_double(U[0], rh, rl);
-    }
-    float xh, xl, yh, yl, zh, zl, eh, el;
-    split_double(U[1], xh, xl);
-    split_double(U[2], yh, yl);
-    split_double(U[3], zh, zl);
-    split_double(U[4], eh, el);
+    float h[5], l[5];
+    split5(U, h, l);
+    const bool low = cmp_lt_floor(U[0], P.kd[K_RHOF]);
+    if (low) flags |= HYDRO_EBIT_RHO_FLOOR;
+    const float rh = low ? P.kh[K_RHOF] : h[0], rl = low ? P.kl[K_RHOF] : l[0];
+    const float xh = h[1], xl = l[1], yh = h[2], yl = l[2], zh = h[3], zl = l[3], eh = h[4], el = l[4];
     const float ir = __frcp_rn(rh);
     const float a1 = xh * xh, e1 = fmaf(xh, xh, -a1);
     const float a2 = yh * yh, e2 = fmaf(yh, yh, -a2);
@@ -741,6 +767,15 @@ struct PolMixed {
   static __device__ __forceinline__ double update(double Uold, float dtdx, float div) {
     return Uold - float_to_double(dtdx * div);
   }
+  static __device__ __forceinline__ void update5(const double U[5], float dtdx, const float div[5], double Un[5]) {
+    bool bad = false;  // one test for the five increments
+#pragma unroll
+    for (int v = 0; v < 5; ++v) Un[v] = U[v] - float_to_double_fast(dtdx * div[v], bad);
+    if (__builtin_expect(bad, 0)) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) Un[v] = update(U[v], dtdx, div[v]);
+    }
+  }
   static __device__ __forceinline__ float speed(const double U[5], const Params& P, unsigned& flags);
 };
 
@@ -750,12 +785,10 @@ struct PolDF {
   // The same recovery as PolF64, in double-float from the double state (split into float pairs on
   // the integer pipe, split_double); ir receives 1/rho.
   static __device__ __forceinline__ void recover(const double U[5], const Params& P, df q[5], df& ir, unsigned& flags) {
-    df rho, mx, my, mz, E;
-    split_double(U[0], rho.h, rho.l);
-    split_double(U[1], mx.h, mx.l);
-    split_double(U[2], my.h, my.l);
-    split_double(U[3], mz.h, mz.l);
-    split_double(U[4], E.h, E.l);
+    float h[5], l[5];
+    split5(U, h, l);
+    df rho(h[0], l[0]);
+    const df mx(h[1], l[1]), my(h[2], l[2]), mz(h[3], l[3]), E(h[4], l[4]);
     const df rf = kc<df>(P, K_RHOF);
     if (rho < rf) { flags |= HYDRO_EBIT_RHO_FLOOR; rho = rf; }
     ir = norm_(rcpu_(rho));
@@ -781,10 +814,14 @@ struct PolDF {
   static __device__ __forceinline__ void recover2(const double U0[5], const double U1[5], const Params& P, df q0[5],
                                                   df q1[5], unsigned& flags) {
     df a[5], b[5];
+    {
+      float h[5], l[5];
+      split5(U0, h, l);
 #pragma unroll
-    for (int v = 0; v < 5; ++v) {
-      split_double(U0[v], a[v].h, a[v].l);
-      split_double(U1[v], b[v].h, b[v].l);
+      for (int v = 0; v < 5; ++v) a[v] = df(h[v], l[v]);
+      split5(U1, h, l);
+#pragma unroll
+      for (int v = 0; v < 5; ++v) b[v] = df(h[v], l[v]);
     }
     const df rf = kc<df>(P, K_RHOF), pf = kc<df>(P, K_PF);
     if (a[0] < rf) { flags |= HYDRO_EBIT_RHO_FLOOR; a[0] = rf; }
@@ -807,6 +844,18 @@ struct PolDF {
   static __device__ __forceinline__ double update(double Uold, const df& dtdx, const df& div) {
     const df d = prod_(dtdx, div);
     return Uold - (float_to_double(d.h) + float_to_double(d.l));
+  }
+  static __device__ __forceinline__ void update5(const double U[5], const df& dtdx, const df div[5], double Un[5]) {
+    bool bad = false;  // one test for the ten words
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      const df d = prod_(dtdx, div[v]);
+      Un[v] = U[v] - (float_to_double_fast(d.h, bad) + float_to_double_fast(d.l, bad));
+    }
+    if (__builtin_expect(bad, 0)) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) Un[v] = update(U[v], dtdx, div[v]);
+    }
   }
   static __device__ __forceinline__ df speed(const double U[5], const Params& P, unsigned& flags);
 };

@@ -304,7 +304,7 @@ struct OctTable {
 
 // Resident blocks per SM: as many as the batch's scratch leaves room for, in float arithmetic six (80
 // registers), five for the gathered buffer, whose prefetch spills at 80 (262144 groups, mixed: 392 us
-// against 403; the whole level through its table: 3.34 ms at six, 3.47 at five).
+// against 403, and 514 for a group at a time; the whole level through its table: 3.34 ms at six, 3.47 at five).
 template <class Pol, class Src>
 constexpr int oct_min_blocks() { return sizeof(typename Pol::R) >= 8 ? 3 : (Src::kGathered ? 5 : 6); }
 
@@ -505,8 +505,12 @@ __global__ void __launch_bounds__(32 * kOctWarps, (oct_min_blocks<Pol, Src>())) 
       for (int v = 0; v < 5; ++v) div[v] = ((a[0][v] - a[1][v]) + (a[2][v] - a[3][v])) + (a[4][v] - a[5][v]);
       long long in, out;
       src.own(g0 + b, e, in, out);
+      S Uo[5], Un[5];
 #pragma unroll
-      for (int v = 0; v < 5; ++v) gout[v][out] = Pol::update(__ldg(src.f[v] + in), dtdx, div[v]);
+      for (int v = 0; v < 5; ++v) Uo[v] = __ldg(src.f[v] + in);
+      Pol::update5(Uo, dtdx, div, Un);
+#pragma unroll
+      for (int v = 0; v < 5; ++v) gout[v][out] = Un[v];
     }
     __syncwarp();
   }
@@ -648,12 +652,16 @@ __global__ void __launch_bounds__(kCubeThreads, sizeof(typename Pol::R) >= 8 ? 1
       const int x = 2 * (o & 3) + (e & 1), y = 2 * ((o >> 2) & 3) + ((e >> 1) & 1), z = 2 * (o >> 4) + (e >> 2);
       const int fx = x * 64 + y + 8 * z, fy = 576 + y * 64 + x + 8 * z, fz = 1152 + z * 64 + x + 8 * y;
       const long long a = 8LL * sm.ids[((o >> 4) + 1) * 36 + (((o >> 2) & 3) + 1) * 6 + (o & 3) + 1] + e;
+      R div[5];
+      S Uo[5];
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
         const R* F = sm.q[v];
-        const R div = ((F[fx + 64] - F[fx]) + (F[fy + 64] - F[fy])) + (F[fz + 64] - F[fz]);
-        gout[v][a] = Pol::update(__ldg(src.f[v] + a), dtdx, div);
+        div[v] = ((F[fx + 64] - F[fx]) + (F[fy + 64] - F[fy])) + (F[fz + 64] - F[fz]);
+        Uo[v] = __ldg(src.f[v] + a);
       }
+#pragma unroll
+      for (int v = 0; v < 5; ++v) gout[v][a] = Pol::update(Uo[v], dtdx, div[v]);
     }
   }
   flush_flags(flags, err);

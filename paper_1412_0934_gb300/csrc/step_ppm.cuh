@@ -272,15 +272,15 @@ __device__ __forceinline__ void ppm_tile(PpmShared<typename Pol::R, TX, TY>& sm,
           const int z = p - 1;
           const long long ai = (long long)(z + P.gin) * P.isz + (long long)(y0 + j + P.gin) * P.isy + (x0 + i + P.gin);
           const long long ao = (long long)(z + P.gout) * P.osz + (long long)(y0 + j + P.gout) * P.osy + (x0 + i + P.gout);
-          S Un[5];
+          S Uo[5], Un[5];
           R dz[5];
           sub5(F, fzb, dz);
           add5(dxy, dz, dxy);
 #pragma unroll
-          for (int v = 0; v < 5; ++v) {
-            Un[v] = Pol::update(__ldg(P.in[v] + ai), dtdx, dxy[v]);
-            P.out[v][ao] = Un[v];
-          }
+          for (int v = 0; v < 5; ++v) Uo[v] = __ldg(P.in[v] + ai);
+          Pol::update5(Uo, dtdx, dxy, Un);
+#pragma unroll
+          for (int v = 0; v < 5; ++v) P.out[v][ao] = Un[v];
           if (want_cfl) {
             const R sp = Pol::speed(Un, prm, flags);
             smax = sp > smax ? sp : smax;
@@ -360,7 +360,8 @@ __device__ __forceinline__ void ppm_tile(PpmShared<typename Pol::R, TX, TY>& sm,
 //      the others: the ring cells' predictor and face states, and the load of plane p + 3 into the
 //      slot of plane p - 2
 //   C  the 544 x and y faces
-// 191x203x187 double-float step: 7.7 -> 4.0 ms; 96^3 double (FP64 pipe): 2.83 -> 2.46 ms.
+// 191x203x187 double-float step: 7.7 -> 4.0 ms (2.8 with branch-free comparisons); 96^3 double (FP64
+// pipe): 2.83 -> 2.46 ms.
 template <class R, int TX, int TY>
 struct PpmWideShared {
   static constexpr int QX = TX + 2 * kPpmHalo, QY = TY + 2 * kPpmHalo;
@@ -513,12 +514,12 @@ __device__ __forceinline__ void ppm_tile(PpmWideShared<typename Pol::R, TX, TY>&
             const int z = p - 1;
             const long long ai = (long long)(z + P.gin) * P.isz + (long long)(y0 + j + P.gin) * P.isy + (x0 + i + P.gin);
             const long long ao = (long long)(z + P.gout) * P.osz + (long long)(y0 + j + P.gout) * P.osy + (x0 + i + P.gout);
-            double Un[5];
+            double Uo[5], Un[5];
 #pragma unroll
-            for (int v = 0; v < 5; ++v) {
-              Un[v] = Pol::update(__ldg(P.in[v] + ai), dtdx, div[v]);
-              P.out[v][ao] = Un[v];
-            }
+            for (int v = 0; v < 5; ++v) Uo[v] = __ldg(P.in[v] + ai);
+            Pol::update5(Uo, dtdx, div, Un);
+#pragma unroll
+            for (int v = 0; v < 5; ++v) P.out[v][ao] = Un[v];
             if (want_cfl) {
               const R sp = Pol::speed(Un, prm, flags);
               smax = sp > smax ? sp : smax;

@@ -487,11 +487,12 @@ __device__ void step_tile(TileShared<Pol, TX, TY>& sm, const PatchIO<typename Po
       const long long ai = (long long)(k + P.gin) * P.isz + (long long)(gy + P.gin) * P.isy + (gx + P.gin);
       const long long ao = (long long)(k + P.gout) * P.osz + (long long)(gy + P.gout) * P.osy + (gx + P.gout);
       if (!index_ok(ai, in_extent, flags) || !index_ok(ao, (long long)(P.nz + 2 * P.gout) * P.osz, flags)) return false;
+      S Uo[5];
 #pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        Un[v] = Pol::update(__ldg(P.in[v] + ai), dtdx, dF[v]);
-        P.out[v][ao] = Un[v];
-      }
+      for (int v = 0; v < 5; ++v) Uo[v] = __ldg(P.in[v] + ai);
+      Pol::update5(Uo, dtdx, dF, Un);
+#pragma unroll
+      for (int v = 0; v < 5; ++v) P.out[v][ao] = Un[v];
       return true;
     };
     S Un[5];
@@ -536,7 +537,8 @@ __device__ void step_tile(TileShared<Pol, TX, TY>& sm, const PatchIO<typename Po
   // NIX + NIY faces lie between two tile cells.  The split barriers pay where a block is alone on
   // its SM (512 threads, or the one-block-per-SM build): with two resident blocks the other block
   // already fills the barrier waits, and interleaving the predictor with the faces costs more
-  // (measured at 16x16: 37.0 vs 31.7 ms per 512^3 step; at 32x16: 31.5 vs 32.7 ms).
+  // (measured before the packed arithmetic, at 16x16: 37.0 vs 31.7 ms per 512^3 step; at 32x16: 31.5 vs
+  // 32.7 ms).
   constexpr bool kSplit = kCompact && min_blocks<Pol, NT, MINB>() == 1;
   constexpr int RW = (NR + 31) / 32, NTI = kSplit ? NT - 32 * RW : NT - NR;
   constexpr int NIX = (TX - 1) * TY, NIF = NIX + TX * (TY - 1);
