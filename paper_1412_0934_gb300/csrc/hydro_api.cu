@@ -298,8 +298,9 @@ int class_zc(const hydro_ctx* c, int k) { return c->cls_tile[k] >= 0 ? c->cls_zc
 // rest.  Short chunks fill the SMs of a small box (32^3 at one 32-plane chunk of 16x16 tiles is 4 blocks)
 // and repeat two planes each; long ones serve the large boxes.  The constants are fits to steps of 16^3
 // to 512^3 boxes at 2 to 128-plane chunks; the model stays within 5% of those and picks, against the
-// fixed 16x16 tiles of 32 planes: FP64 32^3 1367 -> 97 us, double-float 64^3 359 -> 77, FP32 96^3 76 -> 46,
-// mixed 64^3 124 -> 33; 512^3 within 1% of the best of the sweep.
+// fixed 16x16 tiles of 32 planes: FP64 32^3 1367 -> 97 us, double-float 61^3 256 -> 70, FP32 96^3 76 -> 46,
+// mixed 64^3 124 -> 33; 512^3 within 1% of the best of the sweep.  (Double-float since its comparisons are
+// branch-free: 16x16 tiles with two blocks per SM take the 512^3 step in 20.3 ms, 32x16 tiles in 22.4.)
 struct ShapeCost {
   int tile;
   double plane, start;
@@ -309,7 +310,7 @@ struct ShapeCost {
 constexpr ShapeCost kCostF64[] = {{0, 41.0, 1.2, 2, {0.0, 1.0, 1.77}},
                                   {2, 28.4, 1.25, 3, {0.0, 1.0, 1.0, 1.27}},
                                   {3, 73.6, 1.04, 1, {0.0, 1.0}}};
-constexpr ShapeCost kCostDF[] = {{0, 10.5, 1.9, 2, {0.0, 1.0, 1.3}}, {3, 13.25, 1.8, 1, {0.0, 1.0}}};
+constexpr ShapeCost kCostDF[] = {{0, 7.6, 1.9, 2, {0.0, 1.0, 1.52}}, {3, 12.6, 1.8, 1, {0.0, 1.0}}};
 constexpr ShapeCost kCostF32[] = {{0, 1.95, 5.3, 3, {0.0, 1.0, 1.29, 1.76}},
                                   {1, 1.94, 5.3, 3, {0.0, 1.0, 1.29, 1.76}},
                                   {3, 2.5, 4.9, 1, {0.0, 1.0}}};
@@ -368,7 +369,7 @@ void default_tuning(const hydro_ctx* c, const hydro_patch* in, int n, int* tile,
   // Where that fills every SM four times over there is little left to balance, and differences the model
   // does not hold (caches, uneven patches, the last tiles' tail) decide: the batched, FP64 and PPM steps
   // keep it (4096 uneven patches, mixed: 10.8 ms, 11.6 with the model's choice; FP64 256^3 16.4 against
-  // 16.9).  Uniform boxes in double-float and float still gain 3-4% from fewer start planes.
+  // 16.9).  Uniform boxes in double-float and float still gain 2-4% from fewer start planes.
   if (blocks0 >= 4LL * shapes[0].resident * c->sm_count && (n > 1 || ppm(c) || c->cfg.precision == HYDRO_FP64)) return;
   if (n == 1) {
     // one box: every chunk count up to 64, and two-plane chunks at the least
