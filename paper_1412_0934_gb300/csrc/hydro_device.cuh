@@ -466,8 +466,10 @@ __device__ __forceinline__ void hllc_core(const double qL[5], const double qR[5]
 // left unnormalised inside the formulas, S* from its distance to u_L (S* - u_L = (p_R - p_L + m_R (u_L -
 // u_R)) / (m_L - m_R), which does not cancel in fast flow), and the star energy without 1/m_K: with i =
 // 1/(S_K - S*) and g = (S_K - u_K) i, E* = g E_K + (S* - u_K)(r* S* + p_K i).
-// The fluxes are returned unnormalised (they are only summed).  The kinetic sum's order is (u_n^2 +
-// u_t1^2) + u_t2^2 for every normal.
+// The tangential momentum fluxes are returned unnormalised (they are only summed); the mass flux and the
+// energy's terms are normalised, which costs 2% of the step and keeps the energy's error that of normalising
+// operators throughout (256^3 at Mach 5: 4.4e-15 of its norm, 4.6e-15 with its terms unnormalised).  The
+// kinetic sum's order is (u_n^2 + u_t1^2) + u_t2^2 for every normal.
 __device__ __forceinline__ void hllc_core(const df qL[5], const df qR[5], bool, const df& gamma, const df& inv_gm1,
                                           df F[5]) {
   const df2 r2 = pair_(qL[0], qR[0]), u2 = pair_(qL[1], qR[1]), p2 = pair_(qL[4], qR[4]);
@@ -478,7 +480,7 @@ __device__ __forceinline__ void hllc_core(const df qL[5], const df qR[5], bool, 
   const df SR = aR >= bR ? aR : bR;
   const df2 d2 = pair_(SL, SR) - u2;  // S - u of either side
   const df2 m2 = norm_(prod_(r2, d2));
-  const df du = sum_(qL[1], -qR[1]);
+  const df du = norm_(sum_(qL[1], -qR[1]));
   const df num = sum_(sum_(qR[4], -qL[4]), prod_(second_(m2), du));
   const df dl = norm_(quot_(norm_(num), first_(m2) - second_(m2)));  // S* - u_L
   const df Ss = qL[1] + dl;
@@ -494,15 +496,15 @@ __device__ __forceinline__ void hllc_core(const df qL[5], const df qR[5], bool, 
   const df dK = left ? first_(d2) : second_(d2);
   const df2 tt = pair_(t1, t2);
   const df2 sq = prod_(tt, tt);
-  const df ke = sum_(sum_(prod_(uK, uK), first_(sq)), second_(sq));
-  const df EK = norm_(sum_(prod_(pK, inv_gm1), prod_(half_(rK), ke)));
+  const df ke = norm_(sum_(sum_(prod_(uK, uK), first_(sq)), second_(sq)));
+  const df EK = norm_(prod_(pK, inv_gm1)) + norm_(prod_(half_(rK), ke));
   const df dr = sum_(dl, du);
   const df d = norm_(left ? dl : dr);  // S* - u_K
   const df iD = norm_(rcpu_(dK - d));
-  const df2 rg = prod_(both_(iD), pair_(mK, dK));
+  const df2 rg = norm_(prod_(both_(iD), pair_(mK, dK)));
   const df rs = first_(rg), g = second_(rg);
   const df ps = sum_(pK, prod_(mK, d));
-  const df Es = sum_(prod_(g, EK), prod_(d, sum_(prod_(rs, Ss), prod_(pK, iD))));
+  const df Es = norm_(prod_(g, EK)) + norm_(prod_(d, norm_(sum_(prod_(rs, Ss), prod_(pK, iD)))));
   const df re = star ? rs : rK;
   const df ue = star ? Ss : uK;
   const df pe = star ? ps : pK;
@@ -513,7 +515,7 @@ __device__ __forceinline__ void hllc_core(const df qL[5], const df qR[5], bool, 
   const df2 ft = prod_(both_(mn), tt);
   F[2] = first_(ft);
   F[3] = second_(ft);
-  F[4] = prod_(ue, Ee + pe);
+  F[4] = norm_(prod_(ue, Ee + pe));
 }
 
 template <class R>
