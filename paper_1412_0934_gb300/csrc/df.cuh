@@ -215,18 +215,21 @@ __device__ __forceinline__ df2 rootu_(const df2& x) {
   return df2{s0, mul2_(mul2_(r, make_float2(0.5f, 0.5f)), i0)};
 }
 
-// sqrt(t/r), as a third-order correction of s0 = t rsqrt(t r): one SFU approximation per value where the
-// reciprocal and the root took three, and no quotient.  With d = 1 - s0^2 r / t the root is
-// s0 (1 + d/2 + 3 d^2/8 ...); d is up to 2^-21 (the approximation and three roundings), so a Newton step's
-// missing 3 d^2/8, 2^-44, would be the largest error of the wave speeds.
+// sqrt(t/r), as a third-order correction of s0 = t y0, y0 = rsqrt(t) rsqrt(r): two SFU approximations per
+// value where the reciprocal and the root took three, and no quotient.  (One rsqrt(t r) would do, but the
+// product of a pressure and a density leaves the float range long before either does, and the speed would
+// come out as zero.)  With d = 1 - s0^2 r / t the root is s0 (1 + d/2 + 3 d^2/8 ...); d is up to 2^-20 (the
+// approximations and four roundings), so a Newton step's missing 3 d^2/8, 2^-42, would be the largest error
+// of the wave speeds.
 __device__ __forceinline__ df2 rootq_(const df2& t, const df2& r) {
-  const float2 x = mul2_(t.h, r.h);
-  float2 y0;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y0.x) : "f"(x.x));
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y0.y) : "f"(x.y));
-  y0.x = x.x > 1.2e-38f ? y0.x : 0.f;  // zero (and what .ftz reads as zero) has root zero
-  y0.y = x.y > 1.2e-38f ? y0.y : 0.f;
-  const float2 s0 = mul2_(t.h, y0), p = mul2_(s0, s0);
+  float2 yt, yr;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yt.x) : "f"(t.h.x));
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yt.y) : "f"(t.h.y));
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yr.x) : "f"(r.h.x));
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yr.y) : "f"(r.h.y));
+  yt.x = t.h.x > 1.2e-38f ? yt.x : 0.f;  // zero (and what .ftz reads as zero) has root zero
+  yt.y = t.h.y > 1.2e-38f ? yt.y : 0.f;
+  const float2 y0 = mul2_(yt, yr), s0 = mul2_(t.h, y0), p = mul2_(s0, s0);
   const df2 w = prod_(df2{p, fma2_(s0, s0, neg_(p))}, r);  // s0^2 r
   const float2 e = add2_(sub2_(sub2_(t.h, w.h), w.l), t.l);  // t - s0^2 r
   const float2 c = mul2_(e, y0);                   // s0 d

@@ -77,6 +77,8 @@ __device__ __forceinline__ double div_(double n, double d) {
   const double r = rcp_(d), q = n * r;
   return fma(r, fma(-q, d, n), q);
 }
+// Zero, or what .ftz reads as zero.
+__device__ __forceinline__ bool flushed_(double x) { return ((unsigned)__double2hiint(x) & 0x7fffffffu) < 0x00100000u; }
 __device__ __forceinline__ double rsqrt_(double x) {  // the square root (named like the float one)
   double y0;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
@@ -404,15 +406,16 @@ __device__ __forceinline__ void hllc_core(const R qL[5], const R qR[5], bool zn,
   F[4] = ue * (Ee + pe);
 }
 
-// sqrt(t/r) as t rsqrt(t r): one approximation and the third-order step for both the root and the
-// quotient (zero where t r is zero, or flushed to it).
+// sqrt(t/r) as t y0, y0 = rsqrt(t) rsqrt(r), and one third-order step with e = 1 - (t y0)(r y0): one step
+// for both the root and the quotient, relative error below 2^-52, and no product of t and r, which would leave the
+// range of double before the speed does (zero where t is zero, or flushed to it).
 __device__ __forceinline__ double sound_speed(double t, double r) {
-  const double x = t * r;
-  double y0;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
-  const double s0 = t * y0, e = fma(-(x * y0), y0, 1.0);
+  double yt, yr;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(yt) : "d"(t));
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(yr) : "d"(r));
+  const double y0 = yt * yr, s0 = t * y0, e = fma(-s0, r * y0, 1.0);
   const double s = fma(s0, e * fma(e, 0.375, 0.5), s0);
-  return __double2hiint(x) >= 0x00100000 ? s : 0.0;
+  return flushed_(t) ? 0.0 : s;
 }
 // S* - u_L (the reverse step forms its S* with it too, and selects the same branches).
 __device__ __forceinline__ double contact_offset(const double qL[5], const double qR[5], double mR, double du,
