@@ -120,7 +120,8 @@ __device__ __forceinline__ df norm_(const df& x) { return fast_two_sum(x.h, x.l)
 // reciprocal r0 (1 + e + e^2), e = 1 - y r0, keeps e^2: the approximation's e is up to 2^-23, so e^2 is
 // the largest error of a step whose reciprocals stop at r0 (1 + e).  The
 // quotient's remainder num.h - den.h q is exact in its leading difference (q is the float quotient to
-// a few ulp); the root is one Newton correction, s = s0 + (x - s0^2) / (2 s0).
+// a few ulp); the root is one Newton correction, s = s0 + (x - s0^2) / (2 s0).  Relative errors below 2^-45
+// (sqrt(t/r), further down: 2^-43) where operands, results and t/r lie between 2^-100 and 2^100.
 __device__ __forceinline__ df rcpu_(const df& y) {
   float r0;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(y.h));

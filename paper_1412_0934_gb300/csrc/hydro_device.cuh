@@ -51,11 +51,11 @@ __device__ __forceinline__ R rabs(R x) {
 // Float policies use the SFU approximations (relative error a few ulp of float).  Double starts from the
 // SFU's 20-bit approximations and takes one third-order Newton (Householder) step, 3 to 6 operations on
 // the FP64 pipe, which bounds the double kernels, where the IEEE sequences take about ten and a branch:
-//   1/y:     e = 1 - y r0,        r = r0 (1 + e + e^2)             error below 0.5 ulp + 2^-58
-//   n/d:     q = n r, q + r (n - q d)                              below 0.6 ulp
-//   sqrt(x): s0 = x y0, e = 1 - s0 y0,  s = s0 (1 + e/2 + 3 e^2/8)  below 0.8 ulp
-// for operands and results of magnitude 2^-1020 to 2^1020 (the approximations flush beyond); a zero
-// operand's root is zero.
+//   1/y:     e = 1 - y r0,        r = r0 (1 + e + e^2)             relative error below u + 2^-57, u = 2^-53
+//   n/d:     q = n r, q + r (n - q d)                              below u + 2^-62
+//   sqrt(x): s0 = x y0, e = 1 - s0 y0,  s = s0 (1 + e/2 + 3 e^2/8)  below 1.5 u + 2^-57
+// for operands and results of magnitude 2^-1018 to 2^1018 (the approximations flush beyond; the quotient's
+// remainder needs 2^-900 and more); a zero operand's root is zero.
 __device__ __forceinline__ float rcp_(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -77,14 +77,14 @@ __device__ __forceinline__ double div_(double n, double d) {
   const double r = rcp_(d), q = n * r;
   return fma(r, fma(-q, d, n), q);
 }
-// Zero, or what .ftz reads as zero.
+// Zero, or what .ftz reads as zero (whose root is zero).  A NaN of either sign is neither: its root stays NaN.
 __device__ __forceinline__ bool flushed_(double x) { return ((unsigned)__double2hiint(x) & 0x7fffffffu) < 0x00100000u; }
 __device__ __forceinline__ double rsqrt_(double x) {  // the square root (named like the float one)
   double y0;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
   const double s0 = x * y0, e = fma(-s0, y0, 1.0);
   const double s = fma(s0, e * fma(e, 0.375, 0.5), s0);
-  return __double2hiint(x) >= 0x00100000 ? s : 0.0;  // zero (and what .ftz reads as zero) has root zero
+  return flushed_(x) ? 0.0 : s;
 }
 
 // Constant i of the parameters in arithmetic type R.
@@ -407,7 +407,7 @@ __device__ __forceinline__ void hllc_core(const R qL[5], const R qR[5], bool zn,
 }
 
 // sqrt(t/r) as t y0, y0 = rsqrt(t) rsqrt(r), and one third-order step with e = 1 - (t y0)(r y0): one step
-// for both the root and the quotient, relative error below 2^-52, and no product of t and r, which would leave the
+// for both the root and the quotient, relative error below 2 u + 2^-55, and no product of t and r, which would leave the
 // range of double before the speed does (zero where t is zero, or flushed to it).
 __device__ __forceinline__ double sound_speed(double t, double r) {
   double yt, yr;
