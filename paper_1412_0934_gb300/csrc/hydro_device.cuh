@@ -195,13 +195,24 @@ __device__ __forceinline__ df minmod(const df& a, const df& b) {
 
 // Float: the smaller magnitude with the product of the signs (one min.xorsign.abs) is negative exactly
 // where the signs differ, so max with 0 and the sign of a finish MinMod: three operations on the ALU
-// pipe, which bounds the float kernels together with the issue slots, in place of five.
+// pipe, which bounds the float kernels together with the issue slots, in place of five.  No product is
+// formed, so slopes whose product would underflow count too; a difference that is NaN makes the slope NaN.
 __device__ __forceinline__ float min_xorsign(float a, float b) {
   float t;
-  asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(t) : "f"(a), "f"(b));
+  asm("min.NaN.xorsign.abs.f32 %0, %1, %2;" : "=f"(t) : "f"(a), "f"(b));
   return t;
 }
-__device__ __forceinline__ float minmod(float a, float b) { return copysignf(fmaxf(min_xorsign(a, b), 0.f), a); }
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float t;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(t) : "f"(a), "f"(b));
+  return t;
+}
+__device__ __forceinline__ float min_nan(float a, float b) {
+  float t;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(t) : "f"(a), "f"(b));
+  return t;
+}
+__device__ __forceinline__ float minmod(float a, float b) { return copysignf(max_nan(min_xorsign(a, b), 0.f), a); }
 
 // MC alone (the same values as limited(a, b, HYDRO_MC)); double-float selected, not branched.
 template <class R>
@@ -210,7 +221,7 @@ __device__ __forceinline__ R mc_slope(R a, R b) {
 }
 __device__ __forceinline__ float mc_slope(float a, float b) {
   const float m = fabsf(0.5f * (a + b));
-  return copysignf(fmaxf(fminf(2.f * min_xorsign(a, b), m), 0.f), a);
+  return copysignf(max_nan(min_nan(2.f * min_xorsign(a, b), m), 0.f), a);
 }
 __device__ __forceinline__ df mc_pick(const df& a, const df& b, const df& m) {  // m = (a + b)/2
   const bool pos = a.h > 0.f;
@@ -324,11 +335,6 @@ __device__ __forceinline__ float greater(float a, float b) { return fmaxf(a, b);
 template <class R>
 __device__ __forceinline__ void floor_max(R q[5], R rho_floor, R p_floor) {
   floor_state(q, rho_floor, p_floor);
-}
-__device__ __forceinline__ float max_nan(float a, float b) {
-  float t;
-  asm("max.NaN.f32 %0, %1, %2;" : "=f"(t) : "f"(a), "f"(b));
-  return t;
 }
 __device__ __forceinline__ void floor_max(float q[5], float rho_floor, float p_floor) {
   q[0] = max_nan(q[0], rho_floor);
