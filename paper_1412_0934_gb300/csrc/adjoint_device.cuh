@@ -11,11 +11,15 @@ namespace hydro {
 
 // ------------------------------------------------------------------ limiter with branch code
 // Code: 0 zero slope, 1 the first argument (a, or 2a for MC), 2 the second (b, or 2b for MC),
-// 3 the centred (a+b)/2.  Same comparisons as limited().
+// 3 the centred (a+b)/2.  Same comparisons as limited(), and in float as the forward step's minmod and
+// mc_slope, whose sign test holds where the product underflows.
+template <class R>
+__device__ __forceinline__ bool no_slope(R a, R b) { return prod_nonpos(a, b); }
+__device__ __forceinline__ bool no_slope(float a, float b) { return min_xorsign(a, b) <= 0.f; }
 template <class R>
 __device__ __forceinline__ R limited_code(R a, R b, int lim, unsigned& code) {
   if (lim == HYDRO_NOLIMIT) { code = 3; return half_(a + b); }
-  if (prod_nonpos(a, b)) { code = 0; return R(0); }
+  if (no_slope(a, b)) { code = 0; return R(0); }
   if (lim == HYDRO_MINMOD) {
     if (abs_le(a, b)) { code = 1; return a; }
     code = 2;
