@@ -98,8 +98,7 @@ struct hydro_ctx {
   int rule_n[3] = {0, 0, 0}, rule_tile = 0, rule_zc = 0;  // the rule's choice for the last box size
   // graph cache of hydro_run
   cudaGraphExec_t graph = nullptr;
-  const void* g_a = nullptr;
-  const void* g_b = nullptr;
+  hydro_patch g_a = {}, g_b = {};
   int g_n = -1;
   double* g_dt = nullptr;
   int g_tile = -1, g_zc = -1;
@@ -1511,6 +1510,13 @@ int hydro_prim_to_cons_adjoint(hydro_ctx* c, const hydro_patch* W, const hydro_p
   return HYDRO_OK;
 }
 
+// The same arrays, sizes, strides and cell size: everything of a box that a captured step holds.
+static bool same_box(const hydro_patch& a, const hydro_patch& b) {
+  for (int v = 0; v < 5; ++v)
+    if (a.U[v] != b.U[v]) return false;
+  return a.nx == b.nx && a.ny == b.ny && a.nz == b.nz && a.sy == b.sy && a.sz == b.sz && a.dx == b.dx;
+}
+
 int hydro_run(hydro_ctx* c, const hydro_patch* a, const hydro_patch* b, int nsteps, double* dt_hist_dev,
               int use_graph) {
   if (!c || !a || !b || nsteps < 1 || !dt_hist_dev) return HYDRO_ERR_ARG;
@@ -1531,7 +1537,7 @@ int hydro_run(hydro_ctx* c, const hydro_patch* a, const hydro_patch* b, int nste
     return HYDRO_OK;
   };
   if (!use_graph) return enqueue(c->stream);
-  const bool hit = c->graph && c->g_a == a->U[0] && c->g_b == b->U[0] && c->g_n == nsteps && c->g_dt == dt_hist_dev &&
+  const bool hit = c->graph && same_box(c->g_a, *a) && same_box(c->g_b, *b) && c->g_n == nsteps && c->g_dt == dt_hist_dev &&
                    c->g_tile == c->tile_id && c->g_zc == c->zchunk && c->g_tuned == c->tuned;
   if (!hit) {
     if (c->graph) cudaGraphExecDestroy(c->graph);
@@ -1553,8 +1559,8 @@ int hydro_run(hydro_ctx* c, const hydro_patch* a, const hydro_patch* b, int nste
       c->graph = nullptr;
       return HYDRO_ERR_CUDA;
     }
-    c->g_a = a->U[0];
-    c->g_b = b->U[0];
+    c->g_a = *a;
+    c->g_b = *b;
     c->g_n = nsteps;
     c->g_dt = dt_hist_dev;
     c->g_tile = c->tile_id;
