@@ -128,10 +128,13 @@ struct hydro_ctx {
   // descriptors and block tables
   static constexpr int kAux = 6;  // 0, 1 box fluxes; 2 reflux; 3 average-down; 4 MHD step; 5 MHD CFL
   SetCache aux[kAux];
-  // oct builder scratch: key bitmap, word prefix sums, block prefix sums
+  // oct builder scratch: key bitmap, word prefix sums, block prefix sums; and, for eager calls only (a
+  // graph never holds the address of what a longer list makes the context replace), octs by key
   unsigned* d_octs_scratch = nullptr;
   size_t octs_scratch_cap = 0;
-  // oct step through the table: the list's cubes (OctCubes)
+  int* d_octs_slots = nullptr;
+  size_t octs_slots_cap = 0;
+  // oct step through the table: the list's cubes (OctCubes), for eager calls only too
   char* d_cubes = nullptr;
   size_t cubes_cap = 0;
   // MHD step scratch: constants, face states, fluxes
@@ -221,6 +224,18 @@ int ensure_device(T** d, size_t* cap, size_t n) {
   if (cudaMalloc(reinterpret_cast<void**>(d), n * sizeof(T)) != cudaSuccess) return HYDRO_ERR_NOMEM;
   *cap = n;
   return HYDRO_OK;
+}
+
+// Scratch that a call can do without, for eager calls only; false where it is captured or there is no
+// memory (that failure ends here).
+template <class T>
+bool eager_scratch(hydro_ctx* c, T** d, size_t* cap, size_t n) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone &&
+      ensure_device(d, cap, n) == HYDRO_OK)
+    return true;
+  cudaGetLastError();
+  return false;
 }
 
 template <class T>
@@ -593,6 +608,7 @@ int hydro_finalize(hydro_ctx* c) {
   c->xchg_sets.free_all();
   for (SetCache& s : c->aux) s.free_all();
   cudaFree(c->d_octs_scratch);
+  cudaFree(c->d_octs_slots);
   cudaFree(c->d_cubes);
   cudaFree(c->d_mhd);
   for (cudaEvent_t e : c->ev_copied) cudaEventDestroy(e);
@@ -1202,23 +1218,18 @@ int hydro_octs_build(hydro_ctx* c, const int* pos_dev, int noct, const int dims[
   }
   const size_t nwords = std::max<size_t>(1, ((size_t)1 << (3 * bits)) >> 5);
   const size_t nblocks = (nwords + 1023) / 1024;
-  // Octs by key as well, where the key space is at most eight times the octs (a refined half of a level
-  // per axis): beyond, clearing it costs more than the table's rank lookups; nor does a first call under
-  // capture, or one without the memory, grow the scratch for it.
-  const size_t base = 2 * nwords + nblocks, with_slots = base + 32 * nwords;
-  bool slots = nbr_dev && 32 * nwords <= 8 * (size_t)noct;
-  if (slots && c->octs_scratch_cap < with_slots) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    slots = cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
-            ensure_device(&c->d_octs_scratch, &c->octs_scratch_cap, with_slots) == HYDRO_OK;
-    if (!slots) cudaGetLastError();
-  }
-  int rc = ensure_device(&c->d_octs_scratch, &c->octs_scratch_cap, base);
+  int rc = ensure_device(&c->d_octs_scratch, &c->octs_scratch_cap, 2 * nwords + nblocks);
   if (rc) return rc;
+  // Octs by key as well, where the key space is at most eight times the octs (a refined half of a level
+  // per axis): beyond, clearing it costs more than the table's rank lookups.  A captured call, and one
+  // without the memory, looks ranks up.
+  const bool slots = nbr_dev && 32 * nwords <= 8 * (size_t)noct &&
+                     eager_scratch(c, &c->d_octs_slots, &c->octs_slots_cap, 32 * nwords);
   unsigned* bitmap = c->d_octs_scratch;
   c->launches += nbr_dev ? 5 : 4;
-  return cuda_status(hydro::launch_octs_build(pos_dev, noct, dims, bitmap, bitmap + nwords, bitmap + 2 * nwords,
-                                              nwords, slots ? reinterpret_cast<int*>(bitmap + base) : nullptr, order_dev, nbr_dev, c->d_err, c->stream));
+  return cuda_status(hydro::launch_octs_build(pos_dev, noct, dims, bitmap, bitmap + nwords, bitmap + 2 * nwords, nwords,
+                                              slots ? c->d_octs_slots : nullptr, order_dev, nbr_dev, c->d_err,
+                                              c->stream));
 }
 
 int hydro_step_octs_table(hydro_ctx* c, void* const in[5], void* const out[5], int noct, const int* nbr_dev,
@@ -1239,20 +1250,13 @@ int hydro_step_octs_table(hydro_ctx* c, void* const in[5], void* const out[5], i
       if (a < b + bytes && b < a + bytes) return HYDRO_ERR_ARG;
     }
   // A long list: its 4^3 cubes of octs are found first and stepped as boxes of 8^3 cells.  Lists too short
-  // for one cube per SM keep the one-oct kernel, as does a captured call or one whose scratch cannot be
-  // allocated.
-  const bool cubes_pay = ngroups >= 64LL * c->sm_count && ngroups <= 0x7fffffffLL - 64;
+  // for one cube per SM keep the one-oct kernel, which needs no scratch, as does a captured call (its graph
+  // then holds no memory of the context's) or one whose scratch cannot be allocated.
   hydro::OctCubes cubes;
   bool use = false;
-  if (cubes_pay) {
-    const size_t ints = 2 + (size_t)ngroups / 64 + (size_t)ngroups, need = ints * sizeof(int) + (size_t)ngroups;
-    use = need <= c->cubes_cap;
-    if (!use) {
-      cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-      use = cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
-            ensure_device(&c->d_cubes, &c->cubes_cap, need) == HYDRO_OK;
-      if (!use) cudaGetLastError();  // the allocation's failure is handled here
-    }
+  if (ngroups >= 64LL * c->sm_count && ngroups <= 0x7fffffffLL - 64) {
+    const size_t ints = 2 + (size_t)ngroups / 64 + (size_t)ngroups;
+    use = eager_scratch(c, &c->d_cubes, &c->cubes_cap, ints * sizeof(int) + (size_t)ngroups);
     if (use) {
       cubes.counts = reinterpret_cast<int*>(c->d_cubes);
       cubes.start = cubes.counts + 2;
