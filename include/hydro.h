@@ -25,7 +25,9 @@
  *     descriptors, the tile work-list and its counter, captured CUDA graphs, autotune results.
  *   - Every call is asynchronous on the context's stream, except hydro_get_error (and
  *     hydro_autotune), which synchronise it.  After a first call with a given patch set, calls
- *     with the same set allocate nothing and can be captured in a CUDA graph.
+ *     with the same set allocate nothing and can be captured in a CUDA graph.  What a graph reads
+ *     of the context's memory stays as it is until the graph and its executables are destroyed;
+ *     the context must outlive them, and their launches take their turn with its other calls'.
  *   - Argument errors are detected on the host and return HYDRO_ERR_ARG before anything is
  *     launched.  Physical errors found on the device set bits of the error word
  *     (HYDRO_EBIT_*), read back by hydro_get_error.  CUDA errors return HYDRO_ERR_CUDA.

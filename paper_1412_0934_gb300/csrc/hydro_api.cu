@@ -4,10 +4,12 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -18,11 +20,17 @@
 using hydro::HostPatchIO;
 using hydro::HostTileRec;
 
+// How many graphs hold an address: captured calls add to it, and the graph's and its executables' end
+// takes it back (graph_holds, below), from a thread of the driver's and perhaps after the context's end.
+using GraphRefs = std::shared_ptr<std::atomic<int>>;
+bool held(const GraphRefs& refs) { return refs && refs->load() > 0; }
+
 // What a call derives from its descriptors (field pointers, shapes, origins, boxes) and keeps on the
 // device: descriptor copies, block tables, copy tasks, work-lists.  The last kKept sets of each kind of
 // call stay, the least recently used making room: a level's patches step from one buffer set to another
 // and back, so consecutive calls alternate between sets (with one kept set, each substep of a subcycled
-// level rebuilt its tables and drained the stream for it).
+// level rebuilt its tables and drained the stream for it).  A set that a graph was captured with stays
+// beside them until that graph is gone.
 struct SetCache {
   static constexpr int kKept = 4;
   struct Entry {
@@ -33,23 +41,41 @@ struct SetCache {
     size_t cap = 0;
     size_t off[4] = {};  // offsets of the parts in d
     int n[10] = {};      // counts and settings of the set
+    GraphRefs graphs;
   };
-  Entry entry[kKept];
+  std::vector<std::unique_ptr<Entry>> entry;
   unsigned long long clock = 0;
   Entry* find(const std::vector<char>& key) {
-    for (Entry& e : entry)
-      if (e.valid && e.key == key) {
-        e.used = ++clock;
-        return &e;
+    for (auto& e : entry)
+      if (e->valid && e->key == key) {
+        e->used = ++clock;
+        return e.get();
       }
     return nullptr;
   }
   // The entry to fill for a new key, with room for n bytes (nullptr: no memory); valid once the
   // caller has enqueued its contents and calls done().
   Entry* replace(size_t n) {
-    Entry* o = &entry[0];
-    for (Entry& e : entry)
-      if (e.used < o->used) o = &e;
+    Entry* o = nullptr;
+    for (;;) {  // the least recently used of kKept sets that no graph holds; sets beyond those are freed
+      size_t oldest = 0;
+      int free_sets = 0;
+      for (size_t i = 0; i < entry.size(); ++i)
+        if (!held(entry[i]->graphs)) {
+          if (free_sets++ == 0 || entry[i]->used < entry[oldest]->used) oldest = i;
+        }
+      if (free_sets < kKept) {
+        entry.emplace_back(new Entry);
+        o = entry.back().get();
+        break;
+      }
+      if (free_sets == kKept) {
+        o = entry[oldest].get();
+        break;
+      }
+      cudaFree(entry[oldest]->d);
+      entry.erase(entry.begin() + oldest);
+    }
     o->valid = false;
     if (o->cap < n) {
       cudaFree(o->d);
@@ -66,8 +92,16 @@ struct SetCache {
     e->valid = true;
   }
   void free_all() {
-    for (Entry& e : entry) cudaFree(e.d);
+    for (auto& e : entry) cudaFree(e->d);
   }
+};
+
+// Device scratch that grows with the largest call; what a graph holds is set aside, not freed, when a
+// larger block takes its place.
+struct Scratch {
+  char* d = nullptr;
+  size_t cap = 0;
+  GraphRefs graphs;
 };
 
 struct hydro_ctx {
@@ -104,8 +138,8 @@ struct hydro_ctx {
   int g_tile = -1, g_zc = -1;
   bool g_tuned = false;
   // adjoint scratch
-  void* d_adj = nullptr;
-  size_t adj_cap = 0;
+  Scratch adj;
+  std::vector<Scratch> aside;  // outgrown blocks that graphs held
   // host-buffer step: device staging of one box (in and out), its descriptor and slab tile list,
   // per-slab tile counters, the two copy streams and the events that chain the pipeline
   char* d_stage = nullptr;
@@ -130,16 +164,14 @@ struct hydro_ctx {
   SetCache aux[kAux];
   // oct builder scratch: key bitmap, word prefix sums, block prefix sums; and, for eager calls only (a
   // graph never holds the address of what a longer list makes the context replace), octs by key
-  unsigned* d_octs_scratch = nullptr;
-  size_t octs_scratch_cap = 0;
+  Scratch octs;
   int* d_octs_slots = nullptr;
   size_t octs_slots_cap = 0;
   // oct step through the table: the list's cubes (OctCubes), for eager calls only too
   char* d_cubes = nullptr;
   size_t cubes_cap = 0;
   // MHD step scratch: constants, face states, fluxes
-  char* d_mhd = nullptr;
-  size_t mhd_cap = 0;
+  Scratch mhd;
   long long launches = 0;
 };
 
@@ -226,6 +258,55 @@ int ensure_device(T** d, size_t* cap, size_t n) {
   return HYDRO_OK;
 }
 
+// Where the context's stream is being captured: the graph takes a reference to `refs`, which it drops when
+// it and the executables made of it are destroyed.
+int graph_holds(hydro_ctx* c, GraphRefs& refs) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  cudaGraph_t g = nullptr;
+  if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess) return HYDRO_ERR_CUDA;
+  if (cs == cudaStreamCaptureStatusNone) return HYDRO_OK;
+  if (cudaStreamGetCaptureInfo(c->stream, &cs, nullptr, &g) != cudaSuccess || cs != cudaStreamCaptureStatusActive)
+    return HYDRO_ERR_CUDA;
+  if (!refs) refs = std::make_shared<std::atomic<int>>(0);
+  GraphRefs* mine = new GraphRefs(refs);
+  cudaUserObject_t object;
+  auto drop = [](void* p) {
+    GraphRefs* r = static_cast<GraphRefs*>(p);
+    --**r;
+    delete r;
+  };
+  if (cudaUserObjectCreate(&object, mine, drop, 1, cudaUserObjectNoDestructorSync) != cudaSuccess) {
+    delete mine;
+    return HYDRO_ERR_CUDA;
+  }
+  ++*refs;
+  if (cudaGraphRetainUserObject(g, object, 1, cudaGraphUserObjectMove) != cudaSuccess) {
+    cudaUserObjectRelease(object, 1);  // runs drop
+    return HYDRO_ERR_CUDA;
+  }
+  return HYDRO_OK;
+}
+
+// At least n bytes of scratch, held by the graph where the call is captured.
+int ensure_scratch(hydro_ctx* c, Scratch& s, size_t n) {
+  if (s.cap < n) {
+    if (held(s.graphs)) {
+      c->aside.push_back(s);
+    } else {
+      cudaFree(s.d);
+    }
+    s = Scratch();
+    for (size_t i = c->aside.size(); i-- > 0;)
+      if (!held(c->aside[i].graphs)) {
+        cudaFree(c->aside[i].d);
+        c->aside.erase(c->aside.begin() + i);
+      }
+    if (cudaMalloc(&s.d, n) != cudaSuccess) return HYDRO_ERR_NOMEM;
+    s.cap = n;
+  }
+  return graph_holds(c, s.graphs);
+}
+
 // Scratch that a call can do without, for eager calls only; false where it is captured or there is no
 // memory (that failure ends here).
 template <class T>
@@ -279,7 +360,7 @@ SetCache::Entry* new_entry(hydro_ctx* c, SetCache& cache, size_t n, int* rc) {
 
 // The entry holding `bytes` on the device, uploaded unless one of the last sets has them.
 SetCache::Entry* upload_set(hydro_ctx* c, SetCache& cache, std::vector<char>&& bytes) {
-  if (SetCache::Entry* e = cache.find(bytes)) return e;
+  if (SetCache::Entry* e = cache.find(bytes)) return graph_holds(c, e->graphs) ? nullptr : e;
   int rc;
   SetCache::Entry* e = new_entry(c, cache, bytes.size(), &rc);
   if (!e || !upload(c, e->d, bytes.data(), bytes.size())) return nullptr;
@@ -427,7 +508,7 @@ int prepare_batch(hydro_ctx* c, const hydro_patch* in, const hydro_patch* out, i
     setting[2 * NC + 1] = zchunk;
   }
   append(key, setting, 2 * NC + 2);
-  if ((*entry = c->batch.find(key))) return HYDRO_OK;
+  if ((*entry = c->batch.find(key))) return graph_holds(c, (*entry)->graphs);
   if (!pc && !c->tuned) default_tuning(c, in, n, &tile, &zchunk);
   // patches by class (all in class 0 without a tile shape per class) and tiles per class: the counts on
   // the host size the buffer, the device builds the list itself
@@ -594,7 +675,7 @@ int hydro_finalize(hydro_ctx* c) {
   cudaFree(c->d_err);
   cudaFree(c->d_counter);
   cudaFree(c->d_cls_dt);
-  cudaFree(c->d_adj);
+  cudaFree(c->adj.d);
   if (c->s_h2d) cudaStreamSynchronize(c->s_h2d);
   if (c->s_d2h) cudaStreamSynchronize(c->s_d2h);
   if (c->s_cmp2) cudaStreamSynchronize(c->s_cmp2);
@@ -607,10 +688,11 @@ int hydro_finalize(hydro_ctx* c) {
   c->ghost_sets.free_all();
   c->xchg_sets.free_all();
   for (SetCache& s : c->aux) s.free_all();
-  cudaFree(c->d_octs_scratch);
+  cudaFree(c->octs.d);
   cudaFree(c->d_octs_slots);
   cudaFree(c->d_cubes);
-  cudaFree(c->d_mhd);
+  cudaFree(c->mhd.d);
+  for (Scratch& s : c->aside) cudaFree(s.d);
   for (cudaEvent_t e : c->ev_copied) cudaEventDestroy(e);
   for (cudaEvent_t e : c->ev_stepped) cudaEventDestroy(e);
   for (cudaEvent_t e : c->ev_halo) cudaEventDestroy(e);
@@ -648,6 +730,7 @@ int hydro_cfl_dt(hydro_ctx* c, const hydro_patch* p, int npatch, double* dt_dev)
     if (!upload(c, e->d, io.data(), io.size() * sizeof(io[0]))) return HYDRO_ERR_CUDA;
     c->cfl_sets.done(e, std::move(key));
   }
+  if ((rc = graph_holds(c, e->graphs))) return rc;
   HostPatchIO big = make_io(p[0], p[0]);
   c->launches += 1;
   return cuda_status(c->ops->cfl(reinterpret_cast<const HostPatchIO*>(e->d), big, npatch, c->prm, dt_dev, c->d_err, c->stream));
@@ -941,6 +1024,7 @@ static int fill_ghosts_impl(hydro_ctx* c, const hydro_patch* coarse, const hydro
     e->n[0] = (int)blocks.size();
     c->ghost_sets.done(e, std::move(key));
   }
+  if (int rc = graph_holds(c, e->graphs)) return rc;
   c->launches += 1;
   const HostPatchIO old = coarse_old ? make_io(*coarse_old, *coarse_old) : make_io(C, C);
   return cuda_status(hydro::launch_fill_ghosts(elem_size(c), reinterpret_cast<const hydro::HostGhostPatch*>(e->d),
@@ -1186,6 +1270,7 @@ int hydro_exchange_ghosts(hydro_ctx* c, const hydro_patch* fine, const int* orig
     e->n[0] = (int)tasks.size();
     c->xchg_sets.done(e, std::move(key));
   }
+  if (int rc = graph_holds(c, e->graphs)) return rc;
   if (e->n[0] == 0) return HYDRO_OK;
   c->launches += 1;
   return cuda_status(hydro::launch_copy_boxes(elem_size(c), reinterpret_cast<const hydro::HostGhostPatch*>(e->d),
@@ -1218,14 +1303,14 @@ int hydro_octs_build(hydro_ctx* c, const int* pos_dev, int noct, const int dims[
   }
   const size_t nwords = std::max<size_t>(1, ((size_t)1 << (3 * bits)) >> 5);
   const size_t nblocks = (nwords + 1023) / 1024;
-  int rc = ensure_device(&c->d_octs_scratch, &c->octs_scratch_cap, 2 * nwords + nblocks);
+  int rc = ensure_scratch(c, c->octs, (2 * nwords + nblocks) * sizeof(unsigned));
   if (rc) return rc;
   // Octs by key as well, where the key space is at most eight times the octs (a refined half of a level
   // per axis): beyond, clearing it costs more than the table's rank lookups.  A captured call, and one
   // without the memory, looks ranks up.
   const bool slots = nbr_dev && 32 * nwords <= 8 * (size_t)noct &&
                      eager_scratch(c, &c->d_octs_slots, &c->octs_slots_cap, 32 * nwords);
-  unsigned* bitmap = c->d_octs_scratch;
+  unsigned* bitmap = reinterpret_cast<unsigned*>(c->octs.d);
   c->launches += nbr_dev ? 5 : 4;
   return cuda_status(hydro::launch_octs_build(pos_dev, noct, dims, bitmap, bitmap + nwords, bitmap + 2 * nwords, nwords,
                                               slots ? c->d_octs_slots : nullptr, order_dev, nbr_dev, c->d_err,
@@ -1304,8 +1389,7 @@ int hydro_mhd_step(hydro_ctx* c, void* const in[9], void* const out[9], int nx, 
       const uintptr_t a = reinterpret_cast<uintptr_t>(out[v]), b = reinterpret_cast<uintptr_t>(in[u]);
       if (a < b + bytes && b < a + bytes) return HYDRO_ERR_ARG;
     }
-  int rc = ensure_device(&c->d_mhd, &c->mhd_cap,
-                         hydro::mhd_scratch_bytes(c->cfg.precision, nx, ny, nz, elem_size(c)));
+  int rc = ensure_scratch(c, c->mhd, hydro::mhd_scratch_bytes(c->cfg.precision, nx, ny, nz, elem_size(c)));
   if (rc) return rc;
   if (dt_next_dev) {
     rc = reset_slots(c, dt_next_dev, 1, c->stream);
@@ -1313,7 +1397,7 @@ int hydro_mhd_step(hydro_ctx* c, void* const in[9], void* const out[9], int nx, 
   }
   c->launches += hydro::mhd_step_launches(c->cfg.precision);
   return cuda_status(hydro::launch_mhd_step(c->cfg.precision, mhd_box(in, out, nx, ny, nz, dx), c->prm, dt_dev,
-                                            dt_next_dev, c->d_mhd, c->d_err, c->stream));
+                                            dt_next_dev, c->mhd.d, c->d_err, c->stream));
 }
 
 int hydro_mhd_cfl_dt(hydro_ctx* c, void* const U[9], int nx, int ny, int nz, double dx, double* dt_dev) {
@@ -1414,7 +1498,7 @@ int hydro_mhd_step_patches(hydro_ctx* c, const hydro_mhd_patch* in, const hydro_
   size_t elems = 0;
   int rc = mhd_patch_tables(c, 4, in, out, npatch, true, &dp, &db, &nb, &elems);
   if (rc) return rc;
-  rc = ensure_device(&c->d_mhd, &c->mhd_cap, hydro::mhd_patch_consts_bytes(npatch) + elems * elem_size(c));
+  rc = ensure_scratch(c, c->mhd, hydro::mhd_patch_consts_bytes(npatch) + elems * elem_size(c));
   if (rc) return rc;
   if (dt_next_dev) {
     rc = reset_slots(c, dt_next_dev, npatch, c->stream);
@@ -1422,7 +1506,7 @@ int hydro_mhd_step_patches(hydro_ctx* c, const hydro_mhd_patch* in, const hydro_
   }
   c->launches += hydro::mhd_step_launches(c->cfg.precision);
   return cuda_status(hydro::launch_mhd_patches(c->cfg.precision, dp, db, nb, npatch, c->prm, dt_dev, dt_next_dev,
-                                               c->d_mhd, c->d_err, c->stream));
+                                               c->mhd.d, c->d_err, c->stream));
 }
 
 int hydro_mhd_cfl_patches(hydro_ctx* c, const hydro_mhd_patch* p, int npatch, double* dt_dev) {
@@ -1461,18 +1545,13 @@ int hydro_adjoint_step(hydro_ctx* c, const hydro_patch* U_n, const double* dt_de
   for (int i = 0; i < npatch; ++i) {
     const hydro_patch &U = U_n[i], &L = lam_np1[i], &O = lam_n[i];
     const size_t need = aops->adjoint_scratch_bytes(U.nx, U.ny, U.nz);
-    if (need > c->adj_cap) {
-      cudaFree(c->d_adj);
-      c->d_adj = nullptr;
-      c->adj_cap = 0;
-      if (cudaMalloc(&c->d_adj, need) != cudaSuccess) return HYDRO_ERR_NOMEM;
-      c->adj_cap = need;
-    }
+    const int rc = ensure_scratch(c, c->adj, need);
+    if (rc) return rc;
     void* outp[5];
     for (int v = 0; v < 5; ++v) outp[v] = O.U[v];
     HostPatchIO lam = make_io(L, O);
     c->launches += 2;
-    cudaError_t e = aops->adjoint(make_io(U, O), lam, outp, c->prm, dt_dev + i, c->d_adj, c->adj_cap, c->d_err,
+    cudaError_t e = aops->adjoint(make_io(U, O), lam, outp, c->prm, dt_dev + i, c->adj.d, c->adj.cap, c->d_err,
                                   c->stream);
     if (e == cudaErrorNotSupported) return HYDRO_ERR_STATE;
     if (e != cudaSuccess) return HYDRO_ERR_CUDA;

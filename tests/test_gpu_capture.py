@@ -123,3 +123,134 @@ def test_oct_graph_outlives_longer_lists(with_table):
         assert all(bool((k == 0x5a5a5a5a).all()) for k in keep)
         assert hy.hydro_get_error(ctx) == (hy.HYDRO_OK, 0)
         hy.hydro_finalize(ctx)
+
+
+N = 16
+
+
+def _patches(seed, grow):
+    """A coarse box and three fine patches of it (edges grown by `grow`), ghosts still to be filled."""
+    coarse = _gas(N, seed)
+    dims = [(12 + grow, 8, 10), (6, 8 + grow, 10), (14, 6, 8 + grow)]
+    ins = [torch.zeros((5, z + 4, y + 4, x + 4), dtype=torch.float64, device="cuda") for x, y, z in dims]
+    fine = _gas(2 * N, seed + 50)
+    origins = [(2, 4, 6), (18, 4, 6), (2, 20, 18)]
+    for t, o, (x, y, z) in zip(ins, origins, dims):
+        ix, iy, iz = ((torch.arange(n, device="cuda") + s) % (2 * N) for n, s in zip((x, y, z), o))
+        t[:, 2:-2, 2:-2, 2:-2] = fine[:, iz][:, :, iy][:, :, :, ix]
+    return coarse, origins, dims, ins
+
+
+class _Level:
+    """One patch set's calls and their buffers."""
+
+    def __init__(self, ctx, seed, grow):
+        self.ctx, self.data = ctx, _patches(seed, grow)
+        coarse, self.origins, self.dims, ins = self.data
+        self.ins = [t.clone() for t in ins]
+        self.outs = [torch.zeros_like(t) for t in ins]
+        self.regs = [torch.zeros(5 * hy.register_size(*d), dtype=torch.float64, device="cuda") for d in self.dims]
+        self.dt = torch.full((3,), 2e-3, dtype=torch.float64, device="cuda")
+        self.dn, self.cfl = torch.empty_like(self.dt), torch.empty_like(self.dt)
+        self.c = hy.patch(coarse, 0, 1.0 / N)
+        self.a, self.b = ([hy.patch(t, 2, 0.5 / N) for t in T] for T in (self.ins, self.outs))
+
+    def calls(self):
+        hy.hydro_fill_ghosts(self.ctx, self.c, self.a, self.origins)
+        hy.hydro_exchange_ghosts(self.ctx, self.a, self.origins, (2 * N,) * 3)
+        hy.hydro_patch_fluxes(self.ctx, self.a, self.dt, self.regs)
+        hy.hydro_step(self.ctx, self.a, self.b, self.dt, self.dn)
+        hy.hydro_cfl_dt(self.ctx, self.a, self.cfl)
+
+    def results(self):
+        return self.ins + self.outs + self.regs + [self.dn, self.cfl]
+
+    def clear(self):
+        for t, u in zip(self.ins, self.data[3]):
+            t.copy_(u)
+        for t in self.outs + self.regs + [self.dn, self.cfl]:
+            t.zero_()
+
+
+def test_patch_graphs_outlive_other_sets():
+    """Patch sets' calls captured, more sets than a context keeps, each before the next comes; then other
+    and larger sets; then every graph again.  Graphs that are gone leave their sets to the others."""
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(stream):
+        ctx = hy.hydro_init(precision="fp64")
+        for rounds in range(2):
+            levels, graphs, want = [], [], []
+            for seed in range(6):
+                lv = _Level(ctx, seed, 0)
+                lv.calls()
+                stream.synchronize()
+                want.append([t.clone() for t in lv.results()])
+                lv.clear()
+                graphs.append(_captured(stream, lv.calls))
+                levels.append(lv)
+            others = [_Level(ctx, seed, 2 + seed % 7) for seed in range(20, 30)]
+            for lv in others + others[::-1]:
+                lv.calls()
+            keep = _eaters()
+            for k in (3, 0, 5, 1, 4, 2, 0):
+                levels[k].clear()
+                graphs[k].replay()
+                stream.synchronize()
+                assert all(torch.equal(g, w) for g, w in zip(levels[k].results(), want[k]))
+            assert all(bool((e == 0x5a5a5a5a).all()) for e in keep)
+            for lv in others:  # eager calls beside the graphs
+                first = [t.clone() for t in lv.results()]
+                lv.clear()
+                lv.calls()
+                assert all(torch.equal(g, w) for g, w in zip(lv.results(), first))
+            del graphs
+            stream.synchronize()
+        assert hy.hydro_get_error(ctx) == (hy.HYDRO_OK, 0)
+        hy.hydro_finalize(ctx)
+
+
+def test_scratch_graphs_outlive_larger_calls():
+    """The calls with per-cell scratch (reverse step, MHD in double, the oct builder), captured on a small
+    box; then larger boxes; then the replay."""
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(stream):
+        ctx = hy.hydro_init(precision="fp64")
+        dt = torch.full((1,), 1e-3, dtype=torch.float64, device="cuda")
+
+        def work(n, seed):
+            U, lam, res = _gas(n, seed), _gas(n, seed + 1), torch.zeros((5, n, n, n), dtype=torch.float64, device="cuda")
+            M = torch.cat([U, 0.1 * _gas(n, seed + 2)[1:], ])
+            M[4] += 1.0
+            mout = torch.zeros_like(M)
+            z, y, x = torch.meshgrid(*[torch.arange(n, device="cuda", dtype=torch.int32)] * 3, indexing="ij")
+            pos = torch.stack([x, y, z], dim=-1).reshape(-1, 3).contiguous()
+            order = torch.empty(len(pos), dtype=torch.int32, device="cuda")
+            nbr = torch.empty((len(pos), 27), dtype=torch.int32, device="cuda")
+            pu, pl, pr = hy.patch(U, 0, 1.0 / n), hy.patch(lam, 0, 1.0 / n), hy.patch(res, 0, 1.0 / n)
+
+            def calls():
+                hy.hydro_adjoint_step(ctx, pu, dt, pl, pr)
+                hy.hydro_mhd_step(ctx, M, mout, 1.0 / n, dt)
+                hy.hydro_octs_build(ctx, pos, (n, n, n), order, nbr)
+            return calls, (res, mout, order, nbr), (pu, pl, M, pos)
+
+        calls, out, _keep = work(12, 1)
+        calls()
+        stream.synchronize()
+        want = [t.clone() for t in out]
+        graph = _captured(stream, calls)
+        for n in (20, 36):
+            work(n, 5)[0]()
+            stream.synchronize()
+        keep = _eaters()
+        for _ in range(2):
+            for t in out:
+                t.zero_()
+            graph.replay()
+            stream.synchronize()
+            assert all(torch.equal(g, w) for g, w in zip(out, want))
+        assert all(bool((e == 0x5a5a5a5a).all()) for e in keep)
+        hy.hydro_clear_error(ctx)
+        hy.hydro_finalize(ctx)
