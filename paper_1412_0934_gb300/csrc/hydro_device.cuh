@@ -875,10 +875,12 @@ struct PolDF {
 };
 
 // CFL speed of a recovered state.
-template <class R>
-__device__ __forceinline__ R cfl_speed(const R q[5], R gamma) {
-  const R c = rsqrt_(gamma * q[4] * rcp_(q[0]));
+__device__ __forceinline__ float cfl_speed(const float q[5], float gamma) {
+  const float c = rsqrt_(gamma * q[4] * rcp_(q[0]));
   return ((rabs(q[1]) + rabs(q[2])) + rabs(q[3])) + mulf_(c, 3.f);
+}
+__device__ __forceinline__ double cfl_speed(const double q[5], double gamma) {
+  return fma(sound_speed(gamma * q[4], q[0]), 3.0, (rabs(q[1]) + rabs(q[2])) + rabs(q[3]));
 }
 
 // CFL speed of a stored state (the step's epilogue and the standalone dt kernel share it, so

@@ -54,6 +54,7 @@ def _on_gpu(U):
 
 
 @pytest.mark.parametrize("precision,kind,mach,bound", [
+    ("fp64", "white", 0.3, 1.087e-16), ("fp64", "white", 1.0, 1.004e-16), ("fp64", "cold", 2.0, 1.387e-16),
     ("df64", "white", 0.3, 2.908e-15), ("df64", "white", 1.0, 2.621e-15), ("df64", "cold", 2.0, 6.002e-15),
     ("df64", "cold", 5.0, 1.904e-14)])
 def test_time_step_error(precision, kind, mach, bound):
