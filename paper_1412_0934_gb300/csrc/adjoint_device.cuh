@@ -68,14 +68,9 @@ __device__ __forceinline__ void hllc_core_adj(const R qL[5], const R qR[5], R ke
   const R mL = qL[0] * (SL - uL);
   const R mR = qR[0] * (SR - uR);
   const R den = mL - mR;
-  const R iden = rcp_(den);
-  R Ss;  // S* = num / den, num = p_R - p_L + u_L m_L - u_R m_R; in double as the forward flux forms it
-  if constexpr (std::is_same<R, double>::value) {
-    Ss = uL + contact_offset(qL, qR, mR, uL - uR, den);
-  } else {
-    const R num = qR[4] - qL[4] + uL * mL - uR * mR;
-    Ss = num * iden;
-  }
+  const R num = qR[4] - qL[4] + uL * mL - uR * mR;
+  const R iden = rcp_(den);  // S* = num / den; its sign (the only branch it decides) is exact
+  const R Ss = num * iden;
   const bool SLneg = cmp_neg(SL), SRpos = cmp_pos(SR);
   const bool star = SLneg && SRpos;
   const bool left = !SLneg || (SRpos && !cmp_neg(Ss));

@@ -2,12 +2,16 @@
 plain formulas in correctly rounded double operations and in normalising double-float operators.  The bounds
 are those formulas' errors on the same inputs, measured once (the time step's and double-float's with 1%
 added: rounding takes another course at each change)."""
+import ctypes
 import math
+import os
+import subprocess
 
 import numpy as np
 import pytest
 import torch
 
+import oracle
 import paper_1412_0934_gb300 as hy
 from hydro_testlib import GAMMA, ctx
 
@@ -88,3 +92,50 @@ def test_double_float_step_error(limiter, kind, mach, bounds):
         hy.hydro_finalize(c)
     err = ((out["df64"] - out["fp64"]).norm(dim=1) / out["fp64"].norm(dim=1)).cpu().numpy()
     assert (err <= 1.01 * np.array(bounds)).all(), err
+
+
+@pytest.fixture(scope="module")
+def extended_step(tmp_path_factory):
+    """The oracle's periodic step in extended precision: the same sources with long double for double."""
+    d = tmp_path_factory.mktemp("extended")
+    here = os.path.dirname(os.path.abspath(oracle.__file__))
+    with open(str(d / "capi.cpp"), "w") as f:
+        f.write("".join("#include <%s>\n" % h for h in ("algorithm", "cmath", "cstdint", "cstring", "vector", "type_traits")))
+        f.write("#include <omp.h>\n#define double long double\n#include \"oracle_capi.cpp\"\n")
+    so = str(d / "extended.so")
+    subprocess.check_call(oracle._build.command([str(d / "capi.cpp")], so) + ["-I" + here])
+    lib = ctypes.CDLL(so)
+
+    class Config(ctypes.Structure):
+        _fields_ = [(n, ctypes.c_longdouble) for n in ("gamma", "cfl", "rho_floor", "p_floor")] + [("limiter", ctypes.c_int)]
+
+    vp, ld, i = ctypes.c_void_p, ctypes.c_longdouble, ctypes.c_int
+    lib.oracle_step_periodic.argtypes = [ctypes.POINTER(Config), vp, vp, i, i, i, ld, ld]
+
+    def step(U, dx, dt, limiter):
+        U = np.ascontiguousarray(U, dtype=LD)
+        out = np.empty_like(U)
+        cfg = Config(GAMMA, 0.8, 1e-10, 1e-14, oracle.LIMITERS[limiter])
+        assert lib.oracle_step_periodic(ctypes.byref(cfg), U.ctypes.data, out.ctypes.data, *U.shape[:0:-1], dx, dt) == 0
+        return out
+
+    return step
+
+
+def test_double_step_error(extended_step):
+    """White noise at Mach 3, where every face's wave speeds and contact matter."""
+    n, total, norm = 32, np.zeros(5), np.zeros(5)
+    c = ctx("fp64", cfl=0.8)
+    for seed in range(4):
+        U = _white(np.random.default_rng(seed), (n,) * 3, 3.0)
+        a = torch.from_numpy(U).cuda()
+        b, dt = torch.empty_like(a), torch.empty(1, dtype=torch.float64, device="cuda")
+        hy.hydro_cfl_dt(c, hy.patch(a, 0, 1.0 / n), dt)
+        hy.hydro_step(c, hy.patch(a, 0, 1.0 / n), hy.patch(b, 0, 1.0 / n), dt)
+        want = extended_step(U, 1.0 / n, dt.item(), "minmod")
+        err = (b.cpu().numpy() - want).astype(np.float64)
+        total += (err ** 2).reshape(5, -1).sum(1)
+        norm += (want ** 2).astype(np.float64).reshape(5, -1).sum(1)
+    hy.hydro_finalize(c)
+    err = np.sqrt(total / norm)
+    assert (err <= np.array([6.079e-17, 9.613e-17, 9.596e-17, 9.335e-17, 1.186e-16])).all(), err
