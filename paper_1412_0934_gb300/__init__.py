@@ -225,9 +225,10 @@ def _struct_array(struct, patches):
     """C array of the patches' descriptors, and their number: the structures' bytes joined in one go (a
     level holds thousands of patches; assigning them one by one took longer than the call's kernels)."""
     n = len(patches)
-    if n == 1:
-        return (struct * 1)(patches[0].c), 1
-    return (struct * n).from_buffer_copy(b"".join([p.c for p in patches])) if n else (struct * 0)(), n
+    cs = [p.c for p in patches]
+    if n < 2 or set(map(type, cs)) != {struct}:  # (another structure's bytes: refused here, with TypeError)
+        return (struct * n)(*cs), n
+    return (struct * n).from_buffer_copy(b"".join(cs)), n
 
 
 def _parray(patches):
