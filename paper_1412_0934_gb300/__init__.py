@@ -375,12 +375,11 @@ def register_size(nx, ny, nz):
 
 def _ints(rows):
     """C ints of the rows' values, in order."""
-    rows = list(rows)
+    values = list(itertools.chain.from_iterable(rows))
     try:
-        flat = array.array("i", list(itertools.chain.from_iterable(rows)))
+        flat = array.array("i", values)
     except (TypeError, OverflowError):  # values that int() converts and an int array does not take
-        flat = [int(v) for r in rows for v in r]
-        return (ctypes.c_int * len(flat))(*flat)
+        return (ctypes.c_int * len(values))(*[int(v) for v in values])
     return (ctypes.c_int * len(flat)).from_buffer(flat) if len(flat) else (ctypes.c_int * 0)()
 
 

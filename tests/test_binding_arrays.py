@@ -33,3 +33,13 @@ def test_descriptors_of_the_other_kind_are_refused(n):
         hy._struct_array(hy.hydro_mhd_patch, _descriptors(hy.hydro_patch, n))
     with pytest.raises(TypeError):
         hy._struct_array(hy.hydro_patch, _descriptors(hy.hydro_patch, n) + _descriptors(hy.hydro_mhd_patch, 1))
+
+
+@pytest.mark.parametrize("convert", [list, tuple, iter, lambda r: map(float, r)])
+@pytest.mark.parametrize("outer", [list, iter])
+def test_integers_from_any_rows(convert, outer):
+    """Rows may be iterators, and values anything int() takes."""
+    rows = [(1, 2, 3), (4.0, 5, True), (7, 8.9, 2 ** 31)]
+    got = hy._ints(outer([convert(r) for r in rows]))
+    assert list(got) == [1, 2, 3, 4, 5, 1, 7, 8, ctypes.c_int(2 ** 31).value]
+    assert list(hy._ints([])) == []
