@@ -356,7 +356,8 @@ int hydro_prim_to_cons_adjoint(hydro_ctx* ctx, const hydro_patch* W, const hydro
  * dt_hist_dev[n] and writes dt_hist_dev[n+1] = CFL dt of its result; states ping-pong between
  * a (even n) and b (odd n), so the result is in a if nsteps is even, else in b.
  * dt_hist_dev: device array of nsteps + 1 doubles.  With use_graph != 0 the nsteps launches are
- * captured once into a CUDA graph (cached in the context for the same a, b, nsteps, dt_hist_dev)
+ * captured once into a CUDA graph (cached in the context for the same a, b (arrays, sizes, strides
+ * and cell size), nsteps, dt_hist_dev and tuning)
  * and replayed. */
 int hydro_run(hydro_ctx* ctx, const hydro_patch* a, const hydro_patch* b, int nsteps, double* dt_hist_dev,
               int use_graph);
@@ -391,7 +392,8 @@ int hydro_autotune(hydro_ctx* ctx, const hydro_patch* in, const hydro_patch* out
 
 /* Current tile configuration: *tile_id (index into the compiled tile shapes) and *zchunk (no
  * counterpart in the paper).  A context that no call has tuned reports 0, 32; its hydro_step and
- * hydro_run then choose tile and chunk per box or patch set by a cost rule (the results are the same).  Compiled shapes (columns x rows of one block's tile): 0 16 x 16,
+ * hydro_run then choose tile and chunk per box or patch set by a cost rule (a cell's operations are
+ * the same in every tile).  Compiled shapes (columns x rows of one block's tile): 0 16 x 16,
  * 1 32 x 8, 2 8 x 8, 3 32 x 16, 4 16 x 16 with a whole SM's registers for one block; the PPM
  * kernel has one shape (16 x 16) and ignores tile_id.  hydro_set_tuning refuses tile_id outside
  * [0, HYDRO_NUM_TILES) and zchunk outside [1, 4096]. */

@@ -125,8 +125,9 @@ struct hydro_ctx {
   double* d_cls_dt = nullptr;  // the autotuner's per-class time steps
   size_t cls_dt_cap = 0;
   SetCache cfl_sets;  // CFL of many patches: descriptors
-  // tuning; until a caller sets it (hydro_set_tuning, hydro_set_class_tuning, hydro_autotune), hydro_step
-  // and hydro_run take each box's and patch set's tile shape and z chunk from the rule of default_tuning
+  // tuning; until a caller sets it (hydro_set_tuning, hydro_autotune), hydro_step and hydro_run take each
+  // box's and patch set's tile shape and z chunk from the rule of default_tuning (a batch with a tile shape
+  // per class, hydro_set_class_tuning, takes those, and 16x16 tiles of 32 planes for the other classes)
   int tile_id = 0, zchunk = 32;
   bool tuned = false;
   int rule_n[3] = {0, 0, 0}, rule_tile = 0, rule_zc = 0;  // the rule's choice for the last box size

@@ -170,9 +170,10 @@ cudaError_t launch_cfl(const HostPatchIO* d_patches, const HostPatchIO& single, 
 // recovered into shared memory; the 32 cells next to the oct's faces (the oct and the 24 outside
 // neighbours across its faces) are predicted; 32 of the oct's 36 faces get their HLLC fluxes, one per
 // lane.  The other four (the upper z faces) and the oct's 8 updates would leave most lanes idle, so
-// they wait in shared memory for the batch's end: 8 groups' 32 left faces make one full round and their
-// 64 updates two (float; 4 groups in 8-byte arithmetic, whose scratch is twice as large).  A group of
-// its own took two face rounds and one update round.  Local coordinates run from -2 to 3 (stored at +2).
+// they wait in shared memory for the batch's end: four groups' 16 left faces share one round and their 32
+// updates fill one, where a group of its own took a second face round and an update round for itself (eight
+// groups would fill the left faces' round too, but their scratch leaves too few warps per SM: 262144 groups,
+// mixed, 558 us against 392).  Local coordinates run from -2 to 3 (stored at +2).
 __device__ __forceinline__ bool oct_needed(int x, int y, int z) {
   const int ox = (x < 0 || x > 1), oy = (y < 0 || y > 1), oz = (z < 0 || z > 1);
   const int nout = ox + oy + oz;
@@ -201,8 +202,7 @@ __device__ __forceinline__ int oct_eindex(int x, int y, int z) {
 }
 
 constexpr int kOctWarps = 4;
-template <class Pol>
-constexpr int oct_batch() { return 4; }
+constexpr int kOctBatch = 4;
 
 template <class Pol>
 struct OctSmem {
@@ -210,8 +210,8 @@ struct OctSmem {
   R q[kOctWarps][5][80];      // needed cells in the order of need[]
   R qh[kOctWarps][5][32];
   R sl[kOctWarps][3][5][32];  // kept slopes
-  R f[kOctWarps][oct_batch<Pol>()][5][36];
-  R left[kOctWarps][oct_batch<Pol>()][10][4];  // lower and upper states of the upper z faces
+  R f[kOctWarps][kOctBatch][5][36];
+  R left[kOctWarps][kOctBatch][10][4];  // lower and upper states of the upper z faces
   short need[80], at[216];    // needed cell -> stencil cell, and back
 };
 
@@ -678,7 +678,7 @@ cudaError_t launch_octs_src(const Src& src, void* const out[5], long long ngroup
   if (e != cudaSuccess) return e;
   // groups per batch: full batches once every resident warp has one, fewer on a small list
   const long long warps = 152LL * oct_min_blocks<Pol, Src>() * kOctWarps;
-  const int batch = (int)std::min<long long>(oct_batch<Pol>(), std::max<long long>(1, ngroups / warps));
+  const int batch = (int)std::min<long long>(kOctBatch, std::max<long long>(1, ngroups / warps));
   const long long per_block = (long long)kOctWarps * batch;
   const long long blocks = std::min((ngroups + per_block - 1) / per_block, 152LL * 64);
   k_octs<Pol, Src><<<(unsigned)blocks, 32 * kOctWarps, smem, s>>>(src, (S*)out[0], (S*)out[1], (S*)out[2], (S*)out[3],
