@@ -396,7 +396,7 @@ int class_zc(const hydro_ctx* c, int k) { return c->cls_tile[k] >= 0 ? c->cls_zc
 // to 512^3 boxes at 2 to 128-plane chunks; the model stays within 5% of those and picks, against the
 // fixed 16x16 tiles of 32 planes: FP64 32^3 1367 -> 97 us, double-float 61^3 256 -> 70, FP32 96^3 76 -> 46,
 // mixed 64^3 124 -> 33; 512^3 within 1% of the best of the sweep.  (Double-float since its comparisons are
-// branch-free: 16x16 tiles with two blocks per SM take the 512^3 step in 20.3 ms, 32x16 tiles in 22.4.)
+// branch-free: 16x16 tiles with two blocks per SM take the 512^3 step in 20.8 ms, 32x16 tiles in 23.2.)
 struct ShapeCost {
   int tile;
   double plane, start;

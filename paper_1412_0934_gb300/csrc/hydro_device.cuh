@@ -470,9 +470,9 @@ __device__ __forceinline__ void hllc_core(const double qL[5], const double qR[5]
 // left unnormalised inside the formulas, S* from its distance to u_L (S* - u_L = (p_R - p_L + m_R (u_L -
 // u_R)) / (m_L - m_R), which does not cancel in fast flow), and the star energy as in double.
 // The tangential momentum fluxes are returned unnormalised (they are only summed); the mass flux and the
-// energy's terms are normalised, which costs 2% of the step and keeps the energy's error that of normalising
-// operators throughout (256^3 at Mach 5: 4.4e-15 of its norm, 4.6e-15 with its terms unnormalised).  The
-// kinetic sum's order is (u_n^2 + u_t1^2) + u_t2^2 for every normal.
+// energy's terms are normalised, which costs 2% of the step and, with those of the recovery (PolDF), keeps the
+// energy's error below that of normalising operators throughout (256^3 at Mach 5: 4.2e-15 of its norm against
+// 4.4e-15; 4.6e-15 with neither).  The kinetic sum's order is (u_n^2 + u_t1^2) + u_t2^2 for every normal.
 __device__ __forceinline__ void hllc_core(const df qL[5], const df qR[5], bool, const df& gamma, const df& inv_gm1,
                                           df F[5]) {
   const df2 r2 = pair_(qL[0], qR[0]), u2 = pair_(qL[1], qR[1]), p2 = pair_(qL[4], qR[4]);
